@@ -223,7 +223,7 @@ __global__ void k_adj_seed(StepArgs a, PState st, SeedIn in, AdjState nxt)
     if (g >= a.r.np) return;
     const int i = a.r.p0 + g;
     const size_t cap = a.cap;
-    const int gid = a.scenes[scene_of(a, i)].p_begin + st.id[i];
+    const int gid = a.scenes[scene_of(a, i)].p_begin + state_id(st, i);
     float* dst[4] = {nxt.x, nxt.v, nxt.C, nxt.F};
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_g2p_adj(AdjArgs q)
     __shared__ int s_item[2];
     const int tid = threadIdx.x;
     const size_t cap = a.cap;
-    const int n_act = a.sb.counters[CTR_N_ACT];
+    const int n_act = active_bricks(a.sb);
     int* work = &a.sb.counters[CTR_WORK_G2P];
     walker_init<kAdjThreads>(a, n_act, vw, bar, s_item, work);
     unsigned phase[2] = {0u, 0u};
@@ -254,9 +254,10 @@ __global__ void __launch_bounds__(kAdjThreads) k_g2p_adj(AdjArgs q)
         if (item >= n_act) break;
         for (int t = tid; t < 3 * kWinNodes; t += kAdjThreads) (&gw[0][0])[t] = 0.f;
         if (!walker_next(a, n_act, vw, bar, s_item, work, buf, phase, item)) return;
-        const int start = a.sb.act_start[item], count = a.sb.act_count[item];
-        const SceneDev sc = a.scenes[a.sb.act_scene[item]];
-        const int n = sc.n, nb = sc.nb, lb = a.sb.act_brick[item] - sc.brick_base;
+        const int e = active_entry(a.sb, item);
+        const int start = a.sb.act_start[e], count = a.sb.act_count[e];
+        const SceneDev sc = a.scenes[a.sb.act_scene[e]];
+        const int n = sc.n, nb = sc.nb, lb = a.sb.act_brick[e] - sc.brick_base;
         int ox, oy, oz;
         brick_coords(nb, sc.nb_log2, lb, ox, oy, oz);
         ox *= 4; oy *= 4; oz *= 4;
@@ -266,8 +267,9 @@ __global__ void __launch_bounds__(kAdjThreads) k_g2p_adj(AdjArgs q)
             const int s = start + k;
             const int p = a.sb.perm[s];
             int bc[3];
-            float f[3], w[9], dw[9];
-            particle_weights(a.in.x[p], a.in.x[cap + p], a.in.x[2 * cap + p], n, bc, f, w);
+            float f[3], w[9], dw[9], x[3];
+            load_x(a.in, p, x);
+            particle_weights(x[0], x[1], x[2], n, bc, f, w);
             bspline_d(f[0], dw);
             bspline_d(f[1], dw + 3);
             bspline_d(f[2], dw + 6);
@@ -294,10 +296,10 @@ __global__ void __launch_bounds__(kAdjThreads) k_g2p_adj(AdjArgs q)
                         }
                     }
             float Cn[9], F[9], aF[9], aC[9];
+            load_F(a.in, cap, p, F);
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
                 Cn[i] = c4 * B[i];
-                F[i] = a.in.F[i * cap + p];
                 aF[i] = q.nxt.F[i * cap + s];
                 aC[i] = q.nxt.C[i * cap + s];
             }
@@ -422,7 +424,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_p2g_adj(AdjArgs q)
     __shared__ int s_item[2];
     const int tid = threadIdx.x;
     const size_t cap = a.cap;
-    const int n_act = a.sb.counters[CTR_N_ACT];
+    const int n_act = active_bricks(a.sb);
     int* work = &a.sb.counters[CTR_WORK_P2G];
     walker_init<kAdjThreads>(a, n_act, vw, bar, s_item, work);
     unsigned phase[2] = {0u, 0u};
@@ -431,10 +433,11 @@ __global__ void __launch_bounds__(kAdjThreads) k_p2g_adj(AdjArgs q)
         const int item = s_item[buf];
         if (item >= n_act) break;
         if (!walker_next(a, n_act, vw, bar, s_item, work, buf, phase, item)) return;
-        const int start = a.sb.act_start[item], count = a.sb.act_count[item];
-        const int scene = a.sb.act_scene[item];
+        const int e = active_entry(a.sb, item);
+        const int start = a.sb.act_start[e], count = a.sb.act_count[e];
+        const int scene = a.sb.act_scene[e];
         const SceneDev sc = a.scenes[scene];
-        const int n = sc.n, nb = sc.nb, lb = a.sb.act_brick[item] - sc.brick_base;
+        const int n = sc.n, nb = sc.nb, lb = a.sb.act_brick[e] - sc.brick_base;
         int ox, oy, oz;
         brick_coords(nb, sc.nb_log2, lb, ox, oy, oz);
         ox *= 4; oy *= 4; oz *= 4;
@@ -445,20 +448,17 @@ __global__ void __launch_bounds__(kAdjThreads) k_p2g_adj(AdjArgs q)
             const int s = start + k;
             const int p = a.sb.perm[s];
             int bc[3];
-            float f[3], w[9], dw[9];
-            particle_weights(a.in.x[p], a.in.x[cap + p], a.in.x[2 * cap + p], n, bc, f, w);
+            float f[3], w[9], dw[9], x[3];
+            load_x(a.in, p, x);
+            particle_weights(x[0], x[1], x[2], n, bc, f, w);
             bspline_d(f[0], dw);
             bspline_d(f[1], dw + 3);
             bspline_d(f[2], dw + 6);
             const int l0 = min(max(bc[0] - ox, 0), 3), l1 = min(max(bc[1] - oy, 0), 3), l2 = min(max(bc[2] - oz, 0), 3);
             float F[9], C[9], v[3], tau[9];
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                F[i] = a.in.F[i * cap + p];
-                C[i] = a.in.C[i * cap + p];
-            }
-#pragma unroll
-            for (int d = 0; d < 3; ++d) v[d] = a.in.v[d * cap + p];
+            load_F(a.in, cap, p, F);
+            load_C(a.in, cap, p, C);
+            load_v(a.in, cap, p, v);
             const float mu = sc.pp_mat ? a.in.mu[p] : sc.mu, lam = sc.pp_mat ? a.in.lam[p] : sc.lam;
             float dummy[9], mub0, lamb0;
             stress_and_vjp(a.model, F, mu, lam, tau, nullptr, dummy, mub0, lamb0);
@@ -509,7 +509,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_p2g_adj(AdjArgs q)
                 q.cur.C[i * cap + p] = m * Ab[i];
                 q.cur.F[i * cap + p] += Fb[i];
             }
-            const int gid = sc.p_begin + a.in.id[p];
+            const int gid = sc.p_begin + state_id(a.in, p);
             q.gmu[gid] += mub;
             q.glam[gid] += lamb;
         }
@@ -535,7 +535,7 @@ __global__ void k_adj_out(StepArgs a, PState st0, AdjState adj0, const float* gm
     const int i = a.r.p0 + g;
     const size_t cap = a.cap;
     const SceneDev sc = a.scenes[scene_of(a, i)];
-    const int gid = sc.p_begin + st0.id[i];
+    const int gid = sc.p_begin + state_id(st0, i);
     const float* src[4] = {adj0.x, adj0.v, adj0.C, adj0.F};
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
@@ -650,7 +650,7 @@ int mpm_tape_record_substep(mpm_ctx* c, float dt)
     // the permutation G2P uses (P2G leaves it in cell order inside each pass)
     MPM_CKA(cudaMemcpyAsync(t->perms + (size_t)j * c->cap + a.r.p0, c->sb.perm + a.r.p0, sizeof(int) * a.r.np,
                             cudaMemcpyDeviceToDevice, c->stream));
-    MPM_CKA(launch_grid(a, c->stream));
+    MPM_CKA(launch_grid(a, c->stream, false));
     MPM_CKA(launch_g2p(a, c->stream));
     c->tau_valid = true;
     c->cur ^= 1;
@@ -713,7 +713,7 @@ static int backward_device(mpm_ctx* c, const SeedIn& seeds, const AdjOut& outs)
             a.cell_order = 0;  // the recorded permutation is already the one G2P used
             if ((st = sort_with_perm(c, a, seg_state(j - j0), t->perms + (size_t)j * cap))) return st;
             MPM_CKA(launch_p2g(a, c->stream));
-            MPM_CKA(launch_grid(a, c->stream));
+            MPM_CKA(launch_grid(a, c->stream, false));
             MPM_CKA(launch_g2p(a, c->stream));
         }
         // reverse the segment's substeps
@@ -723,7 +723,7 @@ static int backward_device(mpm_ctx* c, const SeedIn& seeds, const AdjOut& outs)
             a.cell_order = 0;
             if ((st = sort_with_perm(c, a, seg_state(j - j0), t->perms + (size_t)j * cap))) return st;
             MPM_CKA(launch_p2g(a, c->stream));
-            MPM_CKA(launch_grid(a, c->stream));
+            MPM_CKA(launch_grid(a, c->stream, true));
             AdjArgs q{a, adj[nxt], adj[nxt ^ 1], gmu, glam};
             const int ctas = c->num_sms * 2;
             // the walkers fetch work from the G2P and P2G counters: reset them

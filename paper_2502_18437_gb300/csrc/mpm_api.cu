@@ -47,19 +47,15 @@ int wait_stream(mpm_ctx* c)
     }
 }
 
-size_t state_bytes(int cap) { return (size_t)cap * (kStateFloats * sizeof(float) + sizeof(int)); }
+// (rounded up so that states stored one after another keep their planes aligned)
+size_t state_bytes(int cap) { return ((size_t)cap * kStateFloats * sizeof(float) + 255) & ~(size_t)255; }
 
 PState state_view(float* base, int cap)
 {
     PState s;
-    s.x = base;
-    s.v = base + 3 * (size_t)cap;
-    s.C = base + 6 * (size_t)cap;
-    s.F = base + 15 * (size_t)cap;
-    s.tau = base + 24 * (size_t)cap;
-    s.mu = base + 30 * (size_t)cap;
-    s.lam = base + 31 * (size_t)cap;
-    s.id = reinterpret_cast<int*>(base + 32 * (size_t)cap);
+    s.q = reinterpret_cast<float4*>(base);
+    s.mu = base + 4 * (size_t)kPlanes * cap;
+    s.lam = s.mu + cap;
     return s;
 }
 
@@ -183,12 +179,12 @@ StepArgs step_args(mpm_ctx* c, float dt, int s0, int s1, const PState& in, const
     const int ti = g2p_threads == 128 ? 0 : g2p_threads == 512 ? 2 : 1;
     int& og = c->occ_g2p[c->g2p_regs64 ? 1 : 0][ti];
     if (!og) og = std::max(1, occupancy_g2p(g2p_threads, c->g2p_regs64));
+    a.g2p_ctas = c->num_sms * cap_occ(c, og);
     int& op = c->occ_p2g[c->p2g_chunk / kP2GThreads - 2];
     if (!op) op = std::max(1, occupancy_p2g(c->p2g_chunk));
     if (!c->occ_grid) c->occ_grid = std::max(1, occupancy_grid());
     if (!c->occ_grid_plain) c->occ_grid_plain = std::max(1, occupancy_grid_plain());
     if (!c->occ_fused) c->occ_fused = std::max(1, occupancy_g2p2g());
-    a.persistent_ctas = c->num_sms * cap_occ(c, og);
     a.g2p_regs64 = c->g2p_regs64;
     a.p2g_ctas = c->num_sms * cap_occ(c, op);
     a.grid_ctas = c->num_sms * c->occ_grid;
@@ -257,7 +253,7 @@ int enqueue_substep(mpm_ctx* c, float dt, const PState& in, const PState& out, b
                     MPM_CK(cudaMemsetAsync(c->sb.counters + CTR_WORK_P2G, 0, sizeof(int) * 3, c->stream));
                 }
                 MPM_CK(launch_p2g(b, c->stream));
-                MPM_CK(launch_grid(b, c->stream));
+                MPM_CK(launch_grid(b, c->stream, false));
                 if (k + 1 < cycles) MPM_CK(launch_g2p_vc(b, c->stream));
                 else {
                     if (ev) MPM_CK(cudaEventRecord(ev[2], c->stream));
@@ -273,7 +269,7 @@ int enqueue_substep(mpm_ctx* c, float dt, const PState& in, const PState& out, b
             else MPM_CK(launch_p2g(a, c->stream));
         }
         if (ev) MPM_CK(cudaEventRecord(ev[2], c->stream));
-        MPM_CK(launch_grid(a, c->stream));
+        MPM_CK(launch_grid(a, c->stream, c->fused != 0));
         if (ev) MPM_CK(cudaEventRecord(ev[3], c->stream));
         if (c->fused) MPM_CK(launch_g2p2g(a, c->stream));
         else MPM_CK(launch_g2p(a, c->stream));
@@ -293,14 +289,7 @@ int invalidate_pending(mpm_ctx* c)
     return MPM_OK;
 }
 
-cudaError_t reset_histogram(mpm_ctx* c)
-{
-    const size_t nbk = (size_t)c->total_bricks;
-    cudaError_t e = cudaMemsetAsync(c->sb.cnt, 0, sizeof(int) * nbk, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->sb.nflag, 0, sizeof(int) * nbk, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->sb.tile_sum, 0, sizeof(int4) * (size_t)c->total_tiles, c->stream);
-    return e;
-}
+cudaError_t reset_histogram(mpm_ctx* c) { return launch_reset_histogram(c->sb, c->total_bricks, c->total_tiles, c->stream); }
 
 int ensure_keys(mpm_ctx* c)
 {
@@ -341,9 +330,9 @@ static void free_ctx(mpm_ctx* c)
     mpm_tape_free(c);
     clear_graphs(c);
     for (int i = 0; i < 2; ++i) cudaFree(c->state_mem[i]);
-    void* bufs[] = {c->sb.key, c->sb.rank, c->sb.perm, c->sb.scell, c->sb.cnt, c->sb.nflag, c->sb.off, c->sb.act_brick, c->sb.act_start,
+    void* bufs[] = {c->sb.key, c->sb.rank, c->sb.perm, c->sb.scell, c->sb.cnt, c->sb.off, c->sb.act_brick, c->sb.act_start,
                     c->sb.act_count, c->sb.act_scene, c->sb.nact_brick, c->sb.nact_scene, c->sb.counters,
-                    c->sb.tile_sum, c->G, c->V, c->brick_epoch,
+                    c->sb.tile_n, c->G, c->V, c->brick_epoch,
                     c->d_scenes, c->d_rigids, c->d_impulse, c->d_err, c->d_time, c->d_epoch, c->d_stage};
     for (void* p : bufs) cudaFree(p);
     if (c->h_pinned) cudaFreeHost(c->h_pinned);
@@ -386,10 +375,10 @@ extern "C" int mpm_create(const mpm_config* cfg, void* stream, mpm_ctx** out)
     if (bricks * 64 >= ((long long)1 << 31)) { delete c; return MPM_ERR_INVALID_ARGUMENT; }
     c->brick_base[c->n_scenes] = (int)bricks;
     c->total_bricks = (int)bricks;
-    // scan tiles: 2^shift bricks of one scene, at least 1024; wider tiles keep
-    // the number of tiles (whose totals every scan CTA adds up) near 2048 or less
+    // scan tiles: 2^shift bricks of one scene, at least 256; wider tiles keep
+    // the number of tiles (whose counts every scan CTA adds up) near 2048 or less
     {
-        int shift = 10;
+        int shift = kMinTileShift;
         auto tiles = [&](int sh) {
             long long t = 0;
             for (int s = 0; s < c->n_scenes; ++s)
@@ -442,7 +431,6 @@ extern "C" int mpm_create(const mpm_config* cfg, void* stream, mpm_ctx** out)
     alloc((void**)&c->sb.perm, sizeof(int) * c->cap);
     alloc((void**)&c->sb.scell, c->cap);
     alloc((void**)&c->sb.cnt, sizeof(int) * nbk);
-    alloc((void**)&c->sb.nflag, sizeof(int) * nbk);
     alloc((void**)&c->sb.off, sizeof(int) * nbk);
     alloc((void**)&c->sb.act_brick, sizeof(int) * nbk);
     alloc((void**)&c->sb.act_start, sizeof(int) * nbk);
@@ -451,7 +439,8 @@ extern "C" int mpm_create(const mpm_config* cfg, void* stream, mpm_ctx** out)
     alloc((void**)&c->sb.nact_brick, sizeof(int) * nbk);
     alloc((void**)&c->sb.nact_scene, sizeof(int) * nbk);
     alloc((void**)&c->sb.counters, sizeof(int) * CTR_COUNT);
-    alloc((void**)&c->sb.tile_sum, sizeof(int4) * c->total_tiles);
+    alloc((void**)&c->sb.tile_n, sizeof(int) * c->total_tiles);
+    c->sb.list_size = c->total_bricks;
     alloc((void**)&c->G, sizeof(float4) * nbk * 64);
     alloc((void**)&c->V, sizeof(float4) * nbk * 64);
     alloc((void**)&c->brick_epoch, sizeof(int) * nbk);
@@ -465,9 +454,8 @@ extern "C" int mpm_create(const mpm_config* cfg, void* stream, mpm_ctx** out)
     if (e == cudaSuccess) {
         for (int i = 0; i < 2; ++i) c->st[i] = state_view(c->state_mem[i], c->cap);
         cudaMemsetAsync(c->sb.cnt, 0, sizeof(int) * nbk, c->stream);
-        cudaMemsetAsync(c->sb.nflag, 0, sizeof(int) * nbk, c->stream);
         cudaMemsetAsync(c->sb.counters, 0, sizeof(int) * CTR_COUNT, c->stream);
-        cudaMemsetAsync(c->sb.tile_sum, 0, sizeof(int4) * c->total_tiles, c->stream);
+        cudaMemsetAsync(c->sb.tile_n, 0, sizeof(int) * c->total_tiles, c->stream);
         cudaMemsetAsync(c->G, 0, sizeof(float4) * nbk * 64, c->stream);
         cudaMemsetAsync(c->V, 0, sizeof(float4) * nbk * 64, c->stream);
         cudaMemsetAsync(c->brick_epoch, 0xff, sizeof(int) * nbk, c->stream);
@@ -609,18 +597,16 @@ extern "C" int mpm_add_particles(mpm_ctx* c, int scene, int64_t n, const float* 
     if (tail > 0) {
         // make room: copy into the spare buffer with the later scenes shifted by n
         PState nxt = c->st[c->cur ^ 1];
-        float* arr_src[kStateFloats + 1] = {};
-        float* arr_dst[kStateFloats + 1] = {};
-        for (int k = 0; k < kStateFloats; ++k) {
-            arr_src[k] = cur.x + (size_t)k * c->cap;
-            arr_dst[k] = nxt.x + (size_t)k * c->cap;
-        }
-        arr_src[kStateFloats] = reinterpret_cast<float*>(cur.id);
-        arr_dst[kStateFloats] = reinterpret_cast<float*>(nxt.id);
-        for (int k = 0; k <= kStateFloats; ++k) {
-            if (p_at > 0)
-                MPM_CK(cudaMemcpyAsync(arr_dst[k], arr_src[k], sizeof(float) * p_at, cudaMemcpyDeviceToDevice, c->stream));
-            MPM_CK(cudaMemcpyAsync(arr_dst[k] + p_at + n, arr_src[k] + p_at, sizeof(float) * tail,
+        struct Part { const char* src; char* dst; size_t item; };
+        std::vector<Part> parts;
+        for (int k = 0; k < kPlanes; ++k)
+            parts.push_back({reinterpret_cast<const char*>(cur.q + (size_t)k * c->cap),
+                             reinterpret_cast<char*>(nxt.q + (size_t)k * c->cap), sizeof(float4)});
+        parts.push_back({reinterpret_cast<const char*>(cur.mu), reinterpret_cast<char*>(nxt.mu), sizeof(float)});
+        parts.push_back({reinterpret_cast<const char*>(cur.lam), reinterpret_cast<char*>(nxt.lam), sizeof(float)});
+        for (const Part& q : parts) {
+            if (p_at > 0) MPM_CK(cudaMemcpyAsync(q.dst, q.src, q.item * p_at, cudaMemcpyDeviceToDevice, c->stream));
+            MPM_CK(cudaMemcpyAsync(q.dst + q.item * (p_at + n), q.src + q.item * p_at, q.item * tail,
                                    cudaMemcpyDeviceToDevice, c->stream));
         }
         c->cur ^= 1;
@@ -994,15 +980,14 @@ extern "C" int mpm_autotune(mpm_ctx* c, float dt, int trial_substeps, float* bes
     // snapshot everything a substep changes
     const size_t sbytes = state_bytes(c->cap);
     const size_t nbk = (size_t)c->total_bricks;
-    const size_t total = sbytes + 2 * sizeof(int) * c->cap + sizeof(int) * nbk * 3 + sizeof(int4) * c->total_tiles +
+    const size_t total = sbytes + 2 * sizeof(int) * c->cap + sizeof(int) * nbk * 2 + sizeof(int) * c->total_tiles +
                          (sizeof(double) + sizeof(int) + sizeof(unsigned) + sizeof(double) * kMaxRigids * 6) * c->n_scenes;
     char* snap = nullptr;
     MPM_CK(cudaMalloc(&snap, total));
     struct Item { void* live; size_t bytes; };
     const int cur0 = c->cur;
     Item items[] = {{c->state_mem[cur0], sbytes}, {c->sb.key, sizeof(int) * c->cap}, {c->sb.rank, sizeof(int) * c->cap},
-                    {c->sb.cnt, sizeof(int) * nbk}, {c->sb.nflag, sizeof(int) * nbk},
-                    {c->sb.tile_sum, sizeof(int4) * c->total_tiles},
+                    {c->sb.cnt, sizeof(int) * nbk}, {c->sb.tile_n, sizeof(int) * c->total_tiles},
                     {c->brick_epoch, sizeof(int) * nbk},
                     {c->d_time, sizeof(double) * c->n_scenes}, {c->d_epoch, sizeof(int) * c->n_scenes},
                     {c->d_err, sizeof(unsigned) * c->n_scenes},

@@ -2,10 +2,12 @@
 // Sec. III-B, Algorithm 1) for sm_103a.
 //
 // Layout in HBM
-//  - particles: structure of arrays, component-major: x[3][cap], v[3][cap],
-//    C[9][cap], F[9][cap], tau[6][cap], mu[cap], lam[cap], id[cap].  Two copies ping-pong:
-//    each substep reads one through the sort permutation and G2P writes the
-//    other in sorted order, so particles stay sorted by brick in storage.
+//  - particles: eight planes of float4 [8][cap], 128 bytes per particle (see
+//    PState), and mu[cap], lam[cap].  A particle's fields move in 16-byte words:
+//    a transfer kernel reads 4 to 6 of them instead of 13 to 21 single floats
+//    (and as many addresses).  Two copies ping-pong: each substep reads one
+//    through the sort permutation and G2P writes the other in sorted order, so
+//    particles stay sorted by brick in storage.
 //  - grid: each scene owns a dense block of (n/4)^3 bricks of 4^3 nodes;
 //    brick (bx,by,bz) of scene s is global brick brick_base[s] +
 //    (bx*nb + by)*nb + bz and node (lx,ly,lz) of a brick is at
@@ -95,26 +97,81 @@ struct SolidPose {
     float half[3];
 };
 
+// Particle state: plane k of particle p is q[k * cap + p].
+//   0: x0 x1 x2 id(int bits)   1: F0 F1 F2 F3   2: F4 F5 F6 F7   3: F8 v0 v1 v2
+//   4: C0 C1 C2 C3   5: C4 C5 C6 C7   6: C8 xx xy xz   7: yy yz zz -
+// (xx .. zz: the Kirchhoff stress of F, written by the unfused G2P).  G2P reads
+// planes 0-3 and writes all eight; P2G reads 0 and 3-7.
 struct PState {
-    float* x;
-    float* v;
-    float* C;
-    float* F;
-    float* tau;  // Kirchhoff stress of F (xx xy xz yy yz zz), written by the unfused G2P
+    float4* q;
     float* mu;
     float* lam;
-    int* id;
 };
+
+constexpr int kPlanes = 8;
+// float index of each field's first component in a particle's 32 floats
+constexpr int kAtX = 0, kAtId = 3, kAtF = 4, kAtV = 13, kAtC = 16;
+
+__device__ __forceinline__ float4 plane(const PState& s, size_t cap, int k, int p) { return s.q[k * cap + p]; }
+
+__device__ __forceinline__ float& state_at(const PState& s, size_t cap, int at, int p)
+{
+    return reinterpret_cast<float*>(s.q)[((size_t)(at >> 2) * cap + p) * 4 + (at & 3)];
+}
+
+__device__ __forceinline__ int& state_id(const PState& s, int p) { return reinterpret_cast<int*>(s.q)[(size_t)p * 4 + 3]; }
+
+__device__ __forceinline__ void load_x(const PState& s, int p, float x[3])
+{
+    const float4 a = s.q[p];
+    x[0] = a.x; x[1] = a.y; x[2] = a.z;
+}
+
+__device__ __forceinline__ void load_F(const PState& s, size_t cap, int p, float F[9])
+{
+    const float4 a = plane(s, cap, 1, p), b = plane(s, cap, 2, p);
+    F[0] = a.x; F[1] = a.y; F[2] = a.z; F[3] = a.w;
+    F[4] = b.x; F[5] = b.y; F[6] = b.z; F[7] = b.w;
+    F[8] = state_at(s, cap, kAtF + 8, p);
+}
+
+__device__ __forceinline__ void load_v(const PState& s, size_t cap, int p, float v[3])
+{
+    const float4 a = plane(s, cap, 3, p);
+    v[0] = a.y; v[1] = a.z; v[2] = a.w;
+}
+
+// C and, in t6, the stored stress
+__device__ __forceinline__ void load_C_tau(const PState& s, size_t cap, int p, float C[9], float t6[6])
+{
+    const float4 a = plane(s, cap, 4, p), b = plane(s, cap, 5, p), c = plane(s, cap, 6, p), d = plane(s, cap, 7, p);
+    C[0] = a.x; C[1] = a.y; C[2] = a.z; C[3] = a.w;
+    C[4] = b.x; C[5] = b.y; C[6] = b.z; C[7] = b.w;
+    C[8] = c.x;
+    t6[0] = c.y; t6[1] = c.z; t6[2] = c.w;
+    t6[3] = d.x; t6[4] = d.y; t6[5] = d.z;
+}
+
+__device__ __forceinline__ void load_C(const PState& s, size_t cap, int p, float C[9])
+{
+    const float4 a = plane(s, cap, 4, p), b = plane(s, cap, 5, p);
+    C[0] = a.x; C[1] = a.y; C[2] = a.z; C[3] = a.w;
+    C[4] = b.x; C[5] = b.y; C[6] = b.z; C[7] = b.w;
+    C[8] = state_at(s, cap, kAtC + 8, p);
+}
 
 // Counters shared by the kernels of one substep.
 enum {
-    CTR_N_ACT = 0,     // active particle bricks
-    CTR_N_NACT = 1,    // active node bricks
+    CTR_LAST_ACT = 0,  // active particle bricks and node bricks of the last finished substep
+    CTR_LAST_NACT = 1,
     CTR_DONE_G2P = 2,  // CTAs of the G2P launch that have finished (the last one advances the clocks)
     CTR_WORK_P2G = 3,  // dynamic work counters of the persistent kernels
     CTR_WORK_GRID = 4,
     CTR_WORK_G2P = 5,
-    CTR_COUNT = 8
+    CTR_N_BIG = 6,     // active particle bricks of at least kBigBrick particles
+    CTR_N_SMALL = 7,   // the other active particle bricks
+    CTR_N_NACT = 8,    // active node bricks
+    CTR_COUNT = 16
 };
 
 // ----------------------------------------------------------------- helpers

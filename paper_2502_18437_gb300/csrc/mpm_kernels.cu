@@ -1,7 +1,7 @@
 // Forward substep kernels of the MLS-MPM transfer loop (arXiv 2502.18437,
 // Algorithm 1) for GB300 (sm_103a):
 //   k_scan     brick histogram -> particle offsets, active particle-brick and
-//              node-brick lists (tile sums kept by the key producers: no
+//              node-brick lists (tile counts kept by the key producers: no
 //              inter-CTA waits, empty tiles skipped)
 //   k_scatter  counting-sort scatter: permutation sorted slot -> particle
 //   k_p2g      P2G (Eq. 1, Eq. 8): balanced per-cell work items summed in
@@ -9,9 +9,9 @@
 //              to HBM with vector atomics; leaves the permutation in cell order
 //   k_grid     grid update (Eq. 3), rigid contact (Sec. IV, Eq. 11, Eq. 12),
 //              domain walls (k_grid_plain where no scene has a rigid)
-//   k_grid_clear  reset of the P2G accumulator
-//   k_g2p      G2P (Eq. 4, Eq. 9, Eq. 10) with the 2x2x2-brick velocity halo
-//              staged by bulk-copy TMA, plasticity, next brick key + rank
+//   k_grid_clear  reset of the P2G accumulator where no G2P does it
+//   k_g2p      G2P (Eq. 4, Eq. 9, Eq. 10), one thread per slot with its stencil
+//              through L1, plasticity, next brick key + rank, reset of the accumulator
 #include <cstdint>
 #include <cstdio>
 
@@ -22,185 +22,173 @@ namespace mpm {
 // ----------------------------------------------------------------- scan
 //
 // A scan tile is 2^tile_shift consecutive bricks of one scene (tiles never
-// straddle scenes).  Each brick contributes (particles, is an active particle
-// brick, is an active node brick); a node brick is active when it or one of its
-// 7 lower neighbours (-1 in any subset of the axes) holds particles, since a
+// straddle scenes).  The key producers (G2P, k_prepare) count the particles of
+// every brick and every tile as they go, so each CTA of the scan (one per tile of
+// the range) knows the first slot of its bricks from the tile counts before it,
+// without waiting for another CTA.  The lists of active particle bricks and node
+// bricks need no order beyond the big bricks first (they start the persistent
+// transfer kernels, which then end on small ones), so each CTA appends its own to
+// them with one atomic per list.  A node brick is active when it or one of its 7
+// lower neighbours (-1 in any subset of the axes) holds particles, since a
 // particle's 3-node stencil reaches at most 2 nodes beyond its base cell, i.e.
-// into the next brick.  The key producers (G2P, k_prepare) count particles per
-// brick, flag those node bricks when the first particles enter a brick, and add
-// each tile's totals as they go.  So every CTA of the scan (one per tile of
-// the range) knows its exclusive prefix from the tile totals before it,
-// without waiting for another CTA; a tile with no active node brick has
-// nothing to write and returns at once.  The active particle-brick list holds
-// the bricks of at least kBigBrick particles first (in brick order), then the
-// others: the fourth tile total counts the former, and the grand total of the
-// range places the latter.
+// into the next brick: the scan looks the 8 counts up.  (Before, the first warp of
+// G2P to reach a brick marked 8 flags with one exchange after the other: 17 us of
+// G2P's 81 on a 1M block.)  A tile that no particle can reach returns at once.
 
-__device__ __forceinline__ int4 add4(int4 a, int4 b) { return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
-
-__device__ __forceinline__ int4 shfl_up4(int4 v, int d)
+// Sum of v over the CTA's threads before this one (excl) and over all (total).
+__device__ __forceinline__ void block_scan(int v, int* s_warp, int& excl, int& total)
 {
-    return make_int4(__shfl_up_sync(kFull, v.x, d), __shfl_up_sync(kFull, v.y, d), __shfl_up_sync(kFull, v.z, d),
-                     __shfl_up_sync(kFull, v.w, d));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int incl = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int t = __shfl_up_sync(kFull, incl, d);
+        if (lane >= d) incl += t;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    int before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < kScanThreads / 32; ++w) {
+        const int t = s_warp[w];
+        if (w < warp) before += t;
+        all += t;
+    }
+    __syncthreads();
+    excl = before + incl - v;
+    total = all;
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan(StepArgs a)
 {
-    __shared__ int4 s_warp[kScanThreads / 32];
-    __shared__ int s_wtot[kScanThreads / 32];
-    __shared__ int4 s_prefix;
-    __shared__ int s_big_total;
+    __shared__ int s_warp[kScanThreads / 32];
+    __shared__ int s_sum[3][kScanThreads / 32];
+    __shared__ int s_base[3];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const SortBufs& sb = a.sb;
     const int tile = a.r.t0 + blockIdx.x;
-    const bool last = blockIdx.x == a.r.nt - 1;
     if (blockIdx.x == 0 && tid == 0) {
         sb.counters[CTR_WORK_P2G] = 0;
         sb.counters[CTR_WORK_GRID] = 0;
         sb.counters[CTR_WORK_G2P] = 0;
     }
-    const int4 own = __ldcg(&sb.tile_sum[tile]);
-    if (own.z == 0 && !last) return;  // no active node brick (hence no particle) here
-
-    // exclusive prefix: the totals of the range's tiles before this one; and the
-    // range's count of big bricks (the start of the small bricks in the list)
-    int4 pre = make_int4(0, 0, 0, 0);
-    int wtot = 0;
-    for (int t = a.r.t0 + tid; t < a.r.t0 + a.r.nt; t += kScanThreads) {
-        const int4 ts = __ldcg(&sb.tile_sum[t]);
-        if (t < tile) pre = add4(pre, ts);
-        wtot += ts.w;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        pre.x += __shfl_xor_sync(kFull, pre.x, o);
-        pre.y += __shfl_xor_sync(kFull, pre.y, o);
-        pre.z += __shfl_xor_sync(kFull, pre.z, o);
-        pre.w += __shfl_xor_sync(kFull, pre.w, o);
-        wtot += __shfl_xor_sync(kFull, wtot, o);
-    }
-    if (lane == 0) {
-        s_warp[warp] = pre;
-        s_wtot[warp] = wtot;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        int4 p = make_int4(0, 0, 0, 0);
-        int wt = 0;
-#pragma unroll
-        for (int w = 0; w < kScanThreads / 32; ++w) {
-            p = add4(p, s_warp[w]);
-            wt += s_wtot[w];
-        }
-        s_prefix = p;
-        s_big_total = wt;
-        if (last) {
-            const int4 tot = add4(p, own);
-            if (tot.x == a.r.np) {
-                sb.counters[CTR_N_ACT] = tot.y;
-                sb.counters[CTR_N_NACT] = tot.z;
-            } else {
-                // histogram and particle count disagree: skip this substep's work
-                sb.counters[CTR_N_ACT] = 0;
-                sb.counters[CTR_N_NACT] = 0;
-                atomicOr(&a.err[a.r.s0], MPM_EBIT_INTERNAL);
-            }
-        }
-    }
-    __syncthreads();
-    if (own.z == 0) return;
-    int4 run = s_prefix;
-    const int big_total = s_big_total;
-
     // scene of the tile
-    int s;
-    {
-        int lo = a.r.s0, hi = a.r.s1 - 1;
-        while (lo < hi) {
-            int mid = (lo + hi + 1) >> 1;
-            if (a.scenes[mid].tile_base <= tile) lo = mid;
+    int s = a.r.s0;
+    if (a.r.s1 - a.r.s0 > 1) {
+        int hi = a.r.s1 - 1;
+        while (s < hi) {
+            const int mid = (s + hi + 1) >> 1;
+            if (a.scenes[mid].tile_base <= tile) s = mid;
             else hi = mid - 1;
         }
-        s = lo;
     }
     const SceneDev& sc = a.scenes[s];
-    const int tb = 1 << sb.tile_shift;
-    const int b0 = sc.brick_base + (tile - sc.tile_base) * tb;
-    const int b1 = min(b0 + tb, sc.brick_base + sc.nb * sc.nb * sc.nb);
-    for (int chunk = b0; chunk < b1; chunk += kScanChunk) {
-        const int first = chunk + tid * kScanItems;
-        int c[kScanItems];
-        unsigned pf = 0, nf = 0, bf = 0;
-        int4 local = make_int4(0, 0, 0, 0);
+    const int nb = sc.nb, bricks = nb * nb * nb;
+    const int l0 = (tile - sc.tile_base) << sb.tile_shift, l1 = min(l0 + (1 << sb.tile_shift), bricks);
+    // particles of the tiles before this one, of the whole range, and of the tiles
+    // whose particles can activate a node brick here
+    const int near0 = sc.tile_base + (max(l0 - nb * nb - nb - 1, 0) >> sb.tile_shift);
+    int pre = 0, all = 0, near = 0;
+    for (int t = a.r.t0 + tid; t < a.r.t0 + a.r.nt; t += kScanThreads) {
+        const int c = __ldcg(&sb.tile_n[t]);
+        all += c;
+        if (t < tile) pre += c;
+        if (t >= near0 && t <= tile) near |= c;
+    }
+    pre = __reduce_add_sync(kFull, pre);
+    all = __reduce_add_sync(kFull, all);
+    near = __reduce_or_sync(kFull, near);
+    if (lane == 0) {
+        s_sum[0][warp] = pre;
+        s_sum[1][warp] = all;
+        s_sum[2][warp] = near;
+    }
+    __syncthreads();
+    pre = all = near = 0;
 #pragma unroll
-        for (int k = 0; k < kScanItems; ++k) {
-            const int b = first + k;
-            c[k] = 0;
-            if (b < b1) {
-                c[k] = __ldcg(&sb.cnt[b]);
-                const int flag = __ldcg(&sb.nflag[b]);  // reset by k_grid_clear
-                if (c[k] > 0) pf |= 1u << k;
-                if (c[k] >= kBigBrick) bf |= 1u << k;
-                if (flag) nf |= 1u << k;  // a non-empty brick always flags itself
-                local.x += c[k];
+    for (int w = 0; w < kScanThreads / 32; ++w) {
+        pre += s_sum[0][w];
+        all += s_sum[1][w];
+        near |= s_sum[2][w];
+    }
+    if (all != a.r.np) {
+        // histogram and particle count disagree: empty lists skip this substep's work
+        if (blockIdx.x == 0 && tid == 0) atomicOr(&a.err[a.r.s0], MPM_EBIT_INTERNAL);
+        return;
+    }
+    if (near == 0) return;
+    const unsigned lt = (1u << lane) - 1u;
+    int start0 = a.r.p0 + pre;
+    for (int chunk = l0; chunk < l1; chunk += kScanThreads) {
+        const int lb = chunk + tid, b = sc.brick_base + lb;
+        int c = 0;
+        bool node = false;
+        if (lb < l1) {
+            const int* cnt = sb.cnt + b;
+            int bx, by, bz;
+            brick_coords(nb, sc.nb_log2, lb, bx, by, bz);
+            int n[8];
+#pragma unroll
+            for (int o = 0; o < 8; ++o) {
+                const int dx = o >> 2, dy = (o >> 1) & 1, dz = o & 1;
+                n[o] = bx >= dx && by >= dy && bz >= dz ? __ldcg(cnt - (dx * nb + dy) * nb - dz) : 0;
             }
-        }
-        local.y = __popc(pf);
-        local.z = __popc(nf);
-        local.w = __popc(bf);
-        // block exclusive scan of (particles, pbricks, nbricks)
-        int4 incl = local;
+            c = n[0];
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            int4 t = shfl_up4(incl, d);
-            if (lane >= d) incl = add4(incl, t);
+            for (int o = 0; o < 8; ++o) node = node || n[o] > 0;
         }
-        if (lane == 31) s_warp[warp] = incl;
+        int before, total;
+        block_scan(c, s_warp, before, total);
+        // places in the lists
+        const unsigned big = __ballot_sync(kFull, c >= kBigBrick), small = __ballot_sync(kFull, c > 0 && c < kBigBrick),
+                       nodes = __ballot_sync(kFull, node);
+        if (lane == 0) {
+            s_sum[0][warp] = __popc(big);
+            s_sum[1][warp] = __popc(small);
+            s_sum[2][warp] = __popc(nodes);
+        }
         __syncthreads();
-        if (warp == 0) {
-            int4 w = lane < kScanThreads / 32 ? s_warp[lane] : make_int4(0, 0, 0, 0);
+        if (tid < 3) {
+            int t = 0;
 #pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                int4 t = shfl_up4(w, d);
-                if (lane >= d) w = add4(w, t);
+            for (int w = 0; w < kScanThreads / 32; ++w) {
+                const int k = s_sum[tid][w];
+                s_sum[tid][w] = t;
+                t += k;
             }
-            if (lane < kScanThreads / 32) s_warp[lane] = w;  // inclusive over warps
+            s_base[tid] = t ? atomicAdd(&sb.counters[CTR_N_BIG + tid], t) : 0;
         }
         __syncthreads();
-        int4 excl = make_int4(incl.x - local.x, incl.y - local.y, incl.z - local.z, incl.w - local.w);
-        if (warp > 0) excl = add4(excl, s_warp[warp - 1]);
-        excl = add4(excl, run);
-        // list positions: big bricks from excl.w, the others after all big bricks
-        int po = a.r.p0 + excl.x, bi = excl.w, si = big_total + excl.y - excl.w, ni = excl.z;
-        if (excl.y + local.y > a.r.nbr || ni + local.z > a.r.nbr || bi + local.w > big_total ||
-            si + local.y - local.w > a.r.nbr) {  // tile sums out of step with the bricks
-            atomicOr(&a.err[a.r.s0], MPM_EBIT_INTERNAL);
-            pf = nf = 0u;
+        if (c > 0) {
+            const int e = c >= kBigBrick
+                              ? s_base[0] + s_sum[0][warp] + __popc(big & lt)
+                              : sb.list_size - 1 - (s_base[1] + s_sum[1][warp] + __popc(small & lt));
+            const int start = start0 + before;
+            sb.off[b] = start;
+            sb.act_brick[e] = b;
+            sb.act_start[e] = start;
+            sb.act_count[e] = c;
+            sb.act_scene[e] = s;
         }
-#pragma unroll
-        for (int k = 0; k < kScanItems; ++k) {
-            const int b = first + k;
-            if (pf & (1u << k)) {
-                const int pi = (bf & (1u << k)) ? bi++ : si++;
-                sb.off[b] = po;
-                sb.act_brick[pi] = b;
-                sb.act_start[pi] = po;
-                sb.act_count[pi] = c[k];
-                sb.act_scene[pi] = s;
-            }
-            if (nf & (1u << k)) {
-                sb.nact_brick[ni] = b;
-                sb.nact_scene[ni] = s;
-                ++ni;
-            }
-            po += c[k];
+        if (node) {
+            const int e = s_base[2] + s_sum[2][warp] + __popc(nodes & lt);
+            sb.nact_brick[e] = b;
+            sb.nact_scene[e] = s;
         }
-        run = add4(run, s_warp[kScanThreads / 32 - 1]);
-        __syncthreads();  // s_warp is rewritten by the next chunk
+        start0 += total;
+        __syncthreads();  // s_sum and s_base are rewritten by the next chunk
     }
 }
 
-// Counting-sort scatter; also clears the range's tile sums for the next
+__global__ void k_reset_histogram(SortBufs sb, int bricks, int tiles)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < bricks) sb.cnt[i] = 0;
+    if (i < tiles) sb.tile_n[i] = 0;
+    if (i >= CTR_N_BIG && i <= CTR_N_NACT) sb.counters[i] = 0;
+}
+
+// Counting-sort scatter; also clears the range's tile counts for the next
 // substep (the scan has read them).  write_perm = 0 only clears (the adjoint
 // reuses a recorded permutation).
 // Each thread takes kScatterPer particles, 256 apart, with their loads issued
@@ -235,7 +223,7 @@ __global__ void __launch_bounds__(256) k_scatter(StepArgs a, int write_perm)
                 atomicOr(&a.err[a.r.s0], MPM_EBIT_INTERNAL);
             }
         }
-        if (g < a.r.nt) a.sb.tile_sum[a.r.t0 + g] = make_int4(0, 0, 0, 0);
+        if (g < a.r.nt) a.sb.tile_n[a.r.t0 + g] = 0;
     }
 }
 
@@ -269,10 +257,12 @@ __global__ void __launch_bounds__(256) k_prepare(StepArgs a, PState st)
     const SceneDev sc = a.scenes[scene];
     if (valid) {
         unsigned ood = 0;
-        key = cell_key(sc, st.x[i], st.x[a.cap + i], st.x[2 * a.cap + i], ood);
+        float x[3];
+        load_x(st, i, x);
+        key = cell_key(sc, x[0], x[1], x[2], ood);
         if (ood) ebits |= MPM_EBIT_OUT_OF_DOMAIN;
     }
-    const int rank = aggregated_rank_mark(a.sb, sc, key >> 6, valid, !block_sums);
+    const int rank = brick_rank(a.sb, sc, key, valid, !block_sums);
     if (valid) {
         a.sb.key[i] = key;
         a.sb.rank[i] = rank;
@@ -283,7 +273,7 @@ __global__ void __launch_bounds__(256) k_prepare(StepArgs a, PState st)
     if (block_sums) {
         __syncthreads();
         for (int t = threadIdx.x; t < a.r.nt; t += blockDim.x)
-            if (s_tile[t]) atomicAdd(&a.sb.tile_sum[a.r.t0 + t].x, s_tile[t]);
+            if (s_tile[t]) atomicAdd(&a.sb.tile_n[a.r.t0 + t], s_tile[t]);
     }
 }
 
@@ -312,7 +302,7 @@ __global__ void __launch_bounds__(256) k_prepare(StepArgs a, PState st)
 // At the end of the pass the window is added to HBM with one vector reduction
 // per node.  Stage and windows reuse the record slots.
 
-__device__ __forceinline__ void prefetch_l2(const float* p)
+__device__ __forceinline__ void prefetch_l2(const float4* p)
 {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
@@ -353,7 +343,7 @@ __global__ void __launch_bounds__(kP2GThreads, 4) k_p2g(StepArgs a)
     __shared__ int s_item, s_nitems, s_len[3];
     const int tid = threadIdx.x;
     const int t = tid & 63, slice = tid >> 6;
-    const int n_act = a.sb.counters[CTR_N_ACT];
+    const int n_act = active_bricks(a.sb);
     const int cap = a.cap;
     for (;;) {
         if (tid == 0) s_item = atomicAdd(&a.sb.counters[CTR_WORK_P2G], 1);
@@ -361,8 +351,9 @@ __global__ void __launch_bounds__(kP2GThreads, 4) k_p2g(StepArgs a)
         __syncthreads();
         const int item = s_item;
         if (item >= n_act) break;
-        const int b = a.sb.act_brick[item], start = a.sb.act_start[item], count = a.sb.act_count[item];
-        const int scene = a.sb.act_scene[item];
+        const int e = active_entry(a.sb, item);
+        const int b = a.sb.act_brick[e], start = a.sb.act_start[e], count = a.sb.act_count[e];
+        const int scene = a.sb.act_scene[e];
         const SceneDev sc = a.scenes[scene];
         const int n = sc.n, nb = sc.nb, lb = b - sc.brick_base;
         int ox, oy, oz;
@@ -390,8 +381,9 @@ __global__ void __launch_bounds__(kP2GThreads, 4) k_p2g(StepArgs a)
                     } else {
                         // a recorded permutation (differentiation): the cell from x
                         int c[3];
-                        const unsigned ood = base_cell(a.in.x[p], n, c[0]) | base_cell(a.in.x[cap + p], n, c[1]) |
-                                             base_cell(a.in.x[2 * cap + p], n, c[2]);
+                        float x[3];
+                        load_x(a.in, p, x);
+                        const unsigned ood = base_cell(x[0], n, c[0]) | base_cell(x[1], n, c[1]) | base_cell(x[2], n, c[2]);
                         if (ood) ebits |= MPM_EBIT_OUT_OF_DOMAIN;
                         const int l0 = min(max(c[0] - ox, 0), 3), l1 = min(max(c[1] - oy, 0), 3),
                                   l2 = min(max(c[2] - oz, 0), 3);
@@ -406,20 +398,10 @@ __global__ void __launch_bounds__(kP2GThreads, 4) k_p2g(StepArgs a)
             for (int u = 0; u < PER; ++u) {
                 if (pc[u] < 0) continue;
                 const int p = pp[u];
+                const bool stress = MODE == kP2GStress && a.tau_valid;
 #pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    prefetch_l2(a.in.x + (size_t)q * cap + p);
-                    prefetch_l2(a.in.v + (size_t)q * cap + p);
-                }
-#pragma unroll
-                for (int q = 0; q < 9; ++q) prefetch_l2(a.in.C + (size_t)q * cap + p);
-                if (MODE == kP2GStress && a.tau_valid) {
-#pragma unroll
-                    for (int q = 0; q < 6; ++q) prefetch_l2(a.in.tau + (size_t)q * cap + p);
-                } else {
-#pragma unroll
-                    for (int q = 0; q < 9; ++q) prefetch_l2(a.in.F + (size_t)q * cap + p);
-                }
+                for (int k = 0; k < kPlanes; ++k)
+                    if (stress ? (k != 1 && k != 2) : k != 7) prefetch_l2(a.in.q + (size_t)k * cap + p);
             }
             __syncthreads();
             if (tid < 32)
@@ -455,28 +437,25 @@ __global__ void __launch_bounds__(kP2GThreads, 4) k_p2g(StepArgs a)
                 }
                 const int p = pp[u];
                 int bc[3];
-                float f[3], w[9];
-                ebits |= particle_weights(a.in.x[p], a.in.x[cap + p], a.in.x[2 * cap + p], n, bc, f, w);
+                float f[3], w[9], x[3];
+                load_x(a.in, p, x);
+                ebits |= particle_weights(x[0], x[1], x[2], n, bc, f, w);
                 float C[9], v[3], t6[6];
-#pragma unroll
-                for (int q = 0; q < 9; ++q) C[q] = a.in.C[(size_t)q * cap + p];
-#pragma unroll
-                for (int q = 0; q < 3; ++q) v[q] = a.in.v[(size_t)q * cap + p];
+                load_v(a.in, cap, p, v);
                 if (MODE == kP2GConstraint) {
                     float F[9];
-#pragma unroll
-                    for (int q = 0; q < 9; ++q) F[q] = a.in.F[(size_t)q * cap + p];
+                    load_C(a.in, cap, p, C);
+                    load_F(a.in, cap, p, F);
                     pb_constraint(F, a.dt, a.pb_beta, C);
 #pragma unroll
                     for (int q = 0; q < 6; ++q) t6[q] = 0.f;
                 } else if (a.tau_valid) {
-#pragma unroll
-                    for (int q = 0; q < 6; ++q) t6[q] = a.in.tau[(size_t)q * cap + p];
+                    load_C_tau(a.in, cap, p, C, t6);
                 } else {
                     // stress of the current F (after host writes, or seeding a fused run)
                     float F[9];
-#pragma unroll
-                    for (int q = 0; q < 9; ++q) F[q] = a.in.F[(size_t)q * cap + p];
+                    load_C(a.in, cap, p, C);
+                    load_F(a.in, cap, p, F);
                     const float mu = sc.pp_mat ? a.in.mu[p] : sc.mu, lam = sc.pp_mat ? a.in.lam[p] : sc.lam;
                     ebits |= constitutive(a.model, 0, 0.f, mu, lam, F, t6);
                 }
@@ -932,9 +911,10 @@ __global__ void __launch_bounds__(kGridThreads, 8) k_grid_plain(StepArgs a)
     }
 }
 
-// Reset of the P2G accumulator and of the node-brick flags of the active node
-// bricks once the grid update and the scan have read them.  Loading and clearing the lines that P2G's reductions just wrote
-// in one kernel measured far slower than two kernels: 13.4 against 11.5 us per
+// Reset of the P2G accumulator of the active node bricks once the grid update has
+// read it, where no G2P follows that does it (the fused G2P + P2G, the reverse
+// substeps).  Loading and clearing the lines that P2G's reductions just wrote in
+// one kernel measured far slower than two kernels: 13.4 against 11.5 us per
 // substep for the 1M block without rigids, 0.138 against 0.047 ms for the 256
 // batched scenes with their blades.
 __global__ void __launch_bounds__(kGridThreads, 8) k_grid_clear(StepArgs a)
@@ -946,7 +926,6 @@ __global__ void __launch_bounds__(kGridThreads, 8) k_grid_clear(StepArgs a)
         if (item < n_nact) {
             const int B = a.sb.nact_brick[item];
             a.G[B * 64 + nid] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (nid == 0) a.sb.nflag[B] = 0;  // the scan has read it (resetting it there was slower)
         }
     }
 }
@@ -1052,167 +1031,184 @@ __global__ void __launch_bounds__(kGridThreads, 4) k_grid(StepArgs a)
 
 // ------------------------------------------------------------------ G2P
 //
-// One CTA per active particle brick.  The 2x2x2 node bricks holding the 6^3
-// velocity window are staged in shared memory by bulk-copy TMA, double
-// buffered: the next brick's window is in flight while this brick computes.
+// One thread per sorted slot (Eq. 4, Eq. 9, Eq. 10, then the constitutive update,
+// the last step of the G2P loop in Algorithm 1).
 
-// G2P of one particle from the staged window (Eq. 4, Eq. 9, Eq. 10) followed by
-// the constitutive update (the last step of the G2P loop in Algorithm 1).
-// Writes x, v, C, F (and id, mu, lam) to slot s of the output state; returns
-// the new position, velocity, C and the Kirchhoff stress of the new F.
+// Result of one particle: the caller stores it (store_particle).
 struct G2POut {
-    float x[3], v[3], C[9], t6[6];
+    float x[3], v[3], C[9], F[9], t6[6];
+    int id;
 };
 
-__device__ __forceinline__ void cp_async4(float* dst, const float* src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// Staged mode (sX != nullptr): x and F of particle p were copied into
-// sX[d * stride] and sF[q * stride] by cp.async one particle ahead; this call
-// starts the copies of particle pnext (when >= 0) as soon as its own values
-// are out of the buffers: x after the gather, F after the F update.
 // Variants of the forward G2P (template flags).
 enum {
-    kG2PSolids = 1,    // push particles out of solid rigids (some scene has a rigid)
+    kG2PSolids = 1,    // push particles out of solid rigids (some scene has a sphere or a box)
     kG2PStdGrad = 2,   // standard MPM: L = sum v_I grad phi^T instead of the APIC C (Eq. 5)
     kG2PNoStress = 4   // PB-MPM: no constitutive update (no stress is stored)
 };
 
-// The new position is returned in o.x and stored by the caller, after the
-// particle push-out (finish_position).
-template <int FLAGS>
-__device__ __forceinline__ unsigned g2p_particle(const StepArgs& a, const SceneDev& sc, const float4* lin, int p, int s,
-                                                 int ox, int oy, int oz, G2POut& o, float* sX = nullptr,
-                                                 float* sF = nullptr, int stride = 0, int pnext = -1,
-                                                 int* sI = nullptr)
+// Velocity and affine matrix gathered at a position:
+//   v = sum W v_I,  B_rc = sum W v_I,r (o_c - f_c),  W = wx_i wy_j wz_k
+// (kG2PStdGrad: the basis gradient in cell units instead, B_rc = sum v_I,r dW/df_c),
+// contracted separably over k, then j, then i; x and y go in paired FMAs.
+// node(i, j, k) returns (v, m) of the stencil's nodes.
+template <int FLAGS, class Node>
+__device__ __forceinline__ void gather_velocity(const float f[3], const float w[9], Node node, float v[3], float B[9])
 {
-    const int cap = a.cap, n = sc.n;
-    const float fn = (float)n, dt = a.dt;
-    unsigned ebits = 0;
-    if (sX) cp_async_wait_all();
-    const float x0 = sX ? sX[0] : a.in.x[p], x1 = sX ? sX[stride] : a.in.x[cap + p],
-                x2 = sX ? sX[2 * stride] : a.in.x[2 * cap + p];
-    const int id_staged = sI ? sI[0] : 0;  // read before the next particle's copy lands
-    int bc[3];
-    float f[3], w[9];
-    particle_weights(x0, x1, x2, n, bc, f, w);
-    const int l0 = min(max(bc[0] - ox, 0), 3), l1 = min(max(bc[1] - oy, 0), 3), l2 = min(max(bc[2] - oz, 0), 3);
-    // separable contraction over k, then j, then i of
-    //   v = sum W v_I,  B_rc = sum W v_I,r (o_c - f_c),  W = wx_i wy_j wz_k
-    const float* wx = w;
     const float* wy = w + 3;
     const float* wz = w + 6;
-    float wxd[3], wyd[3], wzd[3];
+    float wyd[3], wzd[3];
     if (FLAGS & kG2PStdGrad) {
-        // the basis gradient in cell units (times n below): L_rc = n sum v_r dW/df_c
-        bspline_d(f[0], wxd);
         bspline_d(f[1], wyd);
         bspline_d(f[2], wzd);
     } else {
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            wxd[q] = wx[q] * ((float)q - f[0]);
             wyd[q] = wy[q] * ((float)q - f[1]);
             wzd[q] = wz[q] * ((float)q - f[2]);
         }
     }
-    const float4* base = lin + (l0 * 36 + l1 * 6 + l2);
-    float A[3][3], Ay[3][3], Bz[3][3];  // [i][component]
+    const auto two = [](float s) { return make_float2(s, s); };
+    float2 vp = two(0.f), B0 = two(0.f), B1 = two(0.f), B2 = two(0.f);  // x, y rows
+    float vz = 0.f, Bz0 = 0.f, Bz1 = 0.f, Bz2 = 0.f;                    // z row
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) A[i][c] = Ay[i][c] = Bz[i][c] = 0.f;
+        // weight of plane i (as bspline) and its derivative or moment
+        const float fi = (float)i;
+        const float e = f[0] - (1.5f - 0.5f * fi);
+        const float wx = i == 1 ? 0.75f - e * e : 0.5f * e * e;
+        const float wxd = (FLAGS & kG2PStdGrad) ? (i == 1 ? -2.f * e : e) : wx * (fi - f[0]);
+        float2 A = two(0.f), Ay = two(0.f), Az = two(0.f);
+        float zA = 0.f, zAy = 0.f, zAz = 0.f;
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            const float4 g0 = base[i * 36 + j * 6], g1 = base[i * 36 + j * 6 + 1], g2 = base[i * 36 + j * 6 + 2];
-            const float ax = wz[0] * g0.x + wz[1] * g1.x + wz[2] * g2.x;
-            const float ay = wz[0] * g0.y + wz[1] * g1.y + wz[2] * g2.y;
-            const float az = wz[0] * g0.z + wz[1] * g1.z + wz[2] * g2.z;
-            const float bx = wzd[0] * g0.x + wzd[1] * g1.x + wzd[2] * g2.x;
-            const float by = wzd[0] * g0.y + wzd[1] * g1.y + wzd[2] * g2.y;
-            const float bz = wzd[0] * g0.z + wzd[1] * g1.z + wzd[2] * g2.z;
-            A[i][0] += wy[j] * ax; A[i][1] += wy[j] * ay; A[i][2] += wy[j] * az;
-            Ay[i][0] += wyd[j] * ax; Ay[i][1] += wyd[j] * ay; Ay[i][2] += wyd[j] * az;
-            Bz[i][0] += wy[j] * bx; Bz[i][1] += wy[j] * by; Bz[i][2] += wy[j] * bz;
+            float2 p = two(0.f), d = two(0.f);
+            float zp = 0.f, zd = 0.f;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float4 g = node(i, j, k);
+                const float2 xy = make_float2(g.x, g.y);
+                p = __ffma2_rn(two(wz[k]), xy, p);
+                d = __ffma2_rn(two(wzd[k]), xy, d);
+                zp = __fmaf_rn(wz[k], g.z, zp);
+                zd = __fmaf_rn(wzd[k], g.z, zd);
+            }
+            A = __ffma2_rn(two(wy[j]), p, A);
+            Ay = __ffma2_rn(two(wyd[j]), p, Ay);
+            Az = __ffma2_rn(two(wy[j]), d, Az);
+            zA = __fmaf_rn(wy[j], zp, zA);
+            zAy = __fmaf_rn(wyd[j], zp, zAy);
+            zAz = __fmaf_rn(wy[j], zd, zAz);
         }
+        vp = __ffma2_rn(two(wx), A, vp);
+        B0 = __ffma2_rn(two(wxd), A, B0);
+        B1 = __ffma2_rn(two(wx), Ay, B1);
+        B2 = __ffma2_rn(two(wx), Az, B2);
+        vz = __fmaf_rn(wx, zA, vz);
+        Bz0 = __fmaf_rn(wxd, zA, Bz0);
+        Bz1 = __fmaf_rn(wx, zAy, Bz1);
+        Bz2 = __fmaf_rn(wx, zAz, Bz2);
     }
-    float vv[3], B[9];
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        vv[r] = wx[0] * A[0][r] + wx[1] * A[1][r] + wx[2] * A[2][r];
-        B[3 * r] = wxd[0] * A[0][r] + wxd[1] * A[1][r] + wxd[2] * A[2][r];
-        B[3 * r + 1] = wx[0] * Ay[0][r] + wx[1] * Ay[1][r] + wx[2] * Ay[2][r];
-        B[3 * r + 2] = wx[0] * Bz[0][r] + wx[1] * Bz[1][r] + wx[2] * Bz[2][r];
-    }
-    const float v0 = vv[0], v1 = vv[1], v2 = vv[2];
-    if (sX && pnext >= 0) {
-#pragma unroll
-        for (int d = 0; d < 3; ++d) cp_async4(sX + d * stride, a.in.x + (size_t)d * cap + pnext);
-        if (sI) cp_async4(reinterpret_cast<float*>(sI), reinterpret_cast<const float*>(a.in.id + pnext));
-    }
+    v[0] = vp.x; v[1] = vp.y; v[2] = vz;
+    B[0] = B0.x; B[1] = B1.x; B[2] = B2.x;
+    B[3] = B0.y; B[4] = B1.y; B[5] = B2.y;
+    B[6] = Bz0; B[7] = Bz1; B[8] = Bz2;
+}
+
+// G2P of a particle with position (and id) q0 from its stencil's velocities; the
+// new position before the push-out.  stencil(bc) returns the node functor of base
+// cell bc, old_F(F) reads the deformation gradient.
+template <int FLAGS, class Stencil, class OldF>
+__device__ __forceinline__ unsigned g2p_particle(const StepArgs& a, const SceneDev& sc, const float4 q0, float mu, float lam,
+                                                 Stencil stencil, OldF old_F, G2POut& o)
+{
+    const int n = sc.n;
+    const float fn = (float)n, dt = a.dt;
+    unsigned ebits = 0;
+    int bc[3];
+    float f[3], w[9], B[9];
+    particle_weights(q0.x, q0.y, q0.z, n, bc, f, w);
+    o.id = __float_as_int(q0.w);
+    gather_velocity<FLAGS>(f, w, stencil(bc), o.v, B);
     // C = D^-1 sum N v (x_I - x_p)^T = 4/dx^2 * dx * B  (Eq. 9), or for the
     // standard MPM L = n B with the derivative weights (Eq. 5); x += dt v (Eq. 4)
     const float c4 = (FLAGS & kG2PStdGrad) ? fn : 4.0f * fn;
 #pragma unroll
     for (int i = 0; i < 9; ++i) o.C[i] = B[i] * c4;
-    o.v[0] = v0; o.v[1] = v1; o.v[2] = v2;
-    o.x[0] = x0 + dt * v0;
-    o.x[1] = x1 + dt * v1;
-    o.x[2] = x2 + dt * v2;
-#pragma unroll
-    for (int d = 0; d < 3; ++d) a.out.v[(size_t)d * cap + s] = o.v[d];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) a.out.C[(size_t)i * cap + s] = o.C[i];
-    a.out.id[s] = sI ? id_staged : a.in.id[p];
-    float mu, lam;
-    if (sc.pp_mat) {
-        mu = a.in.mu[p];
-        lam = a.in.lam[p];
-        a.out.mu[s] = mu;
-        a.out.lam[s] = lam;
-    } else {
-        mu = sc.mu;
-        lam = sc.lam;
-    }
+    o.x[0] = q0.x + dt * o.v[0];
+    o.x[1] = q0.y + dt * o.v[1];
+    o.x[2] = q0.z + dt * o.v[2];
     // F <- (I + dt C) F  (Eq. 10)
-    float Fn[9];
+    float F[9];
+    old_F(F);
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const float F0 = sF ? sF[c * stride] : a.in.F[(size_t)c * cap + p];
-        const float F1 = sF ? sF[(3 + c) * stride] : a.in.F[(size_t)(3 + c) * cap + p];
-        const float F2 = sF ? sF[(6 + c) * stride] : a.in.F[(size_t)(6 + c) * cap + p];
+        const float F0 = F[c], F1 = F[3 + c], F2 = F[6 + c];
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
             const float Fr = r == 0 ? F0 : (r == 1 ? F1 : F2);
-            Fn[3 * r + c] = Fr + dt * (o.C[3 * r] * F0 + o.C[3 * r + 1] * F1 + o.C[3 * r + 2] * F2);
+            o.F[3 * r + c] = Fr + dt * (o.C[3 * r] * F0 + o.C[3 * r + 1] * F1 + o.C[3 * r + 2] * F2);
         }
     }
-    if (sF && pnext >= 0) {
+    if (!(FLAGS & kG2PNoStress)) {
+        ebits |= constitutive(a.model, a.plasticity, a.yield_stress, mu, lam, o.F, o.t6);
+    } else {
 #pragma unroll
-        for (int q = 0; q < 9; ++q) cp_async4(sF + q * stride, a.in.F + (size_t)q * cap + pnext);
+        for (int i = 0; i < 6; ++i) o.t6[i] = 0.f;
     }
-    if (!(FLAGS & kG2PNoStress)) ebits |= constitutive(a.model, a.plasticity, a.yield_stress, mu, lam, Fn, o.t6);
+    float chk = q0.x + q0.y + q0.z + o.v[0] + o.v[1] + o.v[2];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) a.out.F[(size_t)i * cap + s] = Fn[i];
-    float chk = x0 + x1 + x2 + v0 + v1 + v2;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) chk += Fn[i];
+    for (int i = 0; i < 9; ++i) chk += o.F[i];
     if (!isfinite(chk)) ebits |= MPM_EBIT_NONFINITE;
     return ebits;
 }
 
-// Push-out against the scene's solid rigids at the end of the substep
-// (n_solid = 0: none), then the position store at slot s.
-__device__ __forceinline__ void finish_position(const StepArgs& a, const SolidPose* poses, int n_solid, int s,
-                                                float x[3])
+// All eight planes of slot s, and the material.
+__device__ __forceinline__ void store_particle(const StepArgs& a, int pp_mat, float mu, float lam, int s, const G2POut& o)
 {
-    if (n_solid) push_out(poses, n_solid, x);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) a.out.x[(size_t)d * a.cap + s] = x[d];
+    const size_t cap = a.cap;
+    float4* q = a.out.q + s;
+    q[0] = make_float4(o.x[0], o.x[1], o.x[2], __int_as_float(o.id));
+    q[cap] = make_float4(o.F[0], o.F[1], o.F[2], o.F[3]);
+    q[2 * cap] = make_float4(o.F[4], o.F[5], o.F[6], o.F[7]);
+    q[3 * cap] = make_float4(o.F[8], o.v[0], o.v[1], o.v[2]);
+    q[4 * cap] = make_float4(o.C[0], o.C[1], o.C[2], o.C[3]);
+    q[5 * cap] = make_float4(o.C[4], o.C[5], o.C[6], o.C[7]);
+    q[6 * cap] = make_float4(o.C[8], o.t6[0], o.t6[1], o.t6[2]);
+    q[7 * cap] = make_float4(o.t6[3], o.t6[4], o.t6[5], 0.f);
+    if (pp_mat) {
+        a.out.mu[s] = mu;
+        a.out.lam[s] = lam;
+    }
+}
+
+__device__ __forceinline__ void material_of(const StepArgs& a, const SceneDev& sc, int p, float& mu, float& lam)
+{
+    mu = sc.mu;
+    lam = sc.lam;
+    if (sc.pp_mat) {
+        mu = a.in.mu[p];
+        lam = a.in.lam[p];
+    }
+}
+
+// Scene of slot s (scenes own consecutive slots): two warp-wide probes of the
+// scenes' first slots for the warp's first slot, then the few lanes of later scenes
+// step on.  Every lane of the warp calls it.
+__device__ __forceinline__ int scene_of_slot(const StepArgs& a, int s)
+{
+    if (a.r.s1 - a.r.s0 == 1) return a.r.s0;
+    const int lane = threadIdx.x & 31, s_first = __shfl_sync(kFull, s, 0);
+    int lo = a.r.s0, len = a.r.s1 - a.r.s0;
+    while (len > 1) {  // p_begin never decreases: the last scene that starts at or before s_first
+        const int step = (len + 31) >> 5, at = lane * step;
+        const bool le = at < len && a.scenes[lo + at].p_begin <= s_first;
+        const int k = 31 - __clz(__ballot_sync(kFull, le) | 1u);
+        lo += k * step;
+        len = min(step, len - k * step);
+    }
+    while (lo + 1 < a.r.s1 && a.scenes[lo + 1].p_begin <= s) ++lo;
+    return lo;
 }
 
 // Copy the 6^3 window out of the 2x2x2 staged bricks into a linear array, so
@@ -1226,89 +1222,138 @@ __device__ __forceinline__ void linearize_window(const float4* vw, float4* lin)
     }
 }
 
+// Nodes of a base cell's stencil in the brick layout, read through L1.
+struct GridStencil {
+    const float4* V;
+    int x0, sx, o[6];  // first x, stride of bricks along x, node offsets along y and z (with the scene's first node)
+    __device__ __forceinline__ GridStencil(const float4* V_, const SceneDev& sc, const int bc[3]) : V(V_), x0(bc[0])
+    {
+        const int sy = sc.nb * 64;
+        sx = sc.nb * sy;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int y = bc[1] + i, z = bc[2] + i;
+            o[i] = (y >> 2) * sy + (y & 3) * 4 + sc.brick_base * 64;
+            o[3 + i] = (z >> 2) * 64 + (z & 3);
+        }
+    }
+    __device__ __forceinline__ float4 operator()(int i, int j, int k) const
+    {
+        const int x = x0 + i, ox = (x >> 2) * sx + (x & 3) * 16;
+        return __ldg(V + (ox + o[j] + o[3 + k]));
+    }
+};
+
+__device__ __forceinline__ void cp_async16(float4* dst, const float4* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Persistent CTAs, their warps taking chunks of 32 slots in turn (the chunks in
+// flight then cover one window of the arrays, and neighbouring warps the same nodes).
+// What bounds it is the chain permutation -> planes -> nodes -> rank of each
+// particle: planes 0-3 of a warp's next chunk are copied to shared memory while it
+// computes, and its slots of the permutation are read two chunks ahead.  Read through
+// L1, the stencils need no staging, no barriers and no brick: one CTA per brick with
+// its window copied to shared memory (46.1 M warp instructions at 62 % issue, the SMs
+// idle for a sixth of the launch behind its last bricks) took 70.8 us on a 1M block
+// and 18.8 us on a 64k one; this kernel 59.8 us and 9.5 us, the accumulator's reset
+// (1.8 us in a kernel of its own) included.  Budgets of 64 / 80 / 96 registers: 64.4 /
+// 63.9 / 66.6 us on the 1M block.
 // MINB = CTAs per SM the registers must allow: the larger budget (7 at 128
 // threads, 72 registers; 3 at 256, 80; 1 at 512) or 1024/BLOCK (64 registers,
-// more warps in flight).  SOLIDS: some scene of the launch has a sphere or a
-// box, so particles may need the push-out (a separate variant: its extra live
-// registers would make the plain build spill).
+// more warps in flight).  FLAGS & kG2PSolids: some scene of the launch has a
+// sphere or a box, so particles may need the push-out.
 template <int BLOCK, int MINB, int FLAGS>
 __global__ void __launch_bounds__(BLOCK, MINB) k_g2p(StepArgs a)
 {
     constexpr bool SOLIDS = (FLAGS & kG2PSolids) != 0;
-    // x, F and (with 72 or more registers; the 64-register builds would spill) the
-    // id of each thread's next particle, copied by cp.async one particle ahead
-    constexpr bool STAGE_ID = 65536 / (BLOCK * MINB) >= 72;
-    __shared__ float sX[3 * BLOCK], sF[9 * BLOCK];
-    __shared__ int sI[STAGE_ID ? BLOCK : 1];
-    __shared__ __align__(128) float4 vw[2][8 * 64];
-    __shared__ __align__(16) float4 lin[kWinNodes];
-    __shared__ __align__(8) unsigned long long bar[2];
-    __shared__ int s_item[2];
-    __shared__ SolidPose s_pose[kMaxRigids];  // the scene's rigids at the end of the substep
-    __shared__ int s_pose_scene;
-    const int tid = threadIdx.x;
-    const int n_act = a.sb.counters[CTR_N_ACT];
-    int* work = &a.sb.counters[CTR_WORK_G2P];
-    if (tid == 0) s_pose_scene = -1;
-    walker_init<BLOCK>(a, n_act, vw, bar, s_item, work);
-    unsigned phase[2] = {0u, 0u};
-    int buf = 0;
-    for (;;) {
-        const int item = s_item[buf];
-        if (item >= n_act) break;
-        if (!walker_next(a, n_act, vw, bar, s_item, work, buf, phase, item)) break;
-        const int start = a.sb.act_start[item], count = a.sb.act_count[item], scene = a.sb.act_scene[item];
-        const SceneDev sc = a.scenes[scene];
-        // s_pose_scene changes only after the barrier below, which every thread
-        // passes after this test
-        const int n_solid = SOLIDS ? sc.n_rigid : 0;
-        if (n_solid && scene != s_pose_scene) stage_solids(a, scene, s_pose);
-        const int nb = sc.nb, lb = a.sb.act_brick[item] - sc.brick_base;
-        int ox, oy, oz;
-        brick_coords(nb, sc.nb_log2, lb, ox, oy, oz);
-        ox *= 4; oy *= 4; oz *= 4;
-        // the brick's first particle of each thread: its copies start here (the
-        // thread's last call of the previous brick has read both buffers)
-        int pcur = tid < count ? a.sb.perm[start + tid] : -1;
-        if (pcur >= 0) {
+    constexpr int NW = BLOCK / 32;
+    __shared__ float4 s_q[4][BLOCK];  // planes 0-3 of each thread's next particle
+    __shared__ SolidPose s_pose[SOLIDS ? NW : 1][SOLIDS ? kMaxRigids : 1];  // a scene's rigids at the end of the substep
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // the accumulator of the active node bricks: the grid update has read it
+    const int n_clear = a.sb.counters[CTR_N_NACT] * 64;
+    for (int t = blockIdx.x * BLOCK + tid; t < n_clear; t += gridDim.x * BLOCK)
+        a.G[a.sb.nact_brick[t >> 6] * 64 + (t & 63)] = make_float4(0.f, 0.f, 0.f, 0.f);
+    // (no particle brick: the sort found its bookkeeping inconsistent)
+    const int c1 = active_bricks(a.sb) ? (a.r.np + 31) >> 5 : 0;
+    const int step = gridDim.x * NW;
+    int c = blockIdx.x * NW + warp;
+    const int p_end = a.r.p0 + a.r.np;
+    const size_t cap = a.cap;
+    const auto slot_source = [&](int ch) {
+        const int s = a.r.p0 + ch * 32 + lane;
+        return ch < c1 && s < p_end ? a.sb.perm[s] : -1;
+    };
+    const auto copy_planes = [&](int p) {
+        if (p >= 0) {
 #pragma unroll
-            for (int d = 0; d < 3; ++d) cp_async4(&sX[d * BLOCK + tid], a.in.x + (size_t)d * a.cap + pcur);
-#pragma unroll
-            for (int q = 0; q < 9; ++q) cp_async4(&sF[q * BLOCK + tid], a.in.F + (size_t)q * a.cap + pcur);
-            if (STAGE_ID) cp_async4(reinterpret_cast<float*>(&sI[tid]), reinterpret_cast<const float*>(a.in.id + pcur));
+            for (int k = 0; k < 4; ++k) cp_async16(&s_q[k][tid], a.in.q + k * cap + p);
         }
-        linearize_window<BLOCK>(vw[buf], lin);
-        __syncthreads();
-        if (tid == 0 && n_solid) s_pose_scene = scene;
+        cp_async_commit();
+    };
+    int p = slot_source(c), p_next = slot_source(c + step);
+    copy_planes(p);
+    int posed = -1;
+    for (; c < c1; c += step) {
+        const int p_after = slot_source(c + 2 * step);
+        const int s = min(a.r.p0 + c * 32 + lane, p_end - 1);
+        const bool valid = p >= 0;
+        const int scene = scene_of_slot(a, s);
+        const SceneDev& sc = a.scenes[scene];
+        G2POut o;
         unsigned ebits = 0;
-        for (int k0 = 0; k0 < count; k0 += BLOCK) {
-            const int k = k0 + tid;
-            const bool valid = k < count;
-            int key = 0;
-            if (valid) {
-                G2POut o;
-                const int pnext = k + BLOCK < count ? a.sb.perm[start + k + BLOCK] : -1;
-                ebits |= g2p_particle<FLAGS>(a, sc, lin, pcur, start + k, ox, oy, oz, o, &sX[tid], &sF[tid], BLOCK,
-                                             pnext, STAGE_ID ? &sI[tid] : nullptr);
-                pcur = pnext;
-                if (!(FLAGS & kG2PNoStress))
-#pragma unroll
-                    for (int q = 0; q < 6; ++q) a.out.tau[(size_t)q * a.cap + start + k] = o.t6[q];
-                finish_position(a, SOLIDS ? s_pose : nullptr, n_solid, start + k, o.x);
-                unsigned ood = 0;
-                key = cell_key(sc, o.x[0], o.x[1], o.x[2], ood);
-                if (ood && !(ebits & MPM_EBIT_NONFINITE)) ebits |= MPM_EBIT_OUT_OF_DOMAIN;
-            }
-            const int rank = aggregated_rank_mark(a.sb, sc, key >> 6, valid);
-            if (valid) {
-                a.sb.key[start + k] = key;
-                a.sb.rank[start + k] = rank;
+        float mu = 0.f, lam = 0.f;
+        if (valid) material_of(a, sc, p, mu, lam);
+        cp_async_wait<0>();
+        int key = 0;
+        if (valid)
+            ebits = g2p_particle<FLAGS>(
+                a, sc, s_q[0][tid], mu, lam, [&](const int* bc) { return GridStencil(a.V, sc, bc); },
+                [&](float* F) {
+                    const float4 u = s_q[1][tid], v = s_q[2][tid];
+                    F[0] = u.x; F[1] = u.y; F[2] = u.z; F[3] = u.w;
+                    F[4] = v.x; F[5] = v.y; F[6] = v.z; F[7] = v.w;
+                    F[8] = s_q[3][tid].x;
+                    copy_planes(p_next);
+                },
+                o);
+        else copy_planes(p_next);
+        __syncwarp();
+        if (SOLIDS) {
+            // push-out (Sec. IV-A), scene by scene of the chunk
+            const int sc1 = __shfl_sync(kFull, scene, 31);
+            for (int q = __shfl_sync(kFull, scene, 0); q <= sc1; ++q) {
+                const int nr = a.scenes[q].n_rigid;
+                if (nr == 0) continue;
+                if (q != posed) stage_solids(a, q, s_pose[warp], lane);
+                posed = q;
+                __syncwarp();
+                if (valid && scene == q) push_out(s_pose[warp], nr, o.x);
+                __syncwarp();
             }
         }
-        if (ebits) atomicOr(&a.err[scene], ebits);
-        __syncthreads();
-        buf ^= 1;
+        if (valid) {
+            store_particle(a, sc.pp_mat, mu, lam, s, o);
+            unsigned ood = 0;
+            key = cell_key(sc, o.x[0], o.x[1], o.x[2], ood);
+            a.sb.key[s] = key;
+            if (ood && !(ebits & MPM_EBIT_NONFINITE)) ebits |= MPM_EBIT_OUT_OF_DOMAIN;
+            if (ebits) atomicOr(&a.err[scene], ebits);
+        }
+        const int rank = brick_rank(a.sb, sc, key, valid);
+        if (valid) a.sb.rank[s] = rank;
+        p = p_next;
+        p_next = p_after;
     }
+    cp_async_wait<0>();
+    // every read of the clocks of this CTA lies before the barrier
     walker_exit(a);
 }
 
@@ -1340,7 +1385,7 @@ __global__ void __launch_bounds__(kFusedThreads, 4) k_g2p2g(StepArgs a)
     const int tid = threadIdx.x;
     const int cell = tid & 63, slice = tid >> 6;
     const int cx = cell >> 4, cy = (cell >> 2) & 3, cz = cell & 3;
-    const int n_act = a.sb.counters[CTR_N_ACT];
+    const int n_act = active_bricks(a.sb);
     int* work = &a.sb.counters[CTR_WORK_G2P];
     if (tid == 0) s_pose_scene = -1;
     walker_init<kFusedThreads>(a, n_act, vw, bar, s_item, work);
@@ -1352,11 +1397,12 @@ __global__ void __launch_bounds__(kFusedThreads, 4) k_g2p2g(StepArgs a)
         for (int t = tid; t < 4 * kW8Nodes; t += kFusedThreads) (&win[0][0])[t] = 0.0f;
         if (tid < 64) cell_cnt[tid] = 0;
         if (!walker_next(a, n_act, vw, bar, s_item, work, buf, phase, item)) break;
-        const int start = a.sb.act_start[item], count = a.sb.act_count[item], scene = a.sb.act_scene[item];
+        const int e = active_entry(a.sb, item);
+        const int start = a.sb.act_start[e], count = a.sb.act_count[e], scene = a.sb.act_scene[e];
         const SceneDev sc = a.scenes[scene];
         const int n_solid = a.any_solid ? sc.n_rigid : 0;
-        if (n_solid && scene != s_pose_scene) stage_solids(a, scene, s_pose);
-        const int n = sc.n, nb = sc.nb, lb = a.sb.act_brick[item] - sc.brick_base;
+        if (n_solid && scene != s_pose_scene) stage_solids(a, scene, s_pose, tid);
+        const int n = sc.n, nb = sc.nb, lb = a.sb.act_brick[e] - sc.brick_base;
         int ox, oy, oz;
         brick_coords(nb, sc.nb_log2, lb, ox, oy, oz);
         ox *= 4; oy *= 4; oz *= 4;
@@ -1373,8 +1419,20 @@ __global__ void __launch_bounds__(kFusedThreads, 4) k_g2p2g(StepArgs a)
             int key = 0, my_cell = -1, my_rank = 0;
             if (valid) {
                 G2POut o;
-                ebits |= g2p_particle<0>(a, sc, lin, a.sb.perm[start + k], start + k, ox, oy, oz, o);
-                finish_position(a, s_pose, n_solid, start + k, o.x);
+                const int p = a.sb.perm[start + k];
+                float mu, lam;
+                material_of(a, sc, p, mu, lam);
+                ebits |= g2p_particle<0>(
+                    a, sc, plane(a.in, a.cap, 0, p), mu, lam,
+                    [&](const int* bc) {
+                        const int l0 = min(max(bc[0] - ox, 0), 3), l1 = min(max(bc[1] - oy, 0), 3),
+                                  l2 = min(max(bc[2] - oz, 0), 3);
+                        const float4* base = lin + (l0 * 36 + l1 * 6 + l2);
+                        return [base](int i, int j, int kk) { return base[i * 36 + j * 6 + kk]; };
+                    },
+                    [&](float* F) { load_F(a.in, a.cap, p, F); }, o);
+                if (n_solid) push_out(s_pose, n_solid, o.x);
+                store_particle(a, sc.pp_mat, mu, lam, start + k, o);
                 // P2G of the next substep at the new position
                 int bc[3];
                 float f[3], w[9];
@@ -1420,7 +1478,7 @@ __global__ void __launch_bounds__(kFusedThreads, 4) k_g2p2g(StepArgs a)
                             }
                 }
             }
-            const int rank = aggregated_rank_mark(a.sb, sc, key >> 6, valid);
+            const int rank = brick_rank(a.sb, sc, key, valid);
             if (valid) {
                 a.sb.key[start + k] = key;
                 a.sb.rank[start + k] = rank;
@@ -1479,7 +1537,7 @@ __global__ void __launch_bounds__(kStdThreads) k_p2g_std(StepArgs a)
     __shared__ float win[4][kWinNodes];
     __shared__ int s_item;
     const int tid = threadIdx.x;
-    const int n_act = a.sb.counters[CTR_N_ACT];
+    const int n_act = active_bricks(a.sb);
     const int cap = a.cap;
     for (;;) {
         if (tid == 0) s_item = atomicAdd(&a.sb.counters[CTR_WORK_P2G], 1);
@@ -1487,8 +1545,9 @@ __global__ void __launch_bounds__(kStdThreads) k_p2g_std(StepArgs a)
         __syncthreads();
         const int item = s_item;
         if (item >= n_act) break;
-        const int b = a.sb.act_brick[item], start = a.sb.act_start[item], count = a.sb.act_count[item];
-        const int scene = a.sb.act_scene[item];
+        const int e = active_entry(a.sb, item);
+        const int b = a.sb.act_brick[e], start = a.sb.act_start[e], count = a.sb.act_count[e];
+        const int scene = a.sb.act_scene[e];
         const SceneDev sc = a.scenes[scene];
         const int n = sc.n, nb = sc.nb, lb = b - sc.brick_base;
         int ox, oy, oz;
@@ -1500,24 +1559,25 @@ __global__ void __launch_bounds__(kStdThreads) k_p2g_std(StepArgs a)
         for (int k = tid; k < count; k += kStdThreads) {
             const int p = a.sb.perm[start + k];
             int bc[3];
-            float f[3], w[9], dw[9];
-            ebits |= particle_weights(a.in.x[p], a.in.x[cap + p], a.in.x[2 * cap + p], n, bc, f, w);
+            float f[3], w[9], dw[9], x[3];
+            load_x(a.in, p, x);
+            ebits |= particle_weights(x[0], x[1], x[2], n, bc, f, w);
             bspline_d(f[0], dw);
             bspline_d(f[1], dw + 3);
             bspline_d(f[2], dw + 6);
             float t6[6], v[3];
             if (a.tau_valid) {
-#pragma unroll
-                for (int q = 0; q < 6; ++q) t6[q] = a.in.tau[(size_t)q * cap + p];
+                float C[9];
+                load_C_tau(a.in, cap, p, C, t6);
             } else {
                 float F[9];
-#pragma unroll
-                for (int q = 0; q < 9; ++q) F[q] = a.in.F[(size_t)q * cap + p];
+                load_F(a.in, cap, p, F);
                 const float mu = sc.pp_mat ? a.in.mu[p] : sc.mu, lam = sc.pp_mat ? a.in.lam[p] : sc.lam;
                 ebits |= constitutive(a.model, 0, 0.f, mu, lam, F, t6);
             }
+            load_v(a.in, cap, p, v);
 #pragma unroll
-            for (int q = 0; q < 3; ++q) v[q] = m * a.in.v[(size_t)q * cap + p];
+            for (int q = 0; q < 3; ++q) v[q] *= m;
             const float tau[9] = {t6[0], t6[1], t6[2], t6[1], t6[3], t6[4], t6[2], t6[4], t6[5]};
             const int l0 = min(max(bc[0] - ox, 0), 3), l1 = min(max(bc[1] - oy, 0), 3), l2 = min(max(bc[2] - oz, 0), 3);
 #pragma unroll
@@ -1555,84 +1615,56 @@ __global__ void __launch_bounds__(kStdThreads) k_p2g_std(StepArgs a)
 // G2P of a PB-MPM cycle (Sec. III-C): positions and F stay fixed during the
 // cycles, so each particle's v = sum W v_I and APIC C = 4/dx^2 sum W v_I
 // (x_I - x_p)^T are written back in place (storage order), where the next
-// cycle's P2G reads them through the same permutation.
+// cycle's P2G reads them through the same permutation.  It also resets the
+// accumulator for that P2G.
 
 constexpr int kVcThreads = 128;
 
 __global__ void __launch_bounds__(kVcThreads) k_g2p_vc(StepArgs a)
 {
-    __shared__ __align__(128) float4 vw[2][8 * 64];
-    __shared__ __align__(16) float4 lin[kWinNodes];
-    __shared__ __align__(8) unsigned long long bar[2];
-    __shared__ int s_item[2];
-    const int tid = threadIdx.x;
-    const int n_act = a.sb.counters[CTR_N_ACT];
-    const int cap = a.cap;
-    int* work = &a.sb.counters[CTR_WORK_G2P];
-    walker_init<kVcThreads>(a, n_act, vw, bar, s_item, work);
-    unsigned phase[2] = {0u, 0u};
-    int buf = 0;
-    for (;;) {
-        const int item = s_item[buf];
-        if (item >= n_act) break;
-        if (!walker_next(a, n_act, vw, bar, s_item, work, buf, phase, item)) break;
-        const int start = a.sb.act_start[item], count = a.sb.act_count[item];
-        const SceneDev sc = a.scenes[a.sb.act_scene[item]];
-        const int n = sc.n, nb = sc.nb, lb = a.sb.act_brick[item] - sc.brick_base;
-        int ox, oy, oz;
-        brick_coords(nb, sc.nb_log2, lb, ox, oy, oz);
-        ox *= 4; oy *= 4; oz *= 4;
-        const float c4 = 4.0f * (float)n;
-        linearize_window<kVcThreads>(vw[buf], lin);
-        __syncthreads();
-        for (int k = tid; k < count; k += kVcThreads) {
-            const int p = a.sb.perm[start + k];
-            int bc[3];
-            float f[3], w[9];
-            particle_weights(a.in.x[p], a.in.x[cap + p], a.in.x[2 * cap + p], n, bc, f, w);
-            const int l0 = min(max(bc[0] - ox, 0), 3), l1 = min(max(bc[1] - oy, 0), 3), l2 = min(max(bc[2] - oz, 0), 3);
-            float vv[3] = {0.f, 0.f, 0.f}, B[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const int g = blockIdx.x * kVcThreads + threadIdx.x;
+    const int n_clear = a.sb.counters[CTR_N_NACT] * 64;
+    for (int t = g; t < n_clear; t += gridDim.x * kVcThreads)
+        a.G[a.sb.nact_brick[t >> 6] * 64 + (t & 63)] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int s = a.r.p0 + min(g, a.r.np - 1);
+    const SceneDev sc = a.scenes[scene_of_slot(a, s)];
+    if (g >= a.r.np || active_bricks(a.sb) == 0) return;
+    const size_t cap = a.cap;
+    const int p = a.sb.perm[s];
+    float x[3], f[3], w[9], v[3], B[9];
+    int bc[3];
+    load_x(a.in, p, x);
+    particle_weights(x[0], x[1], x[2], sc.n, bc, f, w);
+    gather_velocity<0>(f, w, GridStencil(a.V, sc, bc), v, B);
+    const float c4 = 4.0f * (float)sc.n;
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-#pragma unroll
-                    for (int kk = 0; kk < 3; ++kk) {
-                        const float W = w[i] * w[3 + j] * w[6 + kk];
-                        const float4 g = lin[(l0 + i) * 36 + (l1 + j) * 6 + (l2 + kk)];
-                        const float d0 = (float)i - f[0], d1 = (float)j - f[1], d2 = (float)kk - f[2];
-                        const float gv[3] = {g.x, g.y, g.z};
-#pragma unroll
-                        for (int r = 0; r < 3; ++r) {
-                            vv[r] += W * gv[r];
-                            B[3 * r] += W * gv[r] * d0;
-                            B[3 * r + 1] += W * gv[r] * d1;
-                            B[3 * r + 2] += W * gv[r] * d2;
-                        }
-                    }
-#pragma unroll
-            for (int r = 0; r < 3; ++r) a.in.v[(size_t)r * cap + p] = vv[r];
-#pragma unroll
-            for (int q = 0; q < 9; ++q) a.in.C[(size_t)q * cap + p] = c4 * B[q];
-        }
-        __syncthreads();
-        buf ^= 1;
-    }
+    for (int i = 0; i < 9; ++i) B[i] *= c4;
+    float4* q = a.in.q + p;
+    const float F8 = state_at(a.in, cap, kAtF + 8, p);
+    q[3 * cap] = make_float4(F8, v[0], v[1], v[2]);
+    q[4 * cap] = make_float4(B[0], B[1], B[2], B[3]);
+    q[5 * cap] = make_float4(B[4], B[5], B[6], B[7]);
+    state_at(a.in, cap, kAtC + 8, p) = B[8];
 }
 
 // ------------------------------------------------------- state I/O kernels
+
+// float index in a particle's state of field 0 x, 1 v, 2 C, 3 F
+__device__ __forceinline__ int field_at(int field)
+{
+    return field == 0 ? kAtX : field == 1 ? kAtV : field == 2 ? kAtC : kAtF;
+}
 
 __global__ void k_gather_field(PState st, int cap, int p0, int np, int field, void* dst)
 {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= np) return;
     const int s = p0 + g;
-    const int id = st.id[s];
+    const int id = state_id(st, s);
     if (field == 4) { static_cast<int*>(dst)[g] = id; return; }
-    const float* src = field == 0 ? st.x : field == 1 ? st.v : field == 2 ? st.C : st.F;
-    const int comps = field < 2 ? 3 : 9;
+    const int comps = field < 2 ? 3 : 9, at = field_at(field);
     float* out = static_cast<float*>(dst) + (size_t)id * comps;
-    for (int c = 0; c < comps; ++c) out[c] = src[(size_t)c * cap + s];
+    for (int c = 0; c < comps; ++c) out[c] = state_at(st, cap, at + c, s);
 }
 
 __global__ void k_scatter_field(PState st, int cap, int p0, int np, int field, const float* src)
@@ -1640,11 +1672,10 @@ __global__ void k_scatter_field(PState st, int cap, int p0, int np, int field, c
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= np) return;
     const int s = p0 + g;
-    const int id = st.id[s];
-    float* dst = field == 0 ? st.x : field == 1 ? st.v : field == 2 ? st.C : st.F;
-    const int comps = field < 2 ? 3 : 9;
+    const int id = state_id(st, s);
+    const int comps = field < 2 ? 3 : 9, at = field_at(field);
     const float* in = src + (size_t)id * comps;
-    for (int c = 0; c < comps; ++c) dst[(size_t)c * cap + s] = in[c];
+    for (int c = 0; c < comps; ++c) state_at(st, cap, at + c, s) = in[c];
 }
 
 // Inverse of a scene's slot -> id map: inv[id] = slot.
@@ -1652,7 +1683,7 @@ __global__ void k_id_inverse(PState st, int p0, int np, int* inv)
 {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= np) return;
-    const int id = st.id[p0 + g];
+    const int id = state_id(st, p0 + g);
     if ((unsigned)id < (unsigned)np) inv[id] = p0 + g;
 }
 
@@ -1679,13 +1710,13 @@ __global__ void __launch_bounds__(kIoBlock) k_fields_host(PState st, int cap, in
         float* hp = h.f[f];
         if (!hp) continue;
         const int k = f < 2 ? 3 : 9;
-        float* soa = f == 0 ? st.x : f == 1 ? st.v : f == 2 ? st.C : st.F;
+        const int at = field_at(f);
         float* chunk = hp + (size_t)g0 * k;
         const int nflt = cnt * k;
         const bool vec = cnt == kIoBlock && (reinterpret_cast<uintptr_t>(chunk) & 15u) == 0;
         if (TO_HOST) {
             if (own)
-                for (int c = 0; c < k; ++c) buf[t * k + c] = soa[(size_t)c * cap + s];
+                for (int c = 0; c < k; ++c) buf[t * k + c] = state_at(st, cap, at + c, s);
             __syncthreads();
             if (vec) {
                 for (int i = t; i < nflt / 4; i += kIoBlock)
@@ -1702,7 +1733,7 @@ __global__ void __launch_bounds__(kIoBlock) k_fields_host(PState st, int cap, in
             }
             __syncthreads();
             if (own)
-                for (int c = 0; c < k; ++c) soa[(size_t)c * cap + s] = buf[t * k + c];
+                for (int c = 0; c < k; ++c) state_at(st, cap, at + c, s) = buf[t * k + c];
         }
         __syncthreads();  // buf is the next field's
     }
@@ -1715,17 +1746,17 @@ __global__ void k_init_particles(PState st, int cap, int p_at, int n, int id0, c
     if (g >= n) return;
     const int s = p_at + g;
     for (int d = 0; d < 3; ++d) {
-        st.x[(size_t)d * cap + s] = x[3 * (size_t)g + d];
-        st.v[(size_t)d * cap + s] = v ? v[3 * (size_t)g + d] : 0.f;
+        state_at(st, cap, kAtX + d, s) = x[3 * (size_t)g + d];
+        state_at(st, cap, kAtV + d, s) = v ? v[3 * (size_t)g + d] : 0.f;
     }
     for (int i = 0; i < 9; ++i) {
-        st.C[(size_t)i * cap + s] = 0.f;
-        st.F[(size_t)i * cap + s] = (i % 4 == 0) ? 1.f : 0.f;
+        state_at(st, cap, kAtC + i, s) = 0.f;
+        state_at(st, cap, kAtF + i, s) = (i % 4 == 0) ? 1.f : 0.f;
     }
     const float e = E ? E[g] : E0, q = nu ? nu[g] : nu0;
     st.mu[s] = e / (2.f * (1.f + q));
     st.lam[s] = e * q / ((1.f + q) * (1.f - 2.f * q));
-    st.id[s] = id0 + g;
+    state_id(st, s) = id0 + g;
 }
 
 __global__ void k_read_grid(const float4* V, const int* brick_epoch, const int* epoch, int scene, int n,
@@ -1753,6 +1784,12 @@ cudaError_t launch_prepare(const StepArgs& a, const PState& st, cudaStream_t s)
 {
     if (a.r.np == 0) return cudaSuccess;
     k_prepare<<<n_blocks(a.r.np, 256), 256, 0, s>>>(a, st);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_reset_histogram(const SortBufs& sb, int bricks, int tiles, cudaStream_t s)
+{
+    k_reset_histogram<<<n_blocks(max(bricks, 32), 256), 256, 0, s>>>(sb, bricks, tiles);
     return cudaGetLastError();
 }
 
@@ -1807,7 +1844,8 @@ cudaError_t launch_p2g_std(const StepArgs& a, cudaStream_t s)
 
 cudaError_t launch_g2p_vc(const StepArgs& a, cudaStream_t s)
 {
-    k_g2p_vc<<<a.persistent_ctas, kVcThreads, 0, s>>>(a);
+    if (a.r.np == 0) return cudaSuccess;
+    k_g2p_vc<<<n_blocks(a.r.np, kVcThreads), kVcThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -1818,19 +1856,19 @@ int occupancy_p2g_std()
     return b;
 }
 
-cudaError_t launch_grid(const StepArgs& a, cudaStream_t s)
+cudaError_t launch_grid(const StepArgs& a, cudaStream_t s, bool clear)
 {
     if (!a.any_rigid) k_grid_plain<<<a.grid_plain_ctas, kGridThreads, 0, s>>>(a);
     else if (a.rigid_ext) k_grid<true><<<a.grid_ctas, kGridThreads, 0, s>>>(a);
     else k_grid<false><<<a.grid_ctas, kGridThreads, 0, s>>>(a);
-    k_grid_clear<<<a.grid_plain_ctas, kGridThreads, 0, s>>>(a);
+    if (clear) k_grid_clear<<<a.grid_plain_ctas, kGridThreads, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 template <int FLAGS>
 static void launch_g2p_variant(const StepArgs& a, cudaStream_t s)
 {
-    const int c = a.persistent_ctas;
+    const int c = min(a.g2p_ctas, n_blocks(max(a.r.np, 1), a.g2p_threads));
     if (a.g2p_regs64) {
         switch (a.g2p_threads) {
         case 128: k_g2p<128, 8, FLAGS><<<c, 128, 0, s>>>(a); break;
@@ -1850,7 +1888,7 @@ static void launch_g2p_variant(const StepArgs& a, cudaStream_t s)
 // threads, 64 registers): the MLS-MPM shapes are what the tuner explores.
 cudaError_t launch_g2p(const StepArgs& a, cudaStream_t s)
 {
-    const int c = a.persistent_ctas;
+    const int c = min(a.g2p_ctas, n_blocks(max(a.r.np, 1), 128));
     // the push-out variant only where a scene has a solid shape: blades, needles and
     // segments push nothing out
     if (a.solver == MPM_SOLVER_STANDARD) {

@@ -18,21 +18,19 @@ struct SortBufs {
     int* perm;      // [cap] sorted slot -> storage index
     unsigned char* scell; // [cap] sorted slot -> base cell inside its brick (the key's low 6 bits)
     int* cnt;       // [bricks] particles per brick (next substep)
-    int* nflag;     // [bricks] node brick touched by a particle brick's stencil (set by the
-                    // key producers, read by the scan, cleared by k_grid_clear)
     int* off;       // [bricks] first slot of each active brick
-    int* act_brick; // [bricks] active particle bricks
+    int* act_brick; // [list_size] active particle bricks: those of at least kBigBrick particles from
+                    // the front, the others from the back (active_entry)
     int* act_start;
     int* act_count;
     int* act_scene;
     int* nact_brick;// [bricks] active node bricks
     int* nact_scene;
     int* counters;  // [CTR_COUNT]
-    int4* tile_sum; // [tiles] per scan tile (particles, active particle bricks, active node
-                    // bricks, particle bricks of at least kBigBrick particles) of the
-                    // next substep, added up by the key producers, read by the scan
-                    // and cleared by the scatter
+    int* tile_n;    // [tiles] particles per scan tile of the next substep, added up by the key
+                    // producers, read by the scan and cleared by the scatter
     int tile_shift; // log2 of the bricks per scan tile
+    int list_size;  // entries of the active-brick lists (all bricks)
 };
 
 struct StepArgs {
@@ -54,7 +52,7 @@ struct StepArgs {
     int bound, floor_sticky;
     int model, plasticity;
     float yield_stress;
-    int persistent_ctas;         // CTAs of the persistent G2P kernel
+    int g2p_ctas;                // most CTAs of the persistent G2P kernel
     int p2g_ctas, grid_ctas;     // CTAs of the persistent P2G and grid kernels
     int grid_plain_ctas;         // CTAs of the grid kernel of launches without rigids
     int fused_ctas;              // CTAs of the fused G2P + P2G kernel
@@ -68,21 +66,23 @@ struct StepArgs {
     float pb_beta;               // PB-MPM constraint blend
 };
 
-constexpr int kStateFloats = 32;  // x3 v3 C9 F9 tau6 mu lam (+ int id)
+constexpr int kStateFloats = 34;  // eight float4 planes, mu, lam
 constexpr int kP2GThreads = 192;  // 64 cells x 3 node slices
 constexpr int kScanThreads = 256;
-constexpr int kScanItems = 4;
-constexpr int kScanChunk = kScanThreads * kScanItems;  // bricks per pass of a scan CTA
+constexpr int kMinTileShift = 8;  // a scan tile holds at least kScanThreads bricks
 constexpr int kScatterPer = 4;  // particles per thread of the counting-sort scatter
 // Particle bricks of at least this many particles come first in the active list,
 // so the persistent transfer kernels end on small bricks (a shorter tail)
 constexpr int kBigBrick = 256;
 
 cudaError_t launch_prepare(const StepArgs& a, const PState& st, cudaStream_t s);
+// zero the brick histogram, the tile counts and the list sizes (all scenes)
+cudaError_t launch_reset_histogram(const SortBufs& sb, int bricks, int tiles, cudaStream_t s);
 cudaError_t launch_sort(const StepArgs& a, cudaStream_t s, bool write_perm = true);
 cudaError_t launch_p2g(const StepArgs& a, cudaStream_t s);
 cudaError_t prepare_p2g();  // shared-memory opt-in of the P2G variants (once per device, before any launch)
-cudaError_t launch_grid(const StepArgs& a, cudaStream_t s);
+// clear: reset the P2G accumulator afterwards (G2P does it otherwise)
+cudaError_t launch_grid(const StepArgs& a, cudaStream_t s, bool clear);
 cudaError_t launch_g2p(const StepArgs& a, cudaStream_t s);
 cudaError_t launch_p2g_std(const StepArgs& a, cudaStream_t s);  // standard MPM P2G
 cudaError_t launch_g2p_vc(const StepArgs& a, cudaStream_t s);   // PB-MPM cycle G2P (v, C in place)

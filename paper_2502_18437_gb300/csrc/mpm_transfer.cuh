@@ -85,52 +85,37 @@ __device__ __forceinline__ int cell_key(const SceneDev& sc, float x0, float x1, 
 }
 
 // Warp-aggregated rank: lanes with the same brick get consecutive ranks from
-// one atomic (all 32 lanes call it; `valid` marks lanes with a particle).  It
-// also keeps the scan's bookkeeping of the next substep:
-//  - the brick's particle count (the rank base) and its scan tile's sums;
-//  - for the first warp to add particles to a brick, the brick and its 7 upper
-//    neighbours (+1 in any subset of the axes) are flagged as node bricks the
-//    scan must activate (a particle's 3-node stencil reaches at most 2 nodes
-//    past its base cell, i.e. into the next brick).  Each flag is set with an
-//    exchange, so that its tile counts every node brick exactly once.
-// brick is the global brick index of the key.  add_x = false leaves the tile's
-// particle count to the caller (which then aggregates it itself).
-__device__ __forceinline__ int aggregated_rank_mark(const SortBufs& sb, const SceneDev& sc, int brick, bool valid,
-                                                    bool add_x = true)
+// one atomic (all 32 lanes call it; `valid` marks lanes with a particle), which
+// also counts the brick's particles and its scan tile's for the next substep's
+// scan.  key is the particle's cell_key.  add_tile = false leaves the tile's count
+// to the caller (which then aggregates it itself).
+__device__ __forceinline__ int brick_rank(const SortBufs& sb, const SceneDev& sc, int key, bool valid, bool add_tile = true)
 {
+    const int lane = threadIdx.x & 31, brick = key >> 6;
     const unsigned active = __ballot_sync(kFull, valid);
-    int rank = 0;
-    const unsigned peers = __match_any_sync(kFull, valid ? brick : -1) & active;
-    if (valid) {
-        const int lane = threadIdx.x & 31;
-        const int leader = __ffs(peers) - 1;
-        int base = 0;
-        if (lane == leader) {
-            const int np = __popc(peers);
-            const int lb = brick - sc.brick_base;
-            int4* ts = sb.tile_sum + sc.tile_base;
-            base = atomicAdd(&sb.cnt[brick], np);
-            if (add_x) atomicAdd(&ts[lb >> sb.tile_shift].x, np);
-            if (base < kBigBrick && base + np >= kBigBrick) atomicAdd(&ts[lb >> sb.tile_shift].w, 1);
-            if (base == 0) {
-                atomicAdd(&ts[lb >> sb.tile_shift].y, 1);
-                const int nb = sc.nb;
-                int bx, by, bz;
-                brick_coords(nb, sc.nb_log2, lb, bx, by, bz);
-#pragma unroll
-                for (int o = 0; o < 8; ++o) {
-                    const int ex = bx + (o >> 2), ey = by + ((o >> 1) & 1), ez = bz + (o & 1);
-                    if (ex < nb && ey < nb && ez < nb) {
-                        const int ln = (ex * nb + ey) * nb + ez;
-                        if (atomicExch(&sb.nflag[sc.brick_base + ln], 1) == 0) atomicAdd(&ts[ln >> sb.tile_shift].z, 1);
-                    }
-                }
-            }
-        }
-        base = __shfl_sync(peers, base, leader);
-        rank = base + __popc(peers & ((1u << lane) - 1u));
+    // particles are sorted by brick: a warp that holds one brick only needs no match
+    const int first = __shfl_sync(kFull, brick, active ? __ffs(active) - 1 : 0);
+    const bool one = __all_sync(kFull, !valid || brick == first);
+    const unsigned peers = one ? active : __match_any_sync(kFull, valid ? brick : -1) & active;
+    const int leader = valid ? __ffs(peers) - 1 : lane;
+    int base = 0;
+    if (valid && lane == leader) {
+        const int np = __popc(peers);
+        base = atomicAdd(&sb.cnt[brick], np);
+        if (add_tile) atomicAdd(&sb.tile_n[sc.tile_base + ((brick - sc.brick_base) >> sb.tile_shift)], np);
     }
-    return rank;
+    __syncwarp();
+    return __shfl_sync(kFull, base, leader) + __popc(peers & ((1u << lane) - 1u));
+}
+
+// The active particle bricks: those of at least kBigBrick particles fill the list
+// from its front, the others from its back.
+__device__ __forceinline__ int active_bricks(const SortBufs& sb) { return sb.counters[CTR_N_BIG] + sb.counters[CTR_N_SMALL]; }
+
+__device__ __forceinline__ int active_entry(const SortBufs& sb, int item)
+{
+    const int n_big = sb.counters[CTR_N_BIG];
+    return item < n_big ? item : sb.list_size - 1 - (item - n_big);
 }
 
 // ------------------------------------------------------ transfer helpers
@@ -403,6 +388,7 @@ __device__ __forceinline__ int node_index(const SceneDev& sc, int gi, int gj, in
 
 __device__ __forceinline__ void issue_halo(const StepArgs& a, int item, float4* dst, unsigned long long* bar)
 {
+    item = active_entry(a.sb, item);
     const int b = a.sb.act_brick[item];
     const SceneDev& sc = a.scenes[a.sb.act_scene[item]];
     const int nb = sc.nb, lb = b - sc.brick_base;
@@ -439,30 +425,48 @@ __device__ __forceinline__ void walker_init(const StepArgs& a, int n_act, float4
     __syncthreads();
 }
 
-// Epilogue of the forward G2P launches, run by every CTA on its way out: the
-// last CTA to finish advances the scene clocks and substep counters (read by
-// the next grid update and the state readback).  No CTA of the launch reads a
-// clock after it has counted itself out, so the clocks stay constant while
-// G2P evaluates rigid poses at the end of the substep.
-__device__ __forceinline__ void walker_exit(const StepArgs& a)
+// The lists of this substep are done with: keep their sizes for mpm_phase_stats
+// and start the next scan's from empty.
+__device__ __forceinline__ void reset_lists(const SortBufs& sb)
 {
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    sb.counters[CTR_LAST_ACT] = active_bricks(sb);
+    sb.counters[CTR_LAST_NACT] = sb.counters[CTR_N_NACT];
+    sb.counters[CTR_N_BIG] = sb.counters[CTR_N_SMALL] = sb.counters[CTR_N_NACT] = 0;
+}
+
+// Epilogue of the forward G2P launches, run by one warp of every CTA on its
+// way out: the last CTA to finish advances the scene clocks and substep counters
+// (read by the next grid update and the state readback).  No CTA of the launch
+// reads a clock after it has counted itself out, so the clocks stay constant
+// while G2P evaluates rigid poses at the end of the substep.
+__device__ __forceinline__ void count_out(const StepArgs& a)
+{
+    const int lane = threadIdx.x & 31;
+    int done = 0;
+    if (lane == 0) {
         __threadfence();
-        const int done = atomicAdd(&a.sb.counters[CTR_DONE_G2P], 1);
-        if (done == (int)gridDim.x - 1) {
-            __threadfence();
-            for (int s = a.r.s0; s < a.r.s1; ++s) {
-                a.t_scene[s] += (double)a.dt;
-                a.epoch[s] += 1;
-            }
-            a.sb.counters[CTR_DONE_G2P] = 0;
-        }
+        done = atomicAdd(&a.sb.counters[CTR_DONE_G2P], 1);
+    }
+    if (__shfl_sync(kFull, done, 0) != (int)gridDim.x - 1) return;
+    __threadfence();
+    for (int s = a.r.s0 + lane; s < a.r.s1; s += 32) {
+        a.t_scene[s] += (double)a.dt;
+        a.epoch[s] += 1;
+    }
+    if (lane == 0) {
+        a.sb.counters[CTR_DONE_G2P] = 0;
+        reset_lists(a.sb);
     }
 }
 
+__device__ __forceinline__ void walker_exit(const StepArgs& a)
+{
+    __syncthreads();
+    if (threadIdx.x < 32) count_out(a);
+}
+
 // Poses at the end of the substep (clock + dt) of the solid rigids of a scene,
-// staged in shared memory by the threads tid < kMaxRigids; returns the rigid
+// staged in shared memory by the threads tid < kMaxRigids of a group; the rigid
 // slots in use (shapes other than sphere and box are staged with type -1).
 __device__ __forceinline__ void rigid_pose_at(const RigidDev& src, double t_now, float c[3], float R[9])
 {
@@ -486,9 +490,8 @@ __device__ __forceinline__ void rigid_pose_at(const RigidDev& src, double t_now,
     quat_to_mat(qw, qx, qy, qz, R);
 }
 
-__device__ __forceinline__ void stage_solids(const StepArgs& a, int scene, SolidPose* poses)
+__device__ __forceinline__ void stage_solids(const StepArgs& a, int scene, SolidPose* poses, int tid)
 {
-    const int tid = threadIdx.x;
     const int nr = a.scenes[scene].n_rigid;
     if (tid < nr) {
         const RigidDev& src = a.rigids[scene * kMaxRigids + tid];
@@ -553,7 +556,7 @@ __device__ __forceinline__ bool walker_next(const StepArgs& a, int n_act, float4
     }
     const bool ok = mbar_wait_bounded(&bar[buf], phase[buf]);
     if (__syncthreads_or(!ok)) {
-        if (threadIdx.x == 0) atomicOr(&a.err[a.sb.act_scene[item]], MPM_EBIT_TIMEOUT);
+        if (threadIdx.x == 0) atomicOr(&a.err[a.sb.act_scene[active_entry(a.sb, item)]], MPM_EBIT_TIMEOUT);
         mbar_wait_bounded(&bar[buf], phase[buf]);  // let copies in flight land before leaving
         mbar_wait_bounded(&bar[buf ^ 1], phase[buf ^ 1]);
         return false;
