@@ -97,7 +97,7 @@ enum {
     MPM_OPT_LAUNCH_MODE = 2,    /* 0: one launch per phase over all scenes;
                                    1: one launch per phase per scene (looped)       */
     MPM_OPT_P2G_THREADS = 3,    /* threads per CTA of the P2G kernel: fixed at 192
-                                   (64 cells x 3 node slices); other values rejected */
+                                   (six warps); other values rejected */
     MPM_OPT_G2P_THREADS = 4,    /* threads per CTA of the G2P kernel: 128 / 256 / 512,
                                    or 0 (default): 256 for launches of fewer than
                                    524,288 particles, else 128 (reads back the shape
@@ -107,13 +107,14 @@ enum {
                                    a call of k substeps replays ceil(k/chunk) graphs */
     MPM_OPT_PHASE_TIMING = 7,   /* 0/1: record CUDA events around each phase of every
                                    substep (forces direct launches); see mpm_phase_stats */
-    MPM_OPT_P2G_CHUNK = 8,      /* particles staged per pass of the P2G kernel: 384,
-                                   576 or 768 (default)                             */
+    MPM_OPT_P2G_CHUNK = 8,      /* particles of two passes of a P2G CTA: 384, 576
+                                   or 768 (default), i.e. 32, 48 or 64 staged by each
+                                   of its six warps; small launches stage 32        */
     MPM_OPT_FUSED = 9,          /* 1: fuse each substep's G2P with the next substep's
                                    P2G; 0 (default): separate P2G and G2P kernels */
     MPM_OPT_G2P_REGS64 = 10     /* 1: G2P variant limited to 64 registers (more
                                    resident warps); 0 (default): the larger budget
-                                   (72 registers at 128 threads, 80 at 256, 112
+                                   (80 registers at 128 and 256 threads, 128
                                    at 512)                                          */
 };
 

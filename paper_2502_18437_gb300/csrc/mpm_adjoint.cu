@@ -647,7 +647,6 @@ int mpm_tape_record_substep(mpm_ctx* c, float dt)
     int st;
     if ((st = status_from_cuda(launch_sort(a, c->stream)))) return st;
     MPM_CKA(launch_p2g(a, c->stream));
-    // the permutation G2P uses (P2G leaves it in cell order inside each pass)
     MPM_CKA(cudaMemcpyAsync(t->perms + (size_t)j * c->cap + a.r.p0, c->sb.perm + a.r.p0, sizeof(int) * a.r.np,
                             cudaMemcpyDeviceToDevice, c->stream));
     MPM_CKA(launch_grid(a, c->stream, false));
@@ -710,7 +709,6 @@ static int backward_device(mpm_ctx* c, const SeedIn& seeds, const AdjOut& outs)
         for (int j = j0; j < j1 - 1; ++j) {
             StepArgs a = step_args(c, t->dts[j], 0, c->n_scenes, seg_state(j - j0), seg_state(j - j0 + 1));
             a.tau_valid = 0;
-            a.cell_order = 0;  // the recorded permutation is already the one G2P used
             if ((st = sort_with_perm(c, a, seg_state(j - j0), t->perms + (size_t)j * cap))) return st;
             MPM_CKA(launch_p2g(a, c->stream));
             MPM_CKA(launch_grid(a, c->stream, false));
@@ -720,7 +718,6 @@ static int backward_device(mpm_ctx* c, const SeedIn& seeds, const AdjOut& outs)
         for (int j = j1 - 1; j >= j0; --j) {
             StepArgs a = step_args(c, t->dts[j], 0, c->n_scenes, seg_state(j - j0), seg_state(j - j0));
             a.tau_valid = 0;
-            a.cell_order = 0;
             if ((st = sort_with_perm(c, a, seg_state(j - j0), t->perms + (size_t)j * cap))) return st;
             MPM_CKA(launch_p2g(a, c->stream));
             MPM_CKA(launch_grid(a, c->stream, true));

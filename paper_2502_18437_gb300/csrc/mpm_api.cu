@@ -135,6 +135,14 @@ static int g2p_threads_for(const mpm_ctx* c, int np)
     return np < (1 << 19) ? 256 : 128;
 }
 
+// Slots that each P2G warp stages: a warp's share of half the set pass, and 32 where
+// the launch would not fill the chip.
+static int p2g_slots_for(const mpm_ctx* c, int np)
+{
+    const int slots = c->p2g_chunk / (2 * kP2GThreads / 32);
+    return (long long)np < (long long)slots * c->num_sms * 24 ? 32 : slots;
+}
+
 static int cap_occ(const mpm_ctx* c, int occ)
 {
     if (occ < 1) occ = 1;
@@ -180,8 +188,9 @@ StepArgs step_args(mpm_ctx* c, float dt, int s0, int s1, const PState& in, const
     int& og = c->occ_g2p[c->g2p_regs64 ? 1 : 0][ti];
     if (!og) og = std::max(1, occupancy_g2p(g2p_threads, c->g2p_regs64));
     a.g2p_ctas = c->num_sms * cap_occ(c, og);
-    int& op = c->occ_p2g[c->p2g_chunk / kP2GThreads - 2];
-    if (!op) op = std::max(1, occupancy_p2g(c->p2g_chunk));
+    a.p2g_slots = p2g_slots_for(c, a.r.np);
+    int& op = c->occ_p2g[a.p2g_slots / 16 - 1];
+    if (!op) op = std::max(1, occupancy_p2g(a.p2g_slots));
     if (!c->occ_grid) c->occ_grid = std::max(1, occupancy_grid());
     if (!c->occ_grid_plain) c->occ_grid_plain = std::max(1, occupancy_grid_plain());
     if (!c->occ_fused) c->occ_fused = std::max(1, occupancy_g2p2g());
@@ -190,15 +199,9 @@ StepArgs step_args(mpm_ctx* c, float dt, int s0, int s1, const PState& in, const
     a.grid_ctas = c->num_sms * c->occ_grid;
     a.grid_plain_ctas = c->num_sms * c->occ_grid_plain;
     a.fused_ctas = c->num_sms * cap_occ(c, c->occ_fused);
-    a.p2g_chunk = c->p2g_chunk;
     a.g2p_threads = g2p_threads;
-    a.cell_order = 1;
     a.solver = c->cfg.solver;
     a.pb_beta = c->cfg.pb_beta;
-    if (a.solver == MPM_SOLVER_STANDARD) {
-        if (!c->occ_p2g_std) c->occ_p2g_std = std::max(1, occupancy_p2g_std());
-        a.p2g_ctas = c->num_sms * c->occ_p2g_std;
-    }
     a.any_rigid = 0;
     a.rigid_ext = 0;
     a.any_solid = 0;
@@ -249,8 +252,6 @@ int enqueue_substep(mpm_ctx* c, float dt, const PState& in, const PState& out, b
                 StepArgs b = a;
                 if (k > 0) {
                     for (int d = 0; d < 3; ++d) b.gravity[d] = 0.f;
-                    b.cell_order = 0;  // the first P2G left the permutation in cell order
-                    MPM_CK(cudaMemsetAsync(c->sb.counters + CTR_WORK_P2G, 0, sizeof(int) * 3, c->stream));
                 }
                 MPM_CK(launch_p2g(b, c->stream));
                 MPM_CK(launch_grid(b, c->stream, false));
@@ -264,10 +265,7 @@ int enqueue_substep(mpm_ctx* c, float dt, const PState& in, const PState& out, b
             if (ev) MPM_CK(cudaEventRecord(ev[4], c->stream));
             continue;
         }
-        if (!c->fused || need_p2g) {
-            if (a.solver == MPM_SOLVER_STANDARD) MPM_CK(launch_p2g_std(a, c->stream));
-            else MPM_CK(launch_p2g(a, c->stream));
-        }
+        if (!c->fused || need_p2g) MPM_CK(launch_p2g(a, c->stream));
         if (ev) MPM_CK(cudaEventRecord(ev[2], c->stream));
         MPM_CK(launch_grid(a, c->stream, c->fused != 0));
         if (ev) MPM_CK(cudaEventRecord(ev[3], c->stream));
@@ -330,7 +328,7 @@ static void free_ctx(mpm_ctx* c)
     mpm_tape_free(c);
     clear_graphs(c);
     for (int i = 0; i < 2; ++i) cudaFree(c->state_mem[i]);
-    void* bufs[] = {c->sb.key, c->sb.rank, c->sb.perm, c->sb.scell, c->sb.cnt, c->sb.off, c->sb.act_brick, c->sb.act_start,
+    void* bufs[] = {c->sb.key, c->sb.rank, c->sb.perm, c->sb.cnt, c->sb.ccnt, c->sb.off, c->sb.act_brick, c->sb.act_start,
                     c->sb.act_count, c->sb.act_scene, c->sb.nact_brick, c->sb.nact_scene, c->sb.counters,
                     c->sb.tile_n, c->G, c->V, c->brick_epoch,
                     c->d_scenes, c->d_rigids, c->d_impulse, c->d_err, c->d_time, c->d_epoch, c->d_stage};
@@ -429,8 +427,8 @@ extern "C" int mpm_create(const mpm_config* cfg, void* stream, mpm_ctx** out)
     alloc((void**)&c->sb.key, sizeof(int) * c->cap);
     alloc((void**)&c->sb.rank, sizeof(int) * c->cap);
     alloc((void**)&c->sb.perm, sizeof(int) * c->cap);
-    alloc((void**)&c->sb.scell, c->cap);
     alloc((void**)&c->sb.cnt, sizeof(int) * nbk);
+    alloc((void**)&c->sb.ccnt, sizeof(int) * nbk * 64);
     alloc((void**)&c->sb.off, sizeof(int) * nbk);
     alloc((void**)&c->sb.act_brick, sizeof(int) * nbk);
     alloc((void**)&c->sb.act_start, sizeof(int) * nbk);
@@ -454,6 +452,7 @@ extern "C" int mpm_create(const mpm_config* cfg, void* stream, mpm_ctx** out)
     if (e == cudaSuccess) {
         for (int i = 0; i < 2; ++i) c->st[i] = state_view(c->state_mem[i], c->cap);
         cudaMemsetAsync(c->sb.cnt, 0, sizeof(int) * nbk, c->stream);
+        cudaMemsetAsync(c->sb.ccnt, 0, sizeof(int) * nbk * 64, c->stream);
         cudaMemsetAsync(c->sb.counters, 0, sizeof(int) * CTR_COUNT, c->stream);
         cudaMemsetAsync(c->sb.tile_n, 0, sizeof(int) * c->total_tiles, c->stream);
         cudaMemsetAsync(c->G, 0, sizeof(float4) * nbk * 64, c->stream);
@@ -980,14 +979,15 @@ extern "C" int mpm_autotune(mpm_ctx* c, float dt, int trial_substeps, float* bes
     // snapshot everything a substep changes
     const size_t sbytes = state_bytes(c->cap);
     const size_t nbk = (size_t)c->total_bricks;
-    const size_t total = sbytes + 2 * sizeof(int) * c->cap + sizeof(int) * nbk * 2 + sizeof(int) * c->total_tiles +
+    const size_t total = sbytes + 2 * sizeof(int) * c->cap + sizeof(int) * nbk * 66 + sizeof(int) * c->total_tiles +
                          (sizeof(double) + sizeof(int) + sizeof(unsigned) + sizeof(double) * kMaxRigids * 6) * c->n_scenes;
     char* snap = nullptr;
     MPM_CK(cudaMalloc(&snap, total));
     struct Item { void* live; size_t bytes; };
     const int cur0 = c->cur;
     Item items[] = {{c->state_mem[cur0], sbytes}, {c->sb.key, sizeof(int) * c->cap}, {c->sb.rank, sizeof(int) * c->cap},
-                    {c->sb.cnt, sizeof(int) * nbk}, {c->sb.tile_n, sizeof(int) * c->total_tiles},
+                    {c->sb.cnt, sizeof(int) * nbk}, {c->sb.ccnt, sizeof(int) * nbk * 64},
+                    {c->sb.tile_n, sizeof(int) * c->total_tiles},
                     {c->brick_epoch, sizeof(int) * nbk},
                     {c->d_time, sizeof(double) * c->n_scenes}, {c->d_epoch, sizeof(int) * c->n_scenes},
                     {c->d_err, sizeof(unsigned) * c->n_scenes},

@@ -66,11 +66,10 @@ struct mpm_ctx {
     int fused = 0;
     // occupancy (resident CTAs per SM) of each kernel variant on this device, 0 = not asked yet
     int occ_g2p[2][3] = {};
-    int occ_p2g[3] = {};
+    int occ_p2g[mpm::kP2GMaxSlots / 16] = {};
     int occ_grid = 0;
     int occ_grid_plain = 0;
     int occ_fused = 0;
-    int occ_p2g_std = 0;
     std::vector<cudaEvent_t> phase_events;  // 5 per timed substep
     size_t phase_used = 0;
     std::map<std::tuple<uint32_t, int, int>, cudaGraphExec_t> graphs;

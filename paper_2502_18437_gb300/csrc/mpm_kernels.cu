@@ -3,10 +3,10 @@
 //   k_scan     brick histogram -> particle offsets, active particle-brick and
 //              node-brick lists (tile counts kept by the key producers: no
 //              inter-CTA waits, empty tiles skipped)
-//   k_scatter  counting-sort scatter: permutation sorted slot -> particle
-//   k_p2g      P2G (Eq. 1, Eq. 8): balanced per-cell work items summed in
-//              registers into shared-memory 6^3 node windows per brick, flushed
-//              to HBM with vector atomics; leaves the permutation in cell order
+//   k_scatter  counting-sort scatter: permutation sorted slot -> particle, by brick
+//              and cell
+//   k_p2g      P2G (Eq. 1, Eq. 8; standard MPM Eq. 2, 3): runs of particles of one
+//              cell summed in registers, added to HBM with vector atomics
 //   k_grid     grid update (Eq. 3), rigid contact (Sec. IV, Eq. 11, Eq. 12),
 //              domain walls (k_grid_plain where no scene has a rigid)
 //   k_grid_clear  reset of the P2G accumulator where no G2P does it
@@ -183,20 +183,28 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(StepArgs a)
 __global__ void k_reset_histogram(SortBufs sb, int bricks, int tiles)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < bricks) sb.cnt[i] = 0;
+    if (i < bricks && sb.cnt[i]) {
+        // only bricks with particles have counts in their cells
+        sb.cnt[i] = 0;
+        for (int k = 0; k < 16; ++k) reinterpret_cast<int4*>(sb.ccnt + (size_t)i * 64)[k] = make_int4(0, 0, 0, 0);
+    }
     if (i < tiles) sb.tile_n[i] = 0;
     if (i >= CTR_N_BIG && i <= CTR_N_NACT) sb.counters[i] = 0;
 }
 
-// Counting-sort scatter; also clears the range's tile counts for the next
-// substep (the scan has read them).  write_perm = 0 only clears (the adjoint
+// Counting-sort scatter: slot = first slot of the brick + particles in the brick's
+// cells before the particle's + its rank in the cell.  The cells' prefix sums are
+// taken by the warp, brick by brick of its particles (nearly always one: the
+// particles were sorted a substep ago).  Also clears the range's tile counts for the
+// next substep (the scan has read them).  write_perm = 0 only clears (the adjoint
 // reuses a recorded permutation).
 // Each thread takes kScatterPer particles, 256 apart, with their loads issued
 // together (a 1M-particle range in one wave of CTAs).
 __global__ void __launch_bounds__(256) k_scatter(StepArgs a, int write_perm)
 {
-    const int g0 = blockIdx.x * (256 * kScatterPer) + threadIdx.x;
-    int key[kScatterPer], rank[kScatterPer], dst[kScatterPer];
+    const int g0 = blockIdx.x * (256 * kScatterPer) + threadIdx.x, lane = threadIdx.x & 31;
+    int key[kScatterPer], rank[kScatterPer], first[kScatterPer], start[kScatterPer];
+    int2 cells[kScatterPer];
 #pragma unroll
     for (int u = 0; u < kScatterPer; ++u) {
         const int g = g0 + u * 256;
@@ -207,21 +215,44 @@ __global__ void __launch_bounds__(256) k_scatter(StepArgs a, int write_perm)
             rank[u] = a.sb.rank[a.r.p0 + g];
         }
     }
+    const auto in_range = [&](int brick) { return brick >= a.r.bb0 && brick < a.r.bb0 + a.r.nbr; };
+    const auto load_cells = [&](int brick) {
+        return in_range(brick) ? reinterpret_cast<const int2*>(a.sb.ccnt + (size_t)brick * 64)[lane] : make_int2(0, 0);
+    };
 #pragma unroll
     for (int u = 0; u < kScatterPer; ++u) {
-        const int brick = key[u] >> 6;
-        dst[u] = (key[u] >= 0 && brick >= a.r.bb0 && brick < a.r.bb0 + a.r.nbr) ? __ldg(&a.sb.off[brick]) + rank[u] : -1;
+        // the brick of the warp's first particle
+        first[u] = __shfl_sync(kFull, key[u] >> 6, 0);
+        cells[u] = load_cells(first[u]);
+        start[u] = in_range(first[u]) ? a.sb.off[first[u]] : 0;
     }
 #pragma unroll
     for (int u = 0; u < kScatterPer; ++u) {
-        const int g = g0 + u * 256;
-        if (write_perm && g < a.r.np) {
-            if (dst[u] >= a.r.p0 && dst[u] < a.r.p0 + a.r.np) {
-                a.sb.perm[dst[u]] = a.r.p0 + g;
-                a.sb.scell[dst[u]] = (unsigned char)(key[u] & 63);
-            } else {
-                atomicOr(&a.err[a.r.s0], MPM_EBIT_INTERNAL);
+        const int g = g0 + u * 256, brick = key[u] >> 6, cell = key[u] & 63;
+        unsigned todo = __ballot_sync(kFull, key[u] >= 0);
+        int dst = -1, b = first[u];
+        int2 c = cells[u];
+        int st = start[u];
+        while (todo) {
+            int incl = c.x + c.y;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int t = __shfl_up_sync(kFull, incl, d);
+                if (lane >= d) incl += t;
             }
+            const int before = __shfl_sync(kFull, incl - c.y, cell >> 1), even = __shfl_sync(kFull, c.x, cell >> 1);
+            const bool mine = key[u] >= 0 && brick == b;
+            if (mine && in_range(b)) dst = st + before - (cell & 1 ? 0 : even) + rank[u];
+            todo &= ~__ballot_sync(kFull, mine);
+            if (todo) {
+                b = __shfl_sync(kFull, brick, __ffs(todo) - 1);
+                c = load_cells(b);
+                st = in_range(b) ? a.sb.off[b] : 0;
+            }
+        }
+        if (write_perm && g < a.r.np) {
+            if (dst >= a.r.p0 && dst < a.r.p0 + a.r.np) a.sb.perm[dst] = a.r.p0 + g;
+            else atomicOr(&a.err[a.r.s0], MPM_EBIT_INTERNAL);
         }
         if (g < a.r.nt) a.sb.tile_n[a.r.t0 + g] = 0;
     }
@@ -262,7 +293,7 @@ __global__ void __launch_bounds__(256) k_prepare(StepArgs a, PState st)
         key = cell_key(sc, x[0], x[1], x[2], ood);
         if (ood) ebits |= MPM_EBIT_OUT_OF_DOMAIN;
     }
-    const int rank = brick_rank(a.sb, sc, key, valid, !block_sums);
+    const int rank = cell_rank_end(cell_rank_begin(a.sb, sc, key, valid, !block_sums));
     if (valid) {
         a.sb.key[i] = key;
         a.sb.rank[i] = rank;
@@ -277,267 +308,317 @@ __global__ void __launch_bounds__(256) k_prepare(StepArgs a, PState st)
     }
 }
 
-// ------------------------------------------------------------------ P2G
-//
-// One CTA per active particle brick (4^3 cells, a 6^3-node window), 192
-// threads.  Per pass over up to PER x 192 particles of the brick:
-//   A1. one thread per particle: base cell (stored by the sort beside the
-//      permutation) and rank inside the cell;
-//   (warp 0) the cells' particles are cut into at most 64 balanced work items
-//      (build_items), so that the lanes of a warp run loops of nearly equal
-//      length instead of as long as the warp's fullest cell;
-//   A2. stress, weights and P2G coefficients into a record in shared memory at
-//      slot base(warp) + (position in item) x 33 + lane of the item, so that
-//      the 32 lanes of a warp read 32 consecutive words in phase B and the
-//      particles of one item (consecutive lanes here when the input is in cell
-//      order) write to different banks; a pass whose two item warps need more
-//      than the pass's record slots falls back to cell-sorted slots.  The pass's slots
-//      of the permutation are rewritten in cell order (cell_order), so that G2P
-//      gathers a warp's 27-node stencils from a few neighbouring cells;
-//   B.  thread (item, slice i) sums, in registers, the contributions of its
-//      item's particles to the 9 nodes cell + (i, j, k) and stages the sums;
-//   C.  thread (cell, slice i) adds the staged sums of its cell's items and
-//      adds them to slice i's copy of the 6^3 window: the 64 cells of a slice
-//      never write the same node at once, so no atomics are needed.
-// At the end of the pass the window is added to HBM with one vector reduction
-// per node.  Stage and windows reuse the record slots.
-
-__device__ __forceinline__ void prefetch_l2(const float4* p)
+// Scene of slot s (scenes own consecutive slots): two warp-wide probes of the
+// scenes' first slots for the warp's first slot, then the few lanes of later scenes
+// step on.  Every lane of the warp calls it.
+__device__ __forceinline__ int scene_of_slot(const StepArgs& a, int s)
 {
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+    if (a.r.s1 - a.r.s0 == 1) return a.r.s0;
+    const int lane = threadIdx.x & 31, s_first = __shfl_sync(kFull, s, 0);
+    int lo = a.r.s0, len = a.r.s1 - a.r.s0;
+    while (len > 1) {  // p_begin never decreases: the last scene that starts at or before s_first
+        const int step = (len + 31) >> 5, at = lane * step;
+        const bool le = at < len && a.scenes[lo + at].p_begin <= s_first;
+        const int k = 31 - __clz(__ballot_sync(kFull, le) | 1u);
+        lo += k * step;
+        len = min(step, len - k * step);
+    }
+    while (lo + 1 < a.r.s1 && a.scenes[lo + 1].p_begin <= s) ++lo;
+    return lo;
 }
 
-constexpr int kP2GSlotPitch = 33;  // 32 lanes + 1: rows of one item fall in different banks
-// record slots of a pass of PER x 192 particles (the rows of the interleaved
-// layout; 768-particle passes need 24).  A smaller record area leaves more of
-// the SM's shared storage to L1.
-template <int PER>
-struct P2GShape {
-    static constexpr int slots = (PER == 4 ? 24 : 21) * kP2GSlotPitch;
-};
-constexpr int kSliceNodes = 4 * 36;  // node planes x = slice .. slice + 3 of the 6^3 window
-constexpr int kStageFloats = 36 * 3 * 64;  // (9 nodes x 4 values) x 3 slices x 64 items
-constexpr int kWinFloats = 3 * 4 * kSliceNodes;  // the slices' windows, after the stage
+__device__ __forceinline__ void cp_async16(float4* dst, const float4* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// ------------------------------------------------------------------ P2G
+//
+// Warps work on their own chunks of sorted slots, without barriers:
+//   A. one lane per particle: weights and coefficients into a record in the warp's
+//      share of the shared memory, and the runs of slots with the same base cell
+//      (the slots are in cell order);
+//   B. one lane per (run, node plane x = i) sums its particles' contributions to the
+//      9 nodes (i, j, k) of the cell in registers;
+//   C. the sums of runs that are neighbours in z are joined by shuffles, and each node
+//      of the joined runs added to HBM with one vector reduction.
+// What bounds it is the instruction issue of B (61 % of the cycles; 28.4 M warp
+// instructions per launch on the 1M block) and the loads of A, which are copied one
+// batch ahead.  Before, a CTA took a brick: ranks in its cells, work items, staged item
+// sums and a 6^3 window, one behind the other with a barrier between: 35.7 M
+// instructions, 13.5 us for a lone brick and so 66 us for the 1M block's 2,744 and 19 us
+// for 64k particles.  Now 49 us and 6 us; PB-MPM's cycles at 131k 39 -> 17 us; the
+// standard MPM at 131k, which took shared-memory atomics, 97 -> 13 us.  The bricks' cell
+// counts come from G2P, so that the sort orders the slots by cell.
+// Joining halves the reductions, and with them the error of the sums: C of a falling 64k
+// block is 4.8e-6 off after 25 substeps, as before; without, 5.4e-6.
+// Tried: a lane per node column (j, k), three groups of lanes at a third of the chunk
+// each: 56 us, every lane reads 18 floats per particle from shared memory; the layer's
+// sums joined in a window of 3 x 6 x 6 nodes: 62 us.
+
+constexpr int kP2GWarps = kP2GThreads / 32;
+constexpr int kRecPitch = 20;  // floats per record: an odd number of 16-byte words
 
 // MODE: kP2GStress (MLS-MPM: the Kirchhoff stress, stored by G2P or computed
-// from F) or kP2GConstraint (PB-MPM: the co-rotational constraint replaces C
-// and there is no stress term).
-enum { kP2GStress = 0, kP2GConstraint = 1 };
+// from F), kP2GConstraint (PB-MPM: the co-rotational constraint replaces C
+// and there is no stress term) or kP2GStd (standard MPM, Sec. III-A: W m v and the
+// internal-force impulse -dt V0 tau grad W, Eq. 2, 3).
+enum { kP2GStress = 0, kP2GConstraint = 1, kP2GStd = 2 };
 
-template <int PER, int MODE>
-__global__ void __launch_bounds__(kP2GThreads, 4) k_p2g(StepArgs a)
+constexpr int kRawPlanes = 7;  // planes of the state that a lane reads
+
+// shared bytes of a warp: records, the next particles' planes, scenes and first slots of the runs
+__host__ __device__ constexpr int p2g_warp_bytes(int slots)
 {
-    constexpr int CHUNK = PER * kP2GThreads;
-    constexpr int kP2GSlots = P2GShape<PER>::slots;
-    static_assert(CHUNK <= kP2GSlots, "a pass fits the record slots");
-    static_assert(kStageFloats + kWinFloats <= kItemRecFields * kP2GSlots, "stage and windows reuse the record slots");
-    extern __shared__ __align__(16) float rec_dyn[];
-    float(*rec)[kP2GSlots] = reinterpret_cast<float(*)[kP2GSlots]>(rec_dyn);  // [kItemRecFields][kP2GSlots]
-    // written once phase B has read every record: the staged item sums [36][3][64]
-    // and one window per slice (slice i writes node planes x = i..i+3 only, so the
-    // slices' writes never collide), added to HBM at the end of each pass
-    float* stage = rec_dyn;
-    float(*win)[4][kSliceNodes] = reinterpret_cast<float(*)[4][kSliceNodes]>(rec_dyn + kStageFloats);
-    __shared__ int cell_cnt[64], cell_off[65];
-    __shared__ short it_cell[64], it_beg[64], it_len[64], c_full[64], c_nf[64], c_rem[64];
-    __shared__ int s_item, s_nitems, s_len[3];
-    const int tid = threadIdx.x;
-    const int t = tid & 63, slice = tid >> 6;
-    const int n_act = active_bricks(a.sb);
-    const int cap = a.cap;
-    for (;;) {
-        if (tid == 0) s_item = atomicAdd(&a.sb.counters[CTR_WORK_P2G], 1);
-        if (tid < 64) cell_cnt[tid] = 0;
-        __syncthreads();
-        const int item = s_item;
-        if (item >= n_act) break;
-        const int e = active_entry(a.sb, item);
-        const int b = a.sb.act_brick[e], start = a.sb.act_start[e], count = a.sb.act_count[e];
-        const int scene = a.sb.act_scene[e];
-        const SceneDev sc = a.scenes[scene];
-        const int n = sc.n, nb = sc.nb, lb = b - sc.brick_base;
-        int ox, oy, oz;
-        brick_coords(nb, sc.nb_log2, lb, ox, oy, oz);
-        ox *= 4; oy *= 4; oz *= 4;
-        const float fn = (float)n, dxs = 1.0f / fn;
-        const float m = sc.m_p;
-        const float kA = a.dt * sc.V0 * 4.0f * fn * fn;
-        unsigned ebits = 0;
+    return slots * (kRecPitch + 1) * (int)sizeof(float) + kRawPlanes * 32 * (int)sizeof(float4) + ((slots + 8) * (int)sizeof(short) + 15) / 16 * 16;
+}
 
-        for (int c0 = 0; c0 < count; c0 += CHUNK) {
-            const int cn = min(CHUNK, count - c0);
-            // A1: cell and rank of each particle of the pass
-            int pp[PER], pc[PER], pr[PER];
+// Record of the particle in storage p, returning its base node's index (key):
+//   fx wy[3] wz[3] -, then for MLS- and PB-MPM q0 q1 A00 A10, A01 A11 A02 A12,
+//   q2 A20 A21 A22: the momentum of node (i, j, k) is W (q + A (i-1, j-1, k-1)) (offsets
+//   from the middle node keep the terms that cancel small); for the standard MPM
+//   m v[3] fy, T0 T1 T2 T3, T4 T5 fz - with T = dt V0 n tau.
+// plane(k) returns plane k of the particle's state.
+template <int MODE, class Plane>
+__device__ __forceinline__ unsigned p2g_record(const StepArgs& a, const SceneDev& sc, int p, Plane plane, float4* rec,
+                                               int& key)
+{
+    const int n = sc.n, nb = sc.nb;
+    const float fn = (float)n, m = sc.m_p;
+    int bc[3];
+    float f[3], w[9], v[3], C[9], t6[6];
+    const float4 x = plane(0), Fv = plane(3);
+    v[0] = Fv.y; v[1] = Fv.z; v[2] = Fv.w;
+    const auto get_F = [&](float* F) {
+        const float4 u = plane(1), t = plane(2);
+        F[0] = u.x; F[1] = u.y; F[2] = u.z; F[3] = u.w;
+        F[4] = t.x; F[5] = t.y; F[6] = t.z; F[7] = t.w;
+        F[8] = Fv.x;
+    };
+    if (MODE != kP2GStd) {
+        const float4 u = plane(4), t = plane(5);
+        C[0] = u.x; C[1] = u.y; C[2] = u.z; C[3] = u.w;
+        C[4] = t.x; C[5] = t.y; C[6] = t.z; C[7] = t.w;
+        C[8] = plane(6).x;
+    }
+    unsigned ebits = particle_weights(x.x, x.y, x.z, n, bc, f, w);
+    key = (sc.brick_base + ((bc[0] >> 2) * nb + (bc[1] >> 2)) * nb + (bc[2] >> 2)) * 64 + (bc[0] & 3) * 16 +
+          (bc[1] & 3) * 4 + (bc[2] & 3);
+    if (MODE == kP2GConstraint) {
+        float F[9];
+        get_F(F);
+        pb_constraint(F, a.dt, a.pb_beta, C);
 #pragma unroll
-            for (int u = 0; u < PER; ++u) {
-                const int k = tid + u * kP2GThreads;
-                pc[u] = -1;
-                if (k < cn) {
-                    const int p = a.sb.perm[start + c0 + k];
-                    pp[u] = p;
-                    if (a.cell_order) {
-                        // the sort stored each slot's cell: no dependent load of x here
-                        pc[u] = a.sb.scell[start + c0 + k];
-                    } else {
-                        // a recorded permutation (differentiation): the cell from x
-                        int c[3];
-                        float x[3];
-                        load_x(a.in, p, x);
-                        const unsigned ood = base_cell(x[0], n, c[0]) | base_cell(x[1], n, c[1]) | base_cell(x[2], n, c[2]);
-                        if (ood) ebits |= MPM_EBIT_OUT_OF_DOMAIN;
-                        const int l0 = min(max(c[0] - ox, 0), 3), l1 = min(max(c[1] - oy, 0), 3),
-                                  l2 = min(max(c[2] - oz, 0), 3);
-                        pc[u] = (l0 * 4 + l1) * 4 + l2;
-                    }
-                    pr[u] = atomicAdd(&cell_cnt[pc[u]], 1);
-                }
+        for (int q = 0; q < 6; ++q) t6[q] = 0.f;
+    } else if (a.tau_valid) {
+        const float4 u = plane(6), t = plane(7);
+        t6[0] = u.y; t6[1] = u.z; t6[2] = u.w;
+        t6[3] = t.x; t6[4] = t.y; t6[5] = t.z;
+    } else {
+        // stress of the current F (after host writes, or seeding a fused run)
+        float F[9];
+        get_F(F);
+        const float mu = sc.pp_mat ? a.in.mu[p] : sc.mu, lam = sc.pp_mat ? a.in.lam[p] : sc.lam;
+        ebits |= constitutive(a.model, 0, 0.f, mu, lam, F, t6);
+    }
+    rec[0] = make_float4(f[0], w[3], w[4], w[5]);
+    rec[1] = make_float4(w[6], w[7], w[8], __int_as_float(key));
+    if (MODE == kP2GStd) {
+        const float kap = a.dt * sc.V0 * fn;  // dt V0 times the n of grad W = n dW/df
+        rec[2] = make_float4(m * v[0], m * v[1], m * v[2], f[1]);
+        rec[3] = make_float4(kap * t6[0], kap * t6[1], kap * t6[2], kap * t6[3]);
+        rec[4] = make_float4(kap * t6[4], kap * t6[5], f[2], 0.f);
+    } else {
+        float q[3], Ad[9];
+        const float fc[3] = {f[0] - 1.f, f[1] - 1.f, f[2] - 1.f};
+        p2g_coeffs(m, a.dt * sc.V0 * 4.0f * fn * fn, 1.0f / fn, v, C, t6, fc, q, Ad);
+        rec[2] = make_float4(q[0], q[1], Ad[0], Ad[3]);
+        rec[3] = make_float4(Ad[1], Ad[4], Ad[2], Ad[5]);
+        rec[4] = make_float4(q[2], Ad[6], Ad[7], Ad[8]);
+    }
+    return ebits;
+}
+
+// Adds a record's contributions to the nodes (i, j, k) of plane i: (p_x, p_y) in
+// acc_a[3 j + k], (p_z, weight) in acc_b.
+template <int MODE>
+__device__ __forceinline__ void p2g_add(const float4* rec, int i, float2 acc_a[9], float2 acc_b[9])
+{
+    const auto two = [](float s) { return make_float2(s, s); };
+    const float4 r0 = rec[0], r1 = rec[1], r2 = rec[2], r3 = rec[3], r4 = rec[4];
+    const float wy[3] = {r0.y, r0.z, r0.w}, wz[3] = {r1.x, r1.y, r1.z};
+    // w_i(f) = alpha + beta (f - gamma)^2
+    const float gam = i == 0 ? 1.5f : (i == 1 ? 1.0f : 0.5f), bet = i == 1 ? -1.0f : 0.5f, alp = i == 1 ? 0.75f : 0.0f;
+    const float e = r0.x - gam, wi = __fmaf_rn(bet * e, e, alp);
+    if (MODE == kP2GStd) {
+        // p = (wx m v - dwx T_x) wy wz - wx (T_y dwy wz + T_z wy dwz)
+        const float dwx = 2.f * bet * e;
+        const float mv[3] = {r2.x, r2.y, r2.z}, T[9] = {r3.x, r3.y, r3.z, r3.y, r3.w, r4.x, r3.z, r4.x, r4.y};
+        float dy[3], dz[3];
+        bspline_d(r2.w, dy);
+        bspline_d(r4.z, dz);
+        float A[3], B[3], C[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            A[c] = wi * mv[c] - dwx * T[3 * c];
+            B[c] = wi * T[3 * c + 1];
+            C[c] = wi * T[3 * c + 2];
+        }
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            float P[3], Q[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                P[c] = wy[j] * A[c] - dy[j] * B[c];
+                Q[c] = -wy[j] * C[c];
             }
-            // the pass's particle fields start towards L2 while warp 0 builds the items
-            // (phase A2 then loads them from L2 rather than from HBM)
+            const float W = wi * wy[j];
 #pragma unroll
-            for (int u = 0; u < PER; ++u) {
-                if (pc[u] < 0) continue;
-                const int p = pp[u];
-                const bool stress = MODE == kP2GStress && a.tau_valid;
-#pragma unroll
-                for (int k = 0; k < kPlanes; ++k)
-                    if (stress ? (k != 1 && k != 2) : k != 7) prefetch_l2(a.in.q + (size_t)k * cap + p);
-            }
-            __syncthreads();
-            if (tid < 32)
-                build_items(cell_cnt, cell_off, cn, it_cell, it_beg, it_len, &s_nitems, c_full, c_nf, c_rem, s_len);
-            __syncthreads();
-            const int L = s_len[0], n_items = s_nitems;
-            const int rows0 = s_len[1], rows1 = s_len[2];  // record rows of the two item warps
-            const bool inter = kP2GSlotPitch * (rows0 + rows1) <= kP2GSlots;
-            const float invL = 1.0f / (float)L;
-            if (tid < 64) cell_cnt[tid] = 0;  // counts of the next pass (last read before the barrier)
-            // A2: records at their slots
-#pragma unroll
-            for (int u = 0; u < PER; ++u) {
-                if (pc[u] < 0) continue;
-                const int c = pc[u], r = pr[u], nf = c_nf[c];
-                // the pass's slots in cell order: G2P then reads (and stores) the
-                // particles of a warp from a few neighbouring cells
-                if (a.cell_order) a.sb.perm[start + c0 + cell_off[c] + r] = pp[u];
-                int slot;
-                if (!inter) {
-                    slot = cell_off[c] + r;
-                } else {
-                    int ti, it;
-                    if (r < nf * L) {
-                        const int j = div_small(r, invL);
-                        ti = c_full[c] + j;
-                        it = r - j * L;
-                    } else {
-                        ti = c_rem[c];
-                        it = r - nf * L;
-                    }
-                    slot = (ti < 32 ? 0 : kP2GSlotPitch * rows0) + it * kP2GSlotPitch + (ti & 31);
-                }
-                const int p = pp[u];
-                int bc[3];
-                float f[3], w[9], x[3];
-                load_x(a.in, p, x);
-                ebits |= particle_weights(x[0], x[1], x[2], n, bc, f, w);
-                float C[9], v[3], t6[6];
-                load_v(a.in, cap, p, v);
-                if (MODE == kP2GConstraint) {
-                    float F[9];
-                    load_C(a.in, cap, p, C);
-                    load_F(a.in, cap, p, F);
-                    pb_constraint(F, a.dt, a.pb_beta, C);
-#pragma unroll
-                    for (int q = 0; q < 6; ++q) t6[q] = 0.f;
-                } else if (a.tau_valid) {
-                    load_C_tau(a.in, cap, p, C, t6);
-                } else {
-                    // stress of the current F (after host writes, or seeding a fused run)
-                    float F[9];
-                    load_C(a.in, cap, p, C);
-                    load_F(a.in, cap, p, F);
-                    const float mu = sc.pp_mat ? a.in.mu[p] : sc.mu, lam = sc.pp_mat ? a.in.lam[p] : sc.lam;
-                    ebits |= constitutive(a.model, 0, 0.f, mu, lam, F, t6);
-                }
-                float q3[3], Ad[9];
-                p2g_coeffs(m, kA, dxs, v, C, t6, f, q3, Ad);
-                put_item_record<kP2GSlots>(rec, slot, f, q3, Ad);
-            }
-            __syncthreads();
-            // B: item sums in registers, then staged
-            float2 acc_a[9], acc_b[9];  // (p_x, p_y), (p_z, weight)
-#pragma unroll
-            for (int q = 0; q < 9; ++q) acc_a[q] = acc_b[q] = make_float2(0.f, 0.f);
-            if (t < n_items)
-                item_accumulate<kP2GSlots>(rec, inter ? (t < 32 ? 0 : kP2GSlotPitch * rows0) + (t & 31) : it_beg[t],
-                                           inter ? kP2GSlotPitch : 1,
-                                           it_len[t], slice, acc_a, acc_b);
-            __syncthreads();
-            for (int q = tid; q < kWinFloats; q += kP2GThreads) (&win[0][0][0])[q] = 0.0f;
-            if (t < n_items) {
-                float* st = stage + slice * 64 + t;
-#pragma unroll
-                for (int q = 0; q < 9; ++q) {
-                    st[(4 * q) * 192] = acc_b[q].y * m;
-                    st[(4 * q + 1) * 192] = acc_a[q].x;
-                    st[(4 * q + 2) * 192] = acc_a[q].y;
-                    st[(4 * q + 3) * 192] = acc_b[q].x;
-                }
-            }
-            __syncthreads();
-            // C: cell owners add their items' sums to their slice's window
-            {
-                const int c = t, nf = c_nf[c], f0 = c_full[c], pr_item = c_rem[c];
-                const int cx = c >> 4, cy = (c >> 2) & 3, cz = c & 3;
-                float sum[36];
-#pragma unroll
-                for (int q = 0; q < 36; ++q) sum[q] = 0.f;
-                const bool any = nf > 0 || pr_item >= 0;
-                for (int j = 0; j <= nf; ++j) {
-                    const int it = j < nf ? f0 + j : pr_item;
-                    if (it < 0) break;
-                    const float* st = stage + slice * 64 + it;
-#pragma unroll
-                    for (int q = 0; q < 36; ++q) sum[q] += st[q * 192];
-                }
-                // for one (j, k) the 64 cells of a slice write distinct nodes (the two
-                // warps of a slice cover disjoint x ranges); a node written for (j, k)
-                // is read for another (j, k) by a neighbour lane: warp barrier between
-                float(*w)[kSliceNodes] = win[slice];
-#pragma unroll
-                for (int q = 0; q < 9; ++q) {
-                    if (any) {
-                        const int node = cx * 36 + (cy + q / 3) * 6 + (cz + q % 3);
-                        w[0][node] += sum[4 * q];
-                        w[1][node] += sum[4 * q + 1];
-                        w[2][node] += sum[4 * q + 2];
-                        w[3][node] += sum[4 * q + 3];
-                    }
-                    __syncwarp();
-                }
-            }
-            __syncthreads();
-            // the pass's window to HBM, one vector reduction per node (read before
-            // the next pass's records overwrite it: two barriers away)
-            for (int q = tid; q < kWinNodes; q += kP2GThreads) {
-                const int X = q / 36, yz = q % 36;
-                float s4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int sl = 0; sl < 3; ++sl) {
-                    const int cx = X - sl;
-                    if (cx < 0 || cx > 3) continue;
-#pragma unroll
-                    for (int comp = 0; comp < 4; ++comp) s4[comp] += win[sl][comp][cx * 36 + yz];
-                }
-                if (s4[0] == 0.0f) continue;
-                const int gi = ox + X, gj = oy + yz / 6, gk = oz + yz % 6;
-                if (gi >= n || gj >= n || gk >= n) continue;
-                red_add_v4(&a.G[node_index(sc, gi, gj, gk)], s4[0], s4[1], s4[2], s4[3]);
+            for (int k = 0; k < 3; ++k) {
+                const int q = 3 * j + k;
+                acc_a[q] = __ffma2_rn(make_float2(P[0], P[1]), two(wz[k]), acc_a[q]);
+                acc_a[q] = __ffma2_rn(make_float2(Q[0], Q[1]), two(dz[k]), acc_a[q]);
+                acc_b[q] = __ffma2_rn(make_float2(P[2], W), two(wz[k]), acc_b[q]);
+                acc_b[q].x = __fmaf_rn(Q[2], dz[k], acc_b[q].x);
             }
         }
-        if (ebits) atomicOr(&a.err[scene], ebits);
-        __syncthreads();
+        return;
     }
+    const float si = (float)(i - 1);
+    const float2 a1 = make_float2(r3.x, r3.y), a2 = make_float2(r3.z, r3.w);
+    const float2 v01 = __ffma2_rn(two(si), make_float2(r2.z, r2.w), make_float2(r2.x, r2.y));
+    const float v2 = __fmaf_rn(si, r4.y, r4.x);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const float wij = wi * wy[j], fj = (float)(j - 1);
+        const float2 s01 = j == 1 ? v01 : __ffma2_rn(two(fj), a1, v01);
+        const float s2 = j == 1 ? v2 : __fmaf_rn(fj, r4.z, v2);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float W = wij * wz[k], fk = (float)(k - 1);
+            const int q = 3 * j + k;
+            const float2 u01 = k == 1 ? s01 : __ffma2_rn(two(fk), a2, s01);
+            const float2 u2w = make_float2(k == 1 ? s2 : __fmaf_rn(fk, r4.w, s2), 1.0f);
+            acc_a[q] = __ffma2_rn(two(W), u01, acc_a[q]);
+            acc_b[q] = __ffma2_rn(two(W), u2w, acc_b[q]);
+        }
+    }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kP2GThreads, 4) k_p2g(StepArgs a)
+{
+    extern __shared__ __align__(16) unsigned char p2g_smem[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int slots = a.p2g_slots, np = a.r.np;
+    float4* rec = reinterpret_cast<float4*>(p2g_smem + warp * p2g_warp_bytes(slots));
+    float4* raw = rec + slots * (kRecPitch / 4) + lane;
+    int* s_scene = reinterpret_cast<int*>(raw - lane + kRawPlanes * 32);
+    short* s_start = reinterpret_cast<short*>(s_scene + slots);
+    if (active_bricks(a.sb) == 0) return;  // the sort found its bookkeeping inconsistent
+    // planes that are read, and where they are staged: with the stored stress 0 and 3-7,
+    // else 0-6
+    const bool stored = MODE != kP2GConstraint && a.tau_valid;
+    const auto at = [&](int k) { return raw + 32 * (k > 0 && stored ? k - 2 : k); };
+    const auto copy_planes = [&](int p) {
+        if (p >= 0) {
+#pragma unroll
+            for (int k = 0; k < kPlanes; ++k)
+                if (stored ? (k == 0 || k == 3 || k > 5 || (MODE != kP2GStd && k > 3)) : k < 7)
+                    cp_async16(at(k), a.in.q + (size_t)k * a.cap + p);
+        }
+        cp_async_commit();
+    };
+    // batches of 32 slots, chunk by chunk: storage index of the lane's slot (the lanes
+    // beyond the chunk's last one repeat it), or -1 after the last chunk
+    const int step = gridDim.x * kP2GWarps * slots;
+    const auto source = [&](int base, int q0) {
+        if (q0 >= min(slots, np - base)) {
+            base += step;
+            q0 = 0;
+        }
+        return base < np ? a.sb.perm[a.r.p0 + min(base + min(q0 + lane, slots - 1), np - 1)] : -1;
+    };
+    int p = source((blockIdx.x * kP2GWarps + warp) * slots, 0);
+    copy_planes(p);
+    for (int base = (blockIdx.x * kP2GWarps + warp) * slots; base < np; base += step) {
+        const int cnt = min(slots, np - base);
+        // A
+        int runs = 0, last = -1;
+        for (int q0 = 0; q0 < cnt; q0 += 32) {
+            const int q = q0 + lane, s = a.r.p0 + base + min(q, cnt - 1);
+            const int scene = scene_of_slot(a, s);
+            const int p_next = source(base, q0 + 32);
+            int key = -1;
+            cp_async_wait<0>();
+            if (q < cnt) {
+                const unsigned ebits = p2g_record<MODE>(
+                    a, a.scenes[scene], p, [&](int k) { return *at(k); }, rec + q * (kRecPitch / 4), key);
+                s_scene[q] = scene;
+                if (ebits) atomicOr(&a.err[scene], ebits);
+            }
+            p = p_next;
+            copy_planes(p);
+            const int up = __shfl_up_sync(kFull, key, 1);
+            const bool head = q < cnt && key != (lane ? up : last);
+            const unsigned heads = __ballot_sync(kFull, head);
+            if (head) s_start[runs + __popc(heads & ((1u << lane) - 1u))] = (short)q;
+            runs += __popc(heads);
+            last = __shfl_sync(kFull, key, 31);
+        }
+        if (lane == 0) s_start[runs] = (short)cnt;
+        __syncwarp();
+        // B
+        for (int job0 = 0; job0 < 3 * runs; job0 += 32) {
+            const int job = job0 + lane, run = min(job / 3, runs - 1), i = job - (job / 3) * 3, beg = s_start[run];
+            const bool own = job < 3 * runs;
+            const int end = own ? s_start[run + 1] : beg;
+            float2 acc_a[9], acc_b[9];
+#pragma unroll
+            for (int q = 0; q < 9; ++q) acc_a[q] = acc_b[q] = make_float2(0.f, 0.f);
+            for (int q = beg; q < end; ++q) p2g_add<MODE>(rec + q * (kRecPitch / 4), i, acc_a, acc_b);
+            __syncwarp();
+            const int key = __float_as_int(rec[beg * (kRecPitch / 4) + 1].w);
+            const int ly = (key >> 2) & 3, lz = key & 3;
+            // C: three lanes on lies the next run; where its cell is the next one in z
+            // (of the brick), its nodes 0 and 1 are this run's 1 and 2
+            const int before = __shfl_up_sync(kFull, key, 3);
+            const bool joined = own && lane >= 3 && lz > 0 && before == key - 1;
+            const bool last = !(__shfl_down_sync(kFull, joined, 3) && lane < 29);
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const auto join = [&](float v0, float& v1, float v2) {
+                    const float c2 = __shfl_up_sync(kFull, v2, 3);
+                    if (joined) v1 += c2;
+                    const float c1 = __shfl_up_sync(kFull, v1, 3);
+                    return joined ? v0 + c1 : v0;
+                };
+                float2 *p = acc_a + 3 * j, *q = acc_b + 3 * j;
+                p[0].x = join(p[0].x, p[1].x, p[2].x);
+                p[0].y = join(p[0].y, p[1].y, p[2].y);
+                q[0].x = join(q[0].x, q[1].x, q[2].x);
+                q[0].y = join(q[0].y, q[1].y, q[2].y);
+            }
+            if (own) {
+                const SceneDev& sc = a.scenes[s_scene[beg]];
+                const int nb = sc.nb, lx = ((key >> 4) & 3) + i;
+                const float m = sc.m_p;
+                float4* g = a.G + (key + i * 16 + (lx > 3 ? (nb * nb - 1) * 64 : 0));
+#pragma unroll
+                for (int q = 0; q < 9; ++q)
+                    if (q % 3 == 0 || last)
+                        red_add_v4(g + ((q / 3) * 4 + q % 3 + (ly + q / 3 > 3 ? nb * 64 - 16 : 0) + (lz + q % 3 > 3 ? 60 : 0)),
+                                   acc_b[q].y * m, acc_a[q].x, acc_a[q].y, acc_b[q].x);
+            }
+        }
+        __syncwarp();  // the records are rewritten
+    }
+    cp_async_wait<0>();
 }
 
 // ----------------------------------------------------------- grid update
@@ -868,10 +949,11 @@ __device__ __forceinline__ void grid_node(const StepArgs& a, int B, int scene, i
         if (gk > hi) v.z = fminf(v.z, 0.f);
     }
     a.V[node] = make_float4(v.x, v.y, v.z, g.x);
+    a.sb.ccnt[node] = 0;
     if (nid == 0) {
         a.brick_epoch[B] = a.epoch[scene];
-        // the histogram of the next substep starts from zero (the scan has
-        // read it; every non-empty brick is an active node brick)
+        // the histograms of the next substep start from zero (the sort has
+        // read them; every non-empty brick is an active node brick)
         a.sb.cnt[B] = 0;
     }
     // impulse on each rigid: -(node momentum change), linear and angular
@@ -1050,7 +1132,9 @@ enum {
 // Velocity and affine matrix gathered at a position:
 //   v = sum W v_I,  B_rc = sum W v_I,r (o_c - f_c),  W = wx_i wy_j wz_k
 // (kG2PStdGrad: the basis gradient in cell units instead, B_rc = sum v_I,r dW/df_c),
-// contracted separably over k, then j, then i; x and y go in paired FMAs.
+// contracted separably over k, then j, then i; x and y go in paired FMAs.  The
+// velocities are taken relative to the middle node's, whose share is known (sum W = 1,
+// B = 0): a bulk motion then leaves no rounding in B.
 // node(i, j, k) returns (v, m) of the stencil's nodes.
 template <int FLAGS, class Node>
 __device__ __forceinline__ void gather_velocity(const float f[3], const float w[9], Node node, float v[3], float B[9])
@@ -1069,6 +1153,7 @@ __device__ __forceinline__ void gather_velocity(const float f[3], const float w[
         }
     }
     const auto two = [](float s) { return make_float2(s, s); };
+    const float4 mid = node(1, 1, 1);
     float2 vp = two(0.f), B0 = two(0.f), B1 = two(0.f), B2 = two(0.f);  // x, y rows
     float vz = 0.f, Bz0 = 0.f, Bz1 = 0.f, Bz2 = 0.f;                    // z row
 #pragma unroll
@@ -1087,11 +1172,12 @@ __device__ __forceinline__ void gather_velocity(const float f[3], const float w[
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const float4 g = node(i, j, k);
-                const float2 xy = make_float2(g.x, g.y);
+                const float2 xy = __fadd2_rn(make_float2(g.x, g.y), make_float2(-mid.x, -mid.y));
+                const float z = g.z - mid.z;
                 p = __ffma2_rn(two(wz[k]), xy, p);
                 d = __ffma2_rn(two(wzd[k]), xy, d);
-                zp = __fmaf_rn(wz[k], g.z, zp);
-                zd = __fmaf_rn(wzd[k], g.z, zd);
+                zp = __fmaf_rn(wz[k], z, zp);
+                zd = __fmaf_rn(wzd[k], z, zd);
             }
             A = __ffma2_rn(two(wy[j]), p, A);
             Ay = __ffma2_rn(two(wyd[j]), p, Ay);
@@ -1109,7 +1195,7 @@ __device__ __forceinline__ void gather_velocity(const float f[3], const float w[
         Bz1 = __fmaf_rn(wx, zAy, Bz1);
         Bz2 = __fmaf_rn(wx, zAz, Bz2);
     }
-    v[0] = vp.x; v[1] = vp.y; v[2] = vz;
+    v[0] = vp.x + mid.x; v[1] = vp.y + mid.y; v[2] = vz + mid.z;
     B[0] = B0.x; B[1] = B1.x; B[2] = B2.x;
     B[3] = B0.y; B[4] = B1.y; B[5] = B2.y;
     B[6] = Bz0; B[7] = Bz1; B[8] = Bz2;
@@ -1117,10 +1203,11 @@ __device__ __forceinline__ void gather_velocity(const float f[3], const float w[
 
 // G2P of a particle with position (and id) q0 from its stencil's velocities; the
 // new position before the push-out.  stencil(bc) returns the node functor of base
-// cell bc, old_F(F) reads the deformation gradient.
-template <int FLAGS, class Stencil, class OldF>
+// cell bc, old_F(F) reads the deformation gradient, early(x, C) takes the new
+// x and C before the constitutive update (C stored there leaves it eight registers more).
+template <int FLAGS, class Stencil, class OldF, class Early>
 __device__ __forceinline__ unsigned g2p_particle(const StepArgs& a, const SceneDev& sc, const float4 q0, float mu, float lam,
-                                                 Stencil stencil, OldF old_F, G2POut& o)
+                                                 Stencil stencil, OldF old_F, Early early, G2POut& o)
 {
     const int n = sc.n;
     const float fn = (float)n, dt = a.dt;
@@ -1150,20 +1237,30 @@ __device__ __forceinline__ unsigned g2p_particle(const StepArgs& a, const SceneD
             o.F[3 * r + c] = Fr + dt * (o.C[3 * r] * F0 + o.C[3 * r + 1] * F1 + o.C[3 * r + 2] * F2);
         }
     }
+    early(o.x, o.C);
+    float chk = q0.x + q0.y + q0.z + o.v[0] + o.v[1] + o.v[2];
     if (!(FLAGS & kG2PNoStress)) {
         ebits |= constitutive(a.model, a.plasticity, a.yield_stress, mu, lam, o.F, o.t6);
     } else {
 #pragma unroll
         for (int i = 0; i < 6; ++i) o.t6[i] = 0.f;
     }
-    float chk = q0.x + q0.y + q0.z + o.v[0] + o.v[1] + o.v[2];
 #pragma unroll
     for (int i = 0; i < 9; ++i) chk += o.F[i];
     if (!isfinite(chk)) ebits |= MPM_EBIT_NONFINITE;
     return ebits;
 }
 
-// All eight planes of slot s, and the material.
+// Planes 4 and 5 (C but its last component) of slot s.
+__device__ __forceinline__ void store_C(const StepArgs& a, int s, const float C[9])
+{
+    const size_t cap = a.cap;
+    float4* q = a.out.q + s;
+    q[4 * cap] = make_float4(C[0], C[1], C[2], C[3]);
+    q[5 * cap] = make_float4(C[4], C[5], C[6], C[7]);
+}
+
+// The other planes of slot s, and the material.
 __device__ __forceinline__ void store_particle(const StepArgs& a, int pp_mat, float mu, float lam, int s, const G2POut& o)
 {
     const size_t cap = a.cap;
@@ -1172,8 +1269,6 @@ __device__ __forceinline__ void store_particle(const StepArgs& a, int pp_mat, fl
     q[cap] = make_float4(o.F[0], o.F[1], o.F[2], o.F[3]);
     q[2 * cap] = make_float4(o.F[4], o.F[5], o.F[6], o.F[7]);
     q[3 * cap] = make_float4(o.F[8], o.v[0], o.v[1], o.v[2]);
-    q[4 * cap] = make_float4(o.C[0], o.C[1], o.C[2], o.C[3]);
-    q[5 * cap] = make_float4(o.C[4], o.C[5], o.C[6], o.C[7]);
     q[6 * cap] = make_float4(o.C[8], o.t6[0], o.t6[1], o.t6[2]);
     q[7 * cap] = make_float4(o.t6[3], o.t6[4], o.t6[5], 0.f);
     if (pp_mat) {
@@ -1190,25 +1285,6 @@ __device__ __forceinline__ void material_of(const StepArgs& a, const SceneDev& s
         mu = a.in.mu[p];
         lam = a.in.lam[p];
     }
-}
-
-// Scene of slot s (scenes own consecutive slots): two warp-wide probes of the
-// scenes' first slots for the warp's first slot, then the few lanes of later scenes
-// step on.  Every lane of the warp calls it.
-__device__ __forceinline__ int scene_of_slot(const StepArgs& a, int s)
-{
-    if (a.r.s1 - a.r.s0 == 1) return a.r.s0;
-    const int lane = threadIdx.x & 31, s_first = __shfl_sync(kFull, s, 0);
-    int lo = a.r.s0, len = a.r.s1 - a.r.s0;
-    while (len > 1) {  // p_begin never decreases: the last scene that starts at or before s_first
-        const int step = (len + 31) >> 5, at = lane * step;
-        const bool le = at < len && a.scenes[lo + at].p_begin <= s_first;
-        const int k = 31 - __clz(__ballot_sync(kFull, le) | 1u);
-        lo += k * step;
-        len = min(step, len - k * step);
-    }
-    while (lo + 1 < a.r.s1 && a.scenes[lo + 1].p_begin <= s) ++lo;
-    return lo;
 }
 
 // Copy the 6^3 window out of the 2x2x2 staged bricks into a linear array, so
@@ -1244,29 +1320,21 @@ struct GridStencil {
     }
 };
 
-__device__ __forceinline__ void cp_async16(float4* dst, const float4* src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 // Persistent CTAs, their warps taking chunks of 32 slots in turn (the chunks in
 // flight then cover one window of the arrays, and neighbouring warps the same nodes).
 // What bounds it is the chain permutation -> planes -> nodes -> rank of each
 // particle: planes 0-3 of a warp's next chunk are copied to shared memory while it
-// computes, and its slots of the permutation are read two chunks ahead.  Read through
+// computes, its slots of the permutation are read two chunks ahead, and the rank's
+// atomic is sent before the constitutive update.  Read through
 // L1, the stencils need no staging, no barriers and no brick: one CTA per brick with
 // its window copied to shared memory (46.1 M warp instructions at 62 % issue, the SMs
 // idle for a sixth of the launch behind its last bricks) took 70.8 us on a 1M block
 // and 18.8 us on a 64k one; this kernel 59.8 us and 9.5 us, the accumulator's reset
-// (1.8 us in a kernel of its own) included.  Budgets of 64 / 80 / 96 registers: 64.4 /
-// 63.9 / 66.6 us on the 1M block.
-// MINB = CTAs per SM the registers must allow: the larger budget (7 at 128
-// threads, 72 registers; 3 at 256, 80; 1 at 512) or 1024/BLOCK (64 registers,
+// (1.8 us in a kernel of its own) included.  Spills cost more than warps in flight bring:
+// a substep of the 1M block takes 126.6 us with 80 registers (32 B spilled), 146.4 with
+// 72 (144 B), 128.4 with 96.
+// MINB = CTAs per SM the registers must allow: the larger budget (6 at 128
+// threads, 3 at 256: 80 registers; 1 at 512: 128) or 1024/BLOCK (64 registers,
 // more warps in flight).  FLAGS & kG2PSolids: some scene of the launch has a
 // sphere or a box, so particles may need the push-out.
 template <int BLOCK, int MINB, int FLAGS>
@@ -1287,10 +1355,8 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_g2p(StepArgs a)
     int c = blockIdx.x * NW + warp;
     const int p_end = a.r.p0 + a.r.np;
     const size_t cap = a.cap;
-    const auto slot_source = [&](int ch) {
-        const int s = a.r.p0 + ch * 32 + lane;
-        return ch < c1 && s < p_end ? a.sb.perm[s] : -1;
-    };
+    // (the lanes beyond the last slot repeat it and store nothing)
+    const auto slot_source = [&](int ch) { return ch < c1 ? a.sb.perm[min(a.r.p0 + ch * 32 + lane, p_end - 1)] : -1; };
     const auto copy_planes = [&](int p) {
         if (p >= 0) {
 #pragma unroll
@@ -1303,28 +1369,36 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_g2p(StepArgs a)
     int posed = -1;
     for (; c < c1; c += step) {
         const int p_after = slot_source(c + 2 * step);
+        const bool valid = a.r.p0 + c * 32 + lane < p_end;
         const int s = min(a.r.p0 + c * 32 + lane, p_end - 1);
-        const bool valid = p >= 0;
         const int scene = scene_of_slot(a, s);
         const SceneDev& sc = a.scenes[scene];
         G2POut o;
-        unsigned ebits = 0;
-        float mu = 0.f, lam = 0.f;
-        if (valid) material_of(a, sc, p, mu, lam);
+        unsigned ood = 0;
+        CellRank rank;
+        float mu, lam;
+        material_of(a, sc, p, mu, lam);
         cp_async_wait<0>();
-        int key = 0;
-        if (valid)
-            ebits = g2p_particle<FLAGS>(
-                a, sc, s_q[0][tid], mu, lam, [&](const int* bc) { return GridStencil(a.V, sc, bc); },
-                [&](float* F) {
-                    const float4 u = s_q[1][tid], v = s_q[2][tid];
-                    F[0] = u.x; F[1] = u.y; F[2] = u.z; F[3] = u.w;
-                    F[4] = v.x; F[5] = v.y; F[6] = v.z; F[7] = v.w;
-                    F[8] = s_q[3][tid].x;
-                    copy_planes(p_next);
-                },
-                o);
-        else copy_planes(p_next);
+        // new key and the atomics of the rank, whose answer is not needed before the end
+        const auto sort_key = [&](const float* x) {
+            const int key = cell_key(sc, x[0], x[1], x[2], ood);
+            rank = cell_rank_begin(a.sb, sc, key, valid);
+            if (valid) a.sb.key[s] = key;
+        };
+        unsigned ebits = g2p_particle<FLAGS>(
+            a, sc, s_q[0][tid], mu, lam, [&](const int* bc) { return GridStencil(a.V, sc, bc); },
+            [&](float* F) {
+                const float4 u = s_q[1][tid], v = s_q[2][tid];
+                F[0] = u.x; F[1] = u.y; F[2] = u.z; F[3] = u.w;
+                F[4] = v.x; F[5] = v.y; F[6] = v.z; F[7] = v.w;
+                F[8] = s_q[3][tid].x;
+                copy_planes(p_next);
+            },
+            [&](const float* x, const float* C) {
+                if (valid) store_C(a, s, C);
+                if (!SOLIDS) sort_key(x);
+            },
+            o);
         __syncwarp();
         if (SOLIDS) {
             // push-out (Sec. IV-A), scene by scene of the chunk
@@ -1335,20 +1409,18 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_g2p(StepArgs a)
                 if (q != posed) stage_solids(a, q, s_pose[warp], lane);
                 posed = q;
                 __syncwarp();
-                if (valid && scene == q) push_out(s_pose[warp], nr, o.x);
+                if (scene == q) push_out(s_pose[warp], nr, o.x);
                 __syncwarp();
             }
+            sort_key(o.x);
         }
+        const int r = cell_rank_end(rank);
         if (valid) {
             store_particle(a, sc.pp_mat, mu, lam, s, o);
-            unsigned ood = 0;
-            key = cell_key(sc, o.x[0], o.x[1], o.x[2], ood);
-            a.sb.key[s] = key;
+            a.sb.rank[s] = r;
             if (ood && !(ebits & MPM_EBIT_NONFINITE)) ebits |= MPM_EBIT_OUT_OF_DOMAIN;
             if (ebits) atomicOr(&a.err[scene], ebits);
         }
-        const int rank = brick_rank(a.sb, sc, key, valid);
-        if (valid) a.sb.rank[s] = rank;
         p = p_next;
         p_next = p_after;
     }
@@ -1430,7 +1502,7 @@ __global__ void __launch_bounds__(kFusedThreads, 4) k_g2p2g(StepArgs a)
                         const float4* base = lin + (l0 * 36 + l1 * 6 + l2);
                         return [base](int i, int j, int kk) { return base[i * 36 + j * 6 + kk]; };
                     },
-                    [&](float* F) { load_F(a.in, a.cap, p, F); }, o);
+                    [&](float* F) { load_F(a.in, a.cap, p, F); }, [&](const float*, const float* C) { store_C(a, start + k, C); }, o);
                 if (n_solid) push_out(s_pose, n_solid, o.x);
                 store_particle(a, sc.pp_mat, mu, lam, start + k, o);
                 // P2G of the next substep at the new position
@@ -1478,7 +1550,7 @@ __global__ void __launch_bounds__(kFusedThreads, 4) k_g2p2g(StepArgs a)
                             }
                 }
             }
-            const int rank = brick_rank(a.sb, sc, key, valid);
+            const int rank = cell_rank_end(cell_rank_begin(a.sb, sc, key, valid));
             if (valid) {
                 a.sb.key[start + k] = key;
                 a.sb.rank[start + k] = rank;
@@ -1519,95 +1591,6 @@ __global__ void __launch_bounds__(kFusedThreads, 4) k_g2p2g(StepArgs a)
         buf ^= 1;
     }
     walker_exit(a);
-}
-
-// ------------------------------------------------------- standard MPM P2G
-//
-// P2G of the standard MPM (Sec. III-A): m_I += W m (Eq. 1), and the momentum
-// W m v plus the internal-force impulse -dt V0 tau grad W (Eq. 2, 3; V sigma =
-// V0 tau).  One CTA per active particle brick accumulates its 6^3 window with
-// shared-memory float atomics and adds it to HBM with one vector reduction per
-// node.  The paper keeps this solver as a reference with fewer features; so
-// does this kernel (no per-cell work items).
-
-constexpr int kStdThreads = 256;
-
-__global__ void __launch_bounds__(kStdThreads) k_p2g_std(StepArgs a)
-{
-    __shared__ float win[4][kWinNodes];
-    __shared__ int s_item;
-    const int tid = threadIdx.x;
-    const int n_act = active_bricks(a.sb);
-    const int cap = a.cap;
-    for (;;) {
-        if (tid == 0) s_item = atomicAdd(&a.sb.counters[CTR_WORK_P2G], 1);
-        for (int t = tid; t < 4 * kWinNodes; t += kStdThreads) (&win[0][0])[t] = 0.0f;
-        __syncthreads();
-        const int item = s_item;
-        if (item >= n_act) break;
-        const int e = active_entry(a.sb, item);
-        const int b = a.sb.act_brick[e], start = a.sb.act_start[e], count = a.sb.act_count[e];
-        const int scene = a.sb.act_scene[e];
-        const SceneDev sc = a.scenes[scene];
-        const int n = sc.n, nb = sc.nb, lb = b - sc.brick_base;
-        int ox, oy, oz;
-        brick_coords(nb, sc.nb_log2, lb, ox, oy, oz);
-        ox *= 4; oy *= 4; oz *= 4;
-        const float fn = (float)n, m = sc.m_p;
-        const float kap = a.dt * sc.V0 * fn;  // dt V0 times the n of grad W = n dW/df
-        unsigned ebits = 0;
-        for (int k = tid; k < count; k += kStdThreads) {
-            const int p = a.sb.perm[start + k];
-            int bc[3];
-            float f[3], w[9], dw[9], x[3];
-            load_x(a.in, p, x);
-            ebits |= particle_weights(x[0], x[1], x[2], n, bc, f, w);
-            bspline_d(f[0], dw);
-            bspline_d(f[1], dw + 3);
-            bspline_d(f[2], dw + 6);
-            float t6[6], v[3];
-            if (a.tau_valid) {
-                float C[9];
-                load_C_tau(a.in, cap, p, C, t6);
-            } else {
-                float F[9];
-                load_F(a.in, cap, p, F);
-                const float mu = sc.pp_mat ? a.in.mu[p] : sc.mu, lam = sc.pp_mat ? a.in.lam[p] : sc.lam;
-                ebits |= constitutive(a.model, 0, 0.f, mu, lam, F, t6);
-            }
-            load_v(a.in, cap, p, v);
-#pragma unroll
-            for (int q = 0; q < 3; ++q) v[q] *= m;
-            const float tau[9] = {t6[0], t6[1], t6[2], t6[1], t6[3], t6[4], t6[2], t6[4], t6[5]};
-            const int l0 = min(max(bc[0] - ox, 0), 3), l1 = min(max(bc[1] - oy, 0), 3), l2 = min(max(bc[2] - oz, 0), 3);
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-#pragma unroll
-                    for (int kk = 0; kk < 3; ++kk) {
-                        const float W = w[i] * w[3 + j] * w[6 + kk];
-                        const float g0 = dw[i] * w[3 + j] * w[6 + kk], g1 = w[i] * dw[3 + j] * w[6 + kk],
-                                    g2 = w[i] * w[3 + j] * dw[6 + kk];
-                        const int node = (l0 + i) * 36 + (l1 + j) * 6 + (l2 + kk);
-                        atomicAdd(&win[0][node], W * m);
-#pragma unroll
-                        for (int r = 0; r < 3; ++r)
-                            atomicAdd(&win[1 + r][node],
-                                      W * v[r] - kap * (tau[3 * r] * g0 + tau[3 * r + 1] * g1 + tau[3 * r + 2] * g2));
-                    }
-        }
-        __syncthreads();
-        for (int q = tid; q < kWinNodes; q += kStdThreads) {
-            const float mm = win[0][q];
-            if (mm == 0.0f) continue;
-            const int gi = ox + q / 36, gj = oy + (q / 6) % 6, gk = oz + q % 6;
-            if (gi >= n || gj >= n || gk >= n) continue;
-            red_add_v4(&a.G[node_index(sc, gi, gj, gk)], mm, win[1][q], win[2][q], win[3][q]);
-        }
-        if (ebits) atomicOr(&a.err[scene], ebits);
-        __syncthreads();
-    }
 }
 
 // ---------------------------------------------------- PB-MPM cycle G2P
@@ -1803,42 +1786,22 @@ cudaError_t launch_sort(const StepArgs& a, cudaStream_t s, bool write_perm)
     return cudaGetLastError();
 }
 
-template <int PER>
-static constexpr size_t p2g_dyn_smem() { return sizeof(float) * kItemRecFields * P2GShape<PER>::slots; }
-
 cudaError_t prepare_p2g()
 {
-    cudaError_t e = cudaFuncSetAttribute(k_p2g<2, kP2GStress>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)p2g_dyn_smem<2>());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_p2g<3, kP2GStress>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)p2g_dyn_smem<3>());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_p2g<4, kP2GStress>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)p2g_dyn_smem<4>());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_p2g<4, kP2GConstraint>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)p2g_dyn_smem<4>());
+    const int most = kP2GWarps * p2g_warp_bytes(kP2GMaxSlots);
+    cudaError_t e = cudaFuncSetAttribute(k_p2g<kP2GStress>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_p2g<kP2GConstraint>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_p2g<kP2GStd>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     return e;
 }
 
 cudaError_t launch_p2g(const StepArgs& a, cudaStream_t s)
 {
-    if (a.solver == MPM_SOLVER_PB) {
-        k_p2g<4, kP2GConstraint><<<a.p2g_ctas, kP2GThreads, p2g_dyn_smem<4>(), s>>>(a);
-        return cudaGetLastError();
-    }
-    switch (a.p2g_chunk) {
-    case 2 * kP2GThreads: k_p2g<2, kP2GStress><<<a.p2g_ctas, kP2GThreads, p2g_dyn_smem<2>(), s>>>(a); break;
-    case 4 * kP2GThreads: k_p2g<4, kP2GStress><<<a.p2g_ctas, kP2GThreads, p2g_dyn_smem<4>(), s>>>(a); break;
-    default: k_p2g<3, kP2GStress><<<a.p2g_ctas, kP2GThreads, p2g_dyn_smem<3>(), s>>>(a); break;
-    }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_p2g_std(const StepArgs& a, cudaStream_t s)
-{
-    k_p2g_std<<<a.p2g_ctas, kStdThreads, 0, s>>>(a);
+    const int c = min(a.p2g_ctas, n_blocks(max(a.r.np, 1), kP2GWarps * a.p2g_slots));
+    const size_t smem = kP2GWarps * p2g_warp_bytes(a.p2g_slots);
+    if (a.solver == MPM_SOLVER_PB) k_p2g<kP2GConstraint><<<c, kP2GThreads, smem, s>>>(a);
+    else if (a.solver == MPM_SOLVER_STANDARD) k_p2g<kP2GStd><<<c, kP2GThreads, smem, s>>>(a);
+    else k_p2g<kP2GStress><<<c, kP2GThreads, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -1847,13 +1810,6 @@ cudaError_t launch_g2p_vc(const StepArgs& a, cudaStream_t s)
     if (a.r.np == 0) return cudaSuccess;
     k_g2p_vc<<<n_blocks(a.r.np, kVcThreads), kVcThreads, 0, s>>>(a);
     return cudaGetLastError();
-}
-
-int occupancy_p2g_std()
-{
-    int b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_p2g_std, kStdThreads, 0);
-    return b;
 }
 
 cudaError_t launch_grid(const StepArgs& a, cudaStream_t s, bool clear)
@@ -1877,7 +1833,7 @@ static void launch_g2p_variant(const StepArgs& a, cudaStream_t s)
         }
     } else {
         switch (a.g2p_threads) {
-        case 128: k_g2p<128, 7, FLAGS><<<c, 128, 0, s>>>(a); break;
+        case 128: k_g2p<128, 6, FLAGS><<<c, 128, 0, s>>>(a); break;
         case 512: k_g2p<512, 1, FLAGS><<<c, 512, 0, s>>>(a); break;
         default: k_g2p<256, 3, FLAGS><<<c, 256, 0, s>>>(a); break;
         }
@@ -1885,18 +1841,18 @@ static void launch_g2p_variant(const StepArgs& a, cudaStream_t s)
 }
 
 // The standard-MPM and PB-MPM variants exist in one launch shape only (128
-// threads, 64 registers): the MLS-MPM shapes are what the tuner explores.
+// threads, 80 registers): the MLS-MPM shapes are what the tuner explores.
 cudaError_t launch_g2p(const StepArgs& a, cudaStream_t s)
 {
     const int c = min(a.g2p_ctas, n_blocks(max(a.r.np, 1), 128));
     // the push-out variant only where a scene has a solid shape: blades, needles and
     // segments push nothing out
     if (a.solver == MPM_SOLVER_STANDARD) {
-        if (a.any_solid) k_g2p<128, 8, kG2PStdGrad | kG2PSolids><<<c, 128, 0, s>>>(a);
-        else k_g2p<128, 8, kG2PStdGrad><<<c, 128, 0, s>>>(a);
+        if (a.any_solid) k_g2p<128, 6, kG2PStdGrad | kG2PSolids><<<c, 128, 0, s>>>(a);
+        else k_g2p<128, 6, kG2PStdGrad><<<c, 128, 0, s>>>(a);
     } else if (a.solver == MPM_SOLVER_PB) {
-        if (a.any_solid) k_g2p<128, 8, kG2PNoStress | kG2PSolids><<<c, 128, 0, s>>>(a);
-        else k_g2p<128, 8, kG2PNoStress><<<c, 128, 0, s>>>(a);
+        if (a.any_solid) k_g2p<128, 6, kG2PNoStress | kG2PSolids><<<c, 128, 0, s>>>(a);
+        else k_g2p<128, 6, kG2PNoStress><<<c, 128, 0, s>>>(a);
     } else if (a.any_solid) {
         launch_g2p_variant<kG2PSolids>(a, s);
     } else {
@@ -1978,15 +1934,10 @@ cudaError_t launch_read_grid(const float4* V, const int* brick_epoch, const int*
     return cudaGetLastError();
 }
 
-int occupancy_p2g(int chunk)
+int occupancy_p2g(int slots)
 {
     int b = 0;
-    if (chunk == 2 * kP2GThreads)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_p2g<2, kP2GStress>, kP2GThreads, p2g_dyn_smem<2>());
-    else if (chunk == 4 * kP2GThreads)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_p2g<4, kP2GStress>, kP2GThreads, p2g_dyn_smem<4>());
-    else
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_p2g<3, kP2GStress>, kP2GThreads, p2g_dyn_smem<3>());
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_p2g<kP2GStress>, kP2GThreads, kP2GWarps * p2g_warp_bytes(slots));
     return b;
 }
 
@@ -2000,7 +1951,7 @@ int occupancy_g2p(int threads, int regs64)
         else if (threads == 512) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<512, 2, kG2PSolids>, 512, 0);
         else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<256, 4, kG2PSolids>, 256, 0);
     } else {
-        if (threads == 128) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<128, 7, kG2PSolids>, 128, 0);
+        if (threads == 128) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<128, 6, kG2PSolids>, 128, 0);
         else if (threads == 512) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<512, 1, kG2PSolids>, 512, 0);
         else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<256, 3, kG2PSolids>, 256, 0);
     }

@@ -14,10 +14,10 @@ struct Range {
 
 struct SortBufs {
     int* key;       // [cap] brick x 64 + base cell of each stored particle (next substep)
-    int* rank;      // [cap] rank of the particle within its brick
+    int* rank;      // [cap] rank of the particle within its cell
     int* perm;      // [cap] sorted slot -> storage index
-    unsigned char* scell; // [cap] sorted slot -> base cell inside its brick (the key's low 6 bits)
     int* cnt;       // [bricks] particles per brick (next substep)
+    int* ccnt;      // [bricks * 64] particles per cell (next substep)
     int* off;       // [bricks] first slot of each active brick
     int* act_brick; // [list_size] active particle bricks: those of at least kBigBrick particles from
                     // the front, the others from the back (active_entry)
@@ -56,18 +56,19 @@ struct StepArgs {
     int p2g_ctas, grid_ctas;     // CTAs of the persistent P2G and grid kernels
     int grid_plain_ctas;         // CTAs of the grid kernel of launches without rigids
     int fused_ctas;              // CTAs of the fused G2P + P2G kernel
-    int p2g_chunk, g2p_threads, g2p_regs64;
+    int p2g_slots;               // slots that a P2G warp stages at once
+    int g2p_threads, g2p_regs64;
     int tau_valid;               // P2G reads the stored stress (else recomputes it from F)
     int any_rigid;               // some scene of the range has a rigid (contact in the grid update)
     int rigid_ext;               // some scene of the range has an arc or a mesh slicer
     int any_solid;               // some scene of the range has a sphere or a box (particle push-out)
-    int cell_order;              // P2G rewrites each pass's permutation slots in cell order
     int solver;                  // MPM_SOLVER_*
     float pb_beta;               // PB-MPM constraint blend
 };
 
 constexpr int kStateFloats = 34;  // eight float4 planes, mu, lam
-constexpr int kP2GThreads = 192;  // 64 cells x 3 node slices
+constexpr int kP2GThreads = 192;  // six warps, each with slots of its own
+constexpr int kP2GMaxSlots = 64;
 constexpr int kScanThreads = 256;
 constexpr int kMinTileShift = 8;  // a scan tile holds at least kScanThreads bricks
 constexpr int kScatterPer = 4;  // particles per thread of the counting-sort scatter
@@ -84,9 +85,7 @@ cudaError_t prepare_p2g();  // shared-memory opt-in of the P2G variants (once pe
 // clear: reset the P2G accumulator afterwards (G2P does it otherwise)
 cudaError_t launch_grid(const StepArgs& a, cudaStream_t s, bool clear);
 cudaError_t launch_g2p(const StepArgs& a, cudaStream_t s);
-cudaError_t launch_p2g_std(const StepArgs& a, cudaStream_t s);  // standard MPM P2G
 cudaError_t launch_g2p_vc(const StepArgs& a, cudaStream_t s);   // PB-MPM cycle G2P (v, C in place)
-int occupancy_p2g_std();
 cudaError_t launch_g2p2g(const StepArgs& a, cudaStream_t s);
 int occupancy_g2p2g();
 int occupancy_grid();
@@ -113,7 +112,7 @@ cudaError_t launch_fields_host(const PState& st, int cap, int p0, int np, const 
                                bool to_host, cudaStream_t s);
 cudaError_t launch_read_grid(const float4* V, const int* brick_epoch, const int* epoch, const SceneDev* scenes,
                              int scene, int n, int brick_base, float* dst, cudaStream_t s);
-int occupancy_p2g(int chunk);
+int occupancy_p2g(int slots);
 int occupancy_g2p(int threads, int regs64);
 
 }  // namespace mpm
