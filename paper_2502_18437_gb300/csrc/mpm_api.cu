@@ -32,7 +32,10 @@ int status_from_cuda(cudaError_t e)
 static int timeout_ms(const mpm_ctx* c) { return c->cfg.timeout_ms > 0 ? c->cfg.timeout_ms : 10000; }
 
 // Wait for all work enqueued on the context's stream, polling an event with a
-// bound instead of blocking inside the driver.
+// bound instead of blocking inside the driver; after kSpinUs with pauses (each takes
+// some 70 us, as long as a small scene's whole readback).
+constexpr int kSpinUs = 20000;
+
 int wait_stream(mpm_ctx* c)
 {
     MPM_CK(cudaEventRecord(c->ev, c->stream));
@@ -41,9 +44,10 @@ int wait_stream(mpm_ctx* c)
         cudaError_t e = cudaEventQuery(c->ev);
         if (e == cudaSuccess) return MPM_OK;
         if (e != cudaErrorNotReady) return status_from_cuda(e);
-        const auto ms = std::chrono::duration_cast<std::chrono::milliseconds>(std::chrono::steady_clock::now() - t0).count();
-        if (ms > timeout_ms(c)) return MPM_ERR_TIMEOUT;
-        std::this_thread::sleep_for(std::chrono::microseconds(20));
+        const auto us = std::chrono::duration_cast<std::chrono::microseconds>(std::chrono::steady_clock::now() - t0).count();
+        if (us / 1000 > timeout_ms(c)) return MPM_ERR_TIMEOUT;
+        if (us < kSpinUs) std::this_thread::yield();
+        else std::this_thread::sleep_for(std::chrono::microseconds(20));
     }
 }
 
@@ -327,12 +331,8 @@ static void free_ctx(mpm_ctx* c)
     cudaStreamSynchronize(c->stream);
     mpm_tape_free(c);
     clear_graphs(c);
-    for (int i = 0; i < 2; ++i) cudaFree(c->state_mem[i]);
-    void* bufs[] = {c->sb.key, c->sb.rank, c->sb.perm, c->sb.cnt, c->sb.ccnt, c->sb.off, c->sb.act_brick, c->sb.act_start,
-                    c->sb.act_count, c->sb.act_scene, c->sb.nact_brick, c->sb.nact_scene, c->sb.counters,
-                    c->sb.tile_n, c->G, c->V, c->brick_epoch,
-                    c->d_scenes, c->d_rigids, c->d_impulse, c->d_err, c->d_time, c->d_epoch, c->d_stage};
-    for (void* p : bufs) cudaFree(p);
+    cudaFree(c->arena);
+    cudaFree(c->d_stage);
     if (c->h_pinned) cudaFreeHost(c->h_pinned);
     if (c->ev) cudaEventDestroy(c->ev);
     for (cudaEvent_t e : c->phase_events) cudaEventDestroy(e);
@@ -420,15 +420,25 @@ extern "C" int mpm_create(const mpm_config* cfg, void* stream, mpm_ctx** out)
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device);
     if (e == cudaSuccess) e = prepare_p2g();
     const size_t nbk = (size_t)c->total_bricks;
-    auto alloc = [&](void** p, size_t bytes) {
-        if (e == cudaSuccess) e = cudaMalloc(p, bytes ? bytes : 16);
-    };
+    // one allocation for all buffers; those that start from zero come first
+    struct Part { void** p; size_t bytes; };
+    std::vector<Part> parts;
+    auto alloc = [&](void** p, size_t bytes) { parts.push_back({p, (bytes + 255) & ~(size_t)255}); };
+    alloc((void**)&c->sb.cnt, sizeof(int) * nbk);
+    alloc((void**)&c->sb.ccnt, sizeof(int) * nbk * 64);
+    alloc((void**)&c->sb.counters, sizeof(int) * CTR_COUNT);
+    alloc((void**)&c->sb.tile_n, sizeof(int) * c->total_tiles);
+    alloc((void**)&c->G, sizeof(float4) * nbk * 64);
+    alloc((void**)&c->V, sizeof(float4) * nbk * 64);
+    alloc((void**)&c->d_impulse, sizeof(double) * c->n_scenes * kMaxRigids * 6);
+    alloc((void**)&c->d_err, sizeof(unsigned) * c->n_scenes);
+    alloc((void**)&c->d_time, sizeof(double) * c->n_scenes);
+    alloc((void**)&c->d_epoch, sizeof(int) * c->n_scenes);
+    const size_t n_zero = parts.size();
     for (int i = 0; i < 2; ++i) alloc((void**)&c->state_mem[i], state_bytes(c->cap));
     alloc((void**)&c->sb.key, sizeof(int) * c->cap);
     alloc((void**)&c->sb.rank, sizeof(int) * c->cap);
     alloc((void**)&c->sb.perm, sizeof(int) * c->cap);
-    alloc((void**)&c->sb.cnt, sizeof(int) * nbk);
-    alloc((void**)&c->sb.ccnt, sizeof(int) * nbk * 64);
     alloc((void**)&c->sb.off, sizeof(int) * nbk);
     alloc((void**)&c->sb.act_brick, sizeof(int) * nbk);
     alloc((void**)&c->sb.act_start, sizeof(int) * nbk);
@@ -436,32 +446,29 @@ extern "C" int mpm_create(const mpm_config* cfg, void* stream, mpm_ctx** out)
     alloc((void**)&c->sb.act_scene, sizeof(int) * nbk);
     alloc((void**)&c->sb.nact_brick, sizeof(int) * nbk);
     alloc((void**)&c->sb.nact_scene, sizeof(int) * nbk);
-    alloc((void**)&c->sb.counters, sizeof(int) * CTR_COUNT);
-    alloc((void**)&c->sb.tile_n, sizeof(int) * c->total_tiles);
     c->sb.list_size = c->total_bricks;
-    alloc((void**)&c->G, sizeof(float4) * nbk * 64);
-    alloc((void**)&c->V, sizeof(float4) * nbk * 64);
     alloc((void**)&c->brick_epoch, sizeof(int) * nbk);
     alloc((void**)&c->d_scenes, sizeof(SceneDev) * c->n_scenes);
     alloc((void**)&c->d_rigids, sizeof(RigidDev) * c->n_scenes * kMaxRigids);
-    alloc((void**)&c->d_impulse, sizeof(double) * c->n_scenes * kMaxRigids * 6);
-    alloc((void**)&c->d_err, sizeof(unsigned) * c->n_scenes);
-    alloc((void**)&c->d_time, sizeof(double) * c->n_scenes);
-    alloc((void**)&c->d_epoch, sizeof(int) * c->n_scenes);
+    alloc((void**)&c->d_inv, sizeof(int) * c->cap);
+    size_t zero = 0, total = 0;
+    for (size_t i = 0; i < parts.size(); ++i) {
+        total += parts[i].bytes;
+        if (i < n_zero) zero += parts[i].bytes;
+    }
+    if (e == cudaSuccess) e = cudaMalloc(&c->arena, total);
+    if (e == cudaSuccess) {
+        char* at = static_cast<char*>(c->arena);
+        for (const Part& q : parts) {
+            *q.p = at;
+            at += q.bytes;
+        }
+    }
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->ev, cudaEventDisableTiming);
     if (e == cudaSuccess) {
         for (int i = 0; i < 2; ++i) c->st[i] = state_view(c->state_mem[i], c->cap);
-        cudaMemsetAsync(c->sb.cnt, 0, sizeof(int) * nbk, c->stream);
-        cudaMemsetAsync(c->sb.ccnt, 0, sizeof(int) * nbk * 64, c->stream);
-        cudaMemsetAsync(c->sb.counters, 0, sizeof(int) * CTR_COUNT, c->stream);
-        cudaMemsetAsync(c->sb.tile_n, 0, sizeof(int) * c->total_tiles, c->stream);
-        cudaMemsetAsync(c->G, 0, sizeof(float4) * nbk * 64, c->stream);
-        cudaMemsetAsync(c->V, 0, sizeof(float4) * nbk * 64, c->stream);
+        cudaMemsetAsync(c->arena, 0, zero, c->stream);
         cudaMemsetAsync(c->brick_epoch, 0xff, sizeof(int) * nbk, c->stream);
-        cudaMemsetAsync(c->d_impulse, 0, sizeof(double) * c->n_scenes * kMaxRigids * 6, c->stream);
-        cudaMemsetAsync(c->d_err, 0, sizeof(unsigned) * c->n_scenes, c->stream);
-        cudaMemsetAsync(c->d_time, 0, sizeof(double) * c->n_scenes, c->stream);
-        cudaMemsetAsync(c->d_epoch, 0, sizeof(int) * c->n_scenes, c->stream);
         e = cudaMemcpyAsync(c->d_rigids, c->h_rigids.data(), sizeof(RigidDev) * c->h_rigids.size(),
                             cudaMemcpyHostToDevice, c->stream);
     }
@@ -707,11 +714,12 @@ extern "C" int mpm_set_rigid(mpm_ctx* c, int scene, int rigid_id, const mpm_rigi
         c->scenes_dirty = true;
         clear_graphs(c);  // captured substeps carry whether any scene has a rigid
     }
-    MPM_CK(cudaMemcpyAsync(c->d_rigids + slot, &c->h_rigids[slot], sizeof(RigidDev), cudaMemcpyHostToDevice, c->stream));
-    int st = upload_scenes(c);
-    if (st) return st;
-    // h_rigids[slot] is the copy source; make sure it is consumed before it can change
-    return wait_stream(c);
+    // the description travels in the launch's arguments: nothing to wait for
+    cudaStreamCaptureStatus capturing;
+    MPM_CK(cudaStreamIsCapturing(c->stream, &capturing));
+    if (capturing != cudaStreamCaptureStatusNone) return MPM_ERR_CUDA;  // poses belong to a moment, not to a graph
+    MPM_CK(launch_set_rigid(d, c->d_rigids + slot, c->stream));
+    return upload_scenes(c);
 }
 
 static uint32_t float_bits(float f)
@@ -826,67 +834,61 @@ extern "C" int mpm_read_state(mpm_ctx* c, int scene, uint32_t fields, void* cons
         }
     int st;
     const PState cur = c->st[c->cur];
-    if (mem == MPM_MEM_HOST && !(fields & ~15u) && np > 0) {
-        // pinned host arrays: one kernel writes them in id order over the host link
-        HostFields h{};
-        bool mapped = true;
-        for (int f = 0, k = 0; f < 4; ++f)
-            if (fields & (1u << f)) {
-                h.f[f] = static_cast<float*>(mapped_host(dst[k++]));
-                mapped = mapped && h.f[f];
-            }
-        if (mapped) {
-            if ((st = ensure_stage(c, sizeof(int) * (size_t)np))) return st;
-            if ((st = ensure_pinned(c, 64))) return st;
-            int* inv = static_cast<int*>(c->d_stage);
-            MPM_CK(launch_id_inverse(cur, sc.p_begin, np, inv, c->stream));
-            MPM_CK(launch_fields_host(cur, c->cap, sc.p_begin, np, inv, h, true, c->stream));
-            MPM_CK(cudaMemcpyAsync(c->h_pinned, c->d_err + scene, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
-            if ((st = wait_stream(c))) return st;
-            return error_status(*static_cast<unsigned*>(c->h_pinned));
+    // device staging for host reads that are not pinned; pinned host arrays of x, v, C and F
+    // are written by the kernel itself
+    bool mapped = mem == MPM_MEM_HOST && !(fields & ~15u);
+    void* at[6] = {};  // where the kernels write each field
+    for (int f = 0, k = 0; f < 6; ++f)
+        if (fields & (1u << f)) {
+            at[f] = mapped ? mapped_host(dst[k]) : dst[k];
+            mapped = mapped && at[f];
+            ++k;
         }
-    }
-    // device staging for host reads that are not pinned
-    size_t stage_need = 0, pin_need = 64;
+    const bool staged = mem == MPM_MEM_HOST && !mapped;
+    size_t bytes[6] = {}, stage_need = 0, pin_need = 64;
     for (int f = 0, k = 0; f < 6; ++f) {
         if (!(fields & (1u << f))) continue;
-        const size_t bytes = f == 5 ? sizeof(double) * kMaxRigids * 6 : sizeof(float) * kFieldComps[f] * (size_t)np;
-        if (mem == MPM_MEM_HOST) {
-            stage_need += align256(bytes);
-            if (!is_pinned_host(dst[k])) pin_need += align256(bytes);
+        bytes[f] = f == 5 ? sizeof(double) * kMaxRigids * 6 : sizeof(float) * kFieldComps[f] * (size_t)np;
+        if (staged) {
+            stage_need += align256(bytes[f]);
+            if (!is_pinned_host(dst[k])) pin_need += align256(bytes[f]);
         }
         ++k;
     }
     if ((st = ensure_stage(c, stage_need))) return st;
     if ((st = ensure_pinned(c, pin_need))) return st;
-    size_t soff = 0, poff = 64;
+    if (staged) {
+        size_t off = 0;
+        for (int f = 0; f < 6; ++f)
+            if (fields & (1u << f)) {
+                at[f] = static_cast<char*>(c->d_stage) + off;
+                off += align256(bytes[f]);
+            }
+    }
+    if (fields & 15u) {
+        Fields h{};
+        for (int f = 0; f < 4; ++f) h.f[f] = static_cast<float*>(at[f]);
+        MPM_CK(launch_fields(cur, c->st[c->cur ^ 1], c->cap, sc.p_begin, np, c->d_inv, h, true, mapped, c->stream));
+    }
+    if (fields & MPM_FIELD_ORDER) MPM_CK(launch_order(cur, sc.p_begin, np, static_cast<int*>(at[4]), c->stream));
+    if (fields & MPM_FIELD_IMPULSE) {
+        double* imp = c->d_impulse + (size_t)scene * kMaxRigids * 6;
+        MPM_CK(cudaMemcpyAsync(at[5], imp, bytes[5], cudaMemcpyDeviceToDevice, c->stream));
+        MPM_CK(cudaMemsetAsync(imp, 0, bytes[5], c->stream));
+    }
+    size_t poff = 64;
     struct Pending { void* dst; size_t poff, bytes; };
     std::vector<Pending> pend;
-    for (int f = 0, k = 0; f < 6; ++f) {
+    for (int f = 0, k = 0; staged && f < 6; ++f) {
         if (!(fields & (1u << f))) continue;
         void* out = dst[k++];
-        const size_t bytes = f == 5 ? sizeof(double) * kMaxRigids * 6 : sizeof(float) * kFieldComps[f] * (size_t)np;
-        void* dev_out = out;
-        if (mem == MPM_MEM_HOST) {
-            dev_out = static_cast<char*>(c->d_stage) + soff;
-            soff += align256(bytes);
-        }
-        if (f == 5) {
-            MPM_CK(cudaMemcpyAsync(dev_out, c->d_impulse + (size_t)scene * kMaxRigids * 6, bytes,
-                                   cudaMemcpyDeviceToDevice, c->stream));
-            MPM_CK(cudaMemsetAsync(c->d_impulse + (size_t)scene * kMaxRigids * 6, 0, bytes, c->stream));
+        if (!bytes[f]) continue;
+        if (is_pinned_host(out)) {
+            MPM_CK(cudaMemcpyAsync(out, at[f], bytes[f], cudaMemcpyDeviceToHost, c->stream));
         } else {
-            MPM_CK(launch_gather_field(cur, c->cap, sc.p_begin, np, f, dev_out, c->stream));
-        }
-        if (mem == MPM_MEM_HOST && bytes) {
-            if (is_pinned_host(out)) {
-                MPM_CK(cudaMemcpyAsync(out, dev_out, bytes, cudaMemcpyDeviceToHost, c->stream));
-            } else {
-                MPM_CK(cudaMemcpyAsync(static_cast<char*>(c->h_pinned) + poff, dev_out, bytes, cudaMemcpyDeviceToHost,
-                                       c->stream));
-                pend.push_back({out, poff, bytes});
-                poff += align256(bytes);
-            }
+            MPM_CK(cudaMemcpyAsync(static_cast<char*>(c->h_pinned) + poff, at[f], bytes[f], cudaMemcpyDeviceToHost, c->stream));
+            pend.push_back({out, poff, bytes[f]});
+            poff += align256(bytes[f]);
         }
     }
     MPM_CK(cudaMemcpyAsync(c->h_pinned, c->d_err + scene, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
@@ -910,35 +912,27 @@ extern "C" int mpm_write_state(mpm_ctx* c, int scene, uint32_t fields, const voi
         }
     int st = MPM_OK;
     const PState cur = c->st[c->cur];
-    if (mem == MPM_MEM_HOST && np > 0) {
-        // pinned host arrays: one kernel reads them in id order over the host link
-        HostFields h{};
-        bool mapped = true;
-        for (int f = 0, k = 0; f < 4; ++f)
-            if (fields & (1u << f)) {
-                h.f[f] = static_cast<float*>(mapped_host(src[k++]));
-                mapped = mapped && h.f[f];
-            }
-        if (mapped) {
-            if ((st = ensure_stage(c, sizeof(int) * (size_t)np))) return st;
-            int* inv = static_cast<int*>(c->d_stage);
-            MPM_CK(launch_id_inverse(cur, sc.p_begin, np, inv, c->stream));
-            MPM_CK(launch_fields_host(cur, c->cap, sc.p_begin, np, inv, h, false, c->stream));
-            if (fields & MPM_FIELD_X) c->keys_valid = false;
-            invalidate_pending(c);
-            return wait_stream(c);
+    Fields h{};
+    bool mapped = mem == MPM_MEM_HOST;  // pinned host arrays are read by the kernel itself
+    for (int f = 0, k = 0; f < 4; ++f)
+        if (fields & (1u << f)) {
+            h.f[f] = static_cast<float*>(mapped ? mapped_host(src[k]) : const_cast<void*>(src[k]));
+            mapped = mapped && h.f[f];
+            ++k;
+        }
+    if (mem == MPM_MEM_HOST && !mapped) {
+        if ((st = ensure_stage(c, need))) return st;
+        size_t off = 0;
+        for (int f = 0, k = 0; f < 4; ++f) {
+            if (!(fields & (1u << f))) continue;
+            const size_t bytes = sizeof(float) * kFieldComps[f] * (size_t)np;
+            const void* d = nullptr;
+            if ((st = stage_input(c, src[k++], bytes, mem, off, &d))) return st;
+            off += align256(bytes);
+            h.f[f] = static_cast<float*>(const_cast<void*>(d));
         }
     }
-    if (mem == MPM_MEM_HOST && (st = ensure_stage(c, need))) return st;
-    size_t off = 0;
-    for (int f = 0, k = 0; f < 4; ++f) {
-        if (!(fields & (1u << f))) continue;
-        const size_t bytes = sizeof(float) * kFieldComps[f] * (size_t)np;
-        const void* d = nullptr;
-        if ((st = stage_input(c, src[k++], bytes, mem, off, &d))) return st;
-        off += align256(bytes);
-        MPM_CK(launch_scatter_field(cur, c->cap, sc.p_begin, np, f, static_cast<const float*>(d), c->stream));
-    }
+    MPM_CK(launch_fields(cur, c->st[c->cur ^ 1], c->cap, sc.p_begin, np, c->d_inv, h, false, mapped, c->stream));
     // new positions need new brick keys; any new field changes the pending P2G
     if (fields & MPM_FIELD_X) c->keys_valid = false;
     invalidate_pending(c);

@@ -24,7 +24,8 @@ struct mpm_ctx {
     std::vector<int> rigid_type;          // per slot, MPM_RIGID_NONE when unset
     double h_time = 0.0;                  // scene time (all scenes advance together)
 
-    // device memory
+    // device memory: buffers of the arena, and the staging area, which grows
+    void* arena = nullptr;
     float* state_mem[2] = {nullptr, nullptr};
     mpm::PState st[2]{};
     int cur = 0;
@@ -40,6 +41,7 @@ struct mpm_ctx {
     unsigned* d_err = nullptr;
     double* d_time = nullptr;
     int* d_epoch = nullptr;
+    int* d_inv = nullptr;  // [cap] id -> slot, scratch of the state I/O
     void* d_stage = nullptr;
     size_t stage_bytes = 0;
     void* h_pinned = nullptr;

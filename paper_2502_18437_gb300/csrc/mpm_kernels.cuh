@@ -92,24 +92,25 @@ int occupancy_grid();
 int occupancy_grid_plain();
 
 // state I/O helpers
-cudaError_t launch_gather_field(const PState& st, int cap, int p0, int np, int field, void* dst,
-                                cudaStream_t s);
 cudaError_t launch_init_particles(const PState& st, int cap, int p_at, int n, int id0, const float* x,
                                   const float* v, const float* E, const float* nu, float E0, float nu0,
                                   cudaStream_t s);
 cudaError_t launch_permute_to_id(const PState& src, const PState& dst, int cap, int p0, int np,
                                  cudaStream_t s);
-cudaError_t launch_scatter_field(const PState& st, int cap, int p0, int np, int field, const float* src,
-                                 cudaStream_t s);
-// x, v, C, F (null: not moved) of one scene as host-mapped arrays in particle-id order
-struct HostFields {
+// x, v, C, F (null: not moved) of one scene as arrays in particle-id order
+struct Fields {
     float* f[4];
 };
-// inv[id] = slot of the scene's particle with that id (np entries)
-cudaError_t launch_id_inverse(const PState& st, int p0, int np, int* inv, cudaStream_t s);
-// state fields <-> host-mapped arrays in one pass (to_host: state -> host)
-cudaError_t launch_fields_host(const PState& st, int cap, int p0, int np, const int* inv, const HostFields& h,
-                               bool to_host, cudaStream_t s);
+// From this many particles the state is read by id, through records; below, by slot, in one
+// kernel.  Measured, by id and by slot: 35 and 33 us at 64k, 36 and 45 at 131k, 49 and 57 at
+// 262k, 133 and 219 at 1M, 485 and 1,306 at 4M.
+constexpr int kIoByIdFrom = 1 << 17;
+// state -> arrays (out) or arrays -> state; inv: scratch of np ints, spare: the state's other
+// buffer (scratch); host: the arrays are pinned host memory
+cudaError_t launch_fields(const PState& st, const PState& spare, int cap, int p0, int np, int* inv, const Fields& h, bool out,
+                          bool host, cudaStream_t s);
+cudaError_t launch_order(const PState& st, int p0, int np, int* dst, cudaStream_t s);  // ids by slot
+cudaError_t launch_set_rigid(const RigidDev& d, RigidDev* dst, cudaStream_t s);
 cudaError_t launch_read_grid(const float4* V, const int* brick_epoch, const int* epoch, const SceneDev* scenes,
                              int scene, int n, int brick_base, float* dst, cudaStream_t s);
 int occupancy_p2g(int slots);
