@@ -702,6 +702,23 @@ extern "C" int mpm_set_rigid(mpm_ctx* c, int scene, int rigid_id, const mpm_rigi
         d.spine_radius = r->spine_radius;
         d.t_set = c->h_time;
         for (int k = 0; k < 3 * d.n_pts; ++k) d.shape.pts[k] = (&r->points[0][0])[k];
+        // (widened by far more than the distances' rounding, relative to the shape and its reach;
+        // without end where a point is not finite)
+        const float reach = std::max(r->type == MPM_SEGMENTS ? r->radius : std::max(0.5f * r->thickness, r->spine_radius), 0.f) +
+                            std::max(r->margin, 0.f);
+        for (int i = 0; i < 3 && d.n_pts > 0; ++i) {
+            float lo = d.shape.pts[i], hi = lo, big = std::fabs(lo), sum = lo;
+            for (int k = 1; k < d.n_pts; ++k) {
+                lo = std::min(lo, d.shape.pts[3 * k + i]);
+                hi = std::max(hi, d.shape.pts[3 * k + i]);
+                sum += d.shape.pts[3 * k + i];
+                big = std::max(big, std::fabs(d.shape.pts[3 * k + i]));
+            }
+            const float wide = std::isfinite(sum) ? reach + 1e-5f * (reach + big) + 1e-30f : INFINITY;
+            if (!std::isfinite(sum)) lo = hi = 0.f;
+            d.lo[i] = lo - wide;
+            d.hi[i] = hi + wide;
+        }
     }
     c->h_rigids[slot] = d;
     if (c->rigid_type[slot] != d.type) clear_graphs(c);  // captured launches carry the kinds of rigids

@@ -74,6 +74,9 @@ struct RigidDev {
     float mu_k, c_d, margin, radius;
     float half[3];
     float thickness, spine_radius;
+    // body-frame box outside which the shape touches no node (segments and mesh slicers:
+    // their points and their reach)
+    float lo[3], hi[3];
     double t_set;    // scene time at which (c0, q0) was the pose
     RigidShape shape;
 };
@@ -85,6 +88,7 @@ struct RigidCur {
     float mu_k, c_d, margin, radius;
     float half[3];
     float thickness, spine_radius;
+    float lo[3], hi[3];
     RigidShape shape;
 };
 
