@@ -439,7 +439,6 @@ extern "C" int mpm_create(const mpm_config* cfg, void* stream, mpm_ctx** out)
     alloc((void**)&c->sb.key, sizeof(int) * c->cap);
     alloc((void**)&c->sb.rank, sizeof(int) * c->cap);
     alloc((void**)&c->sb.perm, sizeof(int) * c->cap);
-    alloc((void**)&c->sb.off, sizeof(int) * nbk);
     alloc((void**)&c->sb.act_brick, sizeof(int) * nbk);
     alloc((void**)&c->sb.act_start, sizeof(int) * nbk);
     alloc((void**)&c->sb.act_count, sizeof(int) * nbk);

@@ -63,7 +63,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(StepArgs a)
 {
     __shared__ int s_warp[kScanThreads / 32];
     __shared__ int s_sum[3][kScanThreads / 32];
-    __shared__ int s_base[3];
+    __shared__ int s_base[3], s_total[3];
+    __shared__ int s_brick[kScanThreads], s_start[kScanThreads];  // the chunk's particle bricks
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const SortBufs& sb = a.sb;
     const int tile = a.r.t0 + blockIdx.x;
@@ -157,6 +158,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(StepArgs a)
                 t += k;
             }
             s_base[tid] = t ? atomicAdd(&sb.counters[CTR_N_BIG + tid], t) : 0;
+            s_total[tid] = t;
         }
         __syncthreads();
         if (c > 0) {
@@ -164,7 +166,9 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(StepArgs a)
                               ? s_base[0] + s_sum[0][warp] + __popc(big & lt)
                               : sb.list_size - 1 - (s_base[1] + s_sum[1][warp] + __popc(small & lt));
             const int start = start0 + before;
-            sb.off[b] = start;
+            const int at = s_sum[0][warp] + s_sum[1][warp] + __popc((big | small) & lt);
+            s_brick[at] = b;
+            s_start[at] = start;
             sb.act_brick[e] = b;
             sb.act_start[e] = start;
             sb.act_count[e] = c;
@@ -176,7 +180,23 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(StepArgs a)
             sb.nact_scene[e] = s;
         }
         start0 += total;
-        __syncthreads();  // s_sum and s_base are rewritten by the next chunk
+        __syncthreads();
+        // a warp per brick: its cells' counts become their first slots
+        const int n_act = s_total[0] + s_total[1];
+#pragma unroll 4
+        for (int i = warp; i < n_act; i += kScanThreads / 32) {
+            int2* cells = reinterpret_cast<int2*>(sb.ccnt + (size_t)s_brick[i] * 64) + lane;
+            const int2 k = *cells;
+            int incl = k.x + k.y;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const int t = __shfl_up_sync(kFull, incl, d);
+                if (lane >= d) incl += t;
+            }
+            const int even = s_start[i] + incl - k.x - k.y;
+            *cells = make_int2(even, even + k.x);
+        }
+        __syncthreads();  // the shared lists are rewritten by the next chunk
     }
 }
 
@@ -192,19 +212,16 @@ __global__ void k_reset_histogram(SortBufs sb, int bricks, int tiles)
     if (i >= CTR_N_BIG && i <= CTR_N_NACT) sb.counters[i] = 0;
 }
 
-// Counting-sort scatter: slot = first slot of the brick + particles in the brick's
-// cells before the particle's + its rank in the cell.  The cells' prefix sums are
-// taken by the warp, brick by brick of its particles (nearly always one: the
-// particles were sorted a substep ago).  Also clears the range's tile counts for the
-// next substep (the scan has read them).  write_perm = 0 only clears (the adjoint
-// reuses a recorded permutation).
+// Counting-sort scatter: a particle's slot is its cell's first slot plus its rank.  Also
+// clears the range's tile counts for the next substep (the scan has read them).
 // Each thread takes kScatterPer particles, 256 apart, with their loads issued
 // together (a 1M-particle range in one wave of CTAs).
+// (The cells' first slots come from the scan, a warp a brick: 1M particles 5.4 us.  Taken
+// here, by each warp for its particles' bricks, 10.5 us, and 89 us for particles in no order.)
 __global__ void __launch_bounds__(256) k_scatter(StepArgs a, int write_perm)
 {
-    const int g0 = blockIdx.x * (256 * kScatterPer) + threadIdx.x, lane = threadIdx.x & 31;
-    int key[kScatterPer], rank[kScatterPer], first[kScatterPer], start[kScatterPer];
-    int2 cells[kScatterPer];
+    const int g0 = blockIdx.x * (256 * kScatterPer) + threadIdx.x;
+    int key[kScatterPer], rank[kScatterPer], dst[kScatterPer];
 #pragma unroll
     for (int u = 0; u < kScatterPer; ++u) {
         const int g = g0 + u * 256;
@@ -215,43 +232,16 @@ __global__ void __launch_bounds__(256) k_scatter(StepArgs a, int write_perm)
             rank[u] = a.sb.rank[a.r.p0 + g];
         }
     }
-    const auto in_range = [&](int brick) { return brick >= a.r.bb0 && brick < a.r.bb0 + a.r.nbr; };
-    const auto load_cells = [&](int brick) {
-        return in_range(brick) ? reinterpret_cast<const int2*>(a.sb.ccnt + (size_t)brick * 64)[lane] : make_int2(0, 0);
-    };
 #pragma unroll
     for (int u = 0; u < kScatterPer; ++u) {
-        // the brick of the warp's first particle
-        first[u] = __shfl_sync(kFull, key[u] >> 6, 0);
-        cells[u] = load_cells(first[u]);
-        start[u] = in_range(first[u]) ? a.sb.off[first[u]] : 0;
+        const int brick = key[u] >> 6;
+        dst[u] = (key[u] >= 0 && brick >= a.r.bb0 && brick < a.r.bb0 + a.r.nbr) ? a.sb.ccnt[key[u]] + rank[u] : -1;
     }
 #pragma unroll
     for (int u = 0; u < kScatterPer; ++u) {
-        const int g = g0 + u * 256, brick = key[u] >> 6, cell = key[u] & 63;
-        unsigned todo = __ballot_sync(kFull, key[u] >= 0);
-        int dst = -1, b = first[u];
-        int2 c = cells[u];
-        int st = start[u];
-        while (todo) {
-            int incl = c.x + c.y;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const int t = __shfl_up_sync(kFull, incl, d);
-                if (lane >= d) incl += t;
-            }
-            const int before = __shfl_sync(kFull, incl - c.y, cell >> 1), even = __shfl_sync(kFull, c.x, cell >> 1);
-            const bool mine = key[u] >= 0 && brick == b;
-            if (mine && in_range(b)) dst = st + before - (cell & 1 ? 0 : even) + rank[u];
-            todo &= ~__ballot_sync(kFull, mine);
-            if (todo) {
-                b = __shfl_sync(kFull, brick, __ffs(todo) - 1);
-                c = load_cells(b);
-                st = in_range(b) ? a.sb.off[b] : 0;
-            }
-        }
+        const int g = g0 + u * 256;
         if (write_perm && g < a.r.np) {
-            if (dst >= a.r.p0 && dst < a.r.p0 + a.r.np) a.sb.perm[dst] = a.r.p0 + g;
+            if (dst[u] >= a.r.p0 && dst[u] < a.r.p0 + a.r.np) a.sb.perm[dst[u]] = a.r.p0 + g;
             else atomicOr(&a.err[a.r.s0], MPM_EBIT_INTERNAL);
         }
         if (g < a.r.nt) a.sb.tile_n[a.r.t0 + g] = 0;

@@ -17,8 +17,8 @@ struct SortBufs {
     int* rank;      // [cap] rank of the particle within its cell
     int* perm;      // [cap] sorted slot -> storage index
     int* cnt;       // [bricks] particles per brick (next substep)
-    int* ccnt;      // [bricks * 64] particles per cell (next substep)
-    int* off;       // [bricks] first slot of each active brick
+    int* ccnt;      // [bricks * 64] particles per cell (next substep); the scan turns an active
+                    // brick's into the cells' first slots
     int* act_brick; // [list_size] active particle bricks: those of at least kBigBrick particles from
                     // the front, the others from the back (active_entry)
     int* act_start;
