@@ -19,6 +19,16 @@
 
 namespace mpm {
 
+// Small launches of the substep chain are made programmatic: a kernel's CTAs come up
+// while the one before it still runs, and wait here for its end and its writes (every
+// thread, before its first access); the next kernel may come up at once.  Elsewhere both
+// do nothing.
+__device__ __forceinline__ void chain_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ----------------------------------------------------------------- scan
 //
 // A scan tile is 2^tile_shift consecutive bricks of one scene (tiles never
@@ -61,6 +71,7 @@ __device__ __forceinline__ void block_scan(int v, int* s_warp, int& excl, int& t
 
 __global__ void __launch_bounds__(kScanThreads) k_scan(StepArgs a)
 {
+    chain_wait();
     __shared__ int s_warp[kScanThreads / 32];
     __shared__ int s_sum[3][kScanThreads / 32];
     __shared__ int s_base[3], s_total[3];
@@ -220,6 +231,7 @@ __global__ void k_reset_histogram(SortBufs sb, int bricks, int tiles)
 // here, by each warp for its particles' bricks, 10.5 us, and 89 us for particles in no order.)
 __global__ void __launch_bounds__(256) k_scatter(StepArgs a, int write_perm)
 {
+    chain_wait();
     const int g0 = blockIdx.x * (256 * kScatterPer) + threadIdx.x;
     int key[kScatterPer], rank[kScatterPer], dst[kScatterPer];
 #pragma unroll
@@ -503,6 +515,7 @@ __device__ __forceinline__ void p2g_add(const float4* rec, int i, float2 acc_a[9
 template <int MODE>
 __global__ void __launch_bounds__(kP2GThreads, 4) k_p2g(StepArgs a)
 {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char p2g_smem[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int slots = a.p2g_slots, np = a.r.np;
@@ -994,6 +1007,7 @@ __device__ __forceinline__ void grid_node(const StepArgs& a, int B, int scene, i
 // the node bricks of a 1M-particle block are taken in one round.
 __global__ void __launch_bounds__(kGridThreads, 8) k_grid_plain(StepArgs a)
 {
+    chain_wait();
     const int tid = threadIdx.x, lane = tid & 31, grp = tid >> 6, nid = tid & 63;
     const int n_nact = a.sb.counters[CTR_N_NACT];
     for (int base = blockIdx.x * 4; base < n_nact; base += gridDim.x * 4) {
@@ -1011,6 +1025,7 @@ __global__ void __launch_bounds__(kGridThreads, 8) k_grid_plain(StepArgs a)
 // batched scenes with their blades.
 __global__ void __launch_bounds__(kGridThreads, 8) k_grid_clear(StepArgs a)
 {
+    chain_wait();
     const int grp = threadIdx.x >> 6, nid = threadIdx.x & 63;
     const int n_nact = a.sb.counters[CTR_N_NACT];
     for (int base = blockIdx.x * 4; base < n_nact; base += gridDim.x * 4) {
@@ -1025,6 +1040,7 @@ __global__ void __launch_bounds__(kGridThreads, 8) k_grid_clear(StepArgs a)
 template <bool EXT>
 __global__ void __launch_bounds__(kGridThreads, 4) k_grid(StepArgs a)
 {
+    chain_wait();
     __shared__ RigidCur rig[kMaxRigids];
     __shared__ float simp[kMaxRigids * 6];
     // per brick of a chunk of the list: node brick, scene, the scene's rigid count
@@ -1347,6 +1363,7 @@ struct GridStencil {
 template <int BLOCK, int MINB, int FLAGS>
 __global__ void __launch_bounds__(BLOCK, MINB) k_g2p(StepArgs a)
 {
+    chain_wait();
     constexpr bool SOLIDS = (FLAGS & kG2PSolids) != 0;
     constexpr int NW = BLOCK / 32;
     __shared__ float4 s_q[4][BLOCK];  // planes 0-3 of each thread's next particle
@@ -1612,6 +1629,7 @@ constexpr int kVcThreads = 128;
 
 __global__ void __launch_bounds__(kVcThreads) k_g2p_vc(StepArgs a)
 {
+    chain_wait();
     const int g = blockIdx.x * kVcThreads + threadIdx.x;
     const int n_clear = a.sb.counters[CTR_N_NACT] * 64;
     for (int t = g; t < n_clear; t += gridDim.x * kVcThreads)
@@ -1854,6 +1872,22 @@ __global__ void k_read_grid(const float4* V, const int* brick_epoch, const int* 
 
 static int n_blocks(long long n, int t) { return (int)((n + t - 1) / t); }
 
+template <class... P, class... A>
+static void launch_chain(const StepArgs& a, void (*k)(P...), int ctas, int threads, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute programmatic;
+    programmatic.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    programmatic.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &programmatic;
+    cfg.numAttrs = a.r.np < kChainBelow ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 cudaError_t launch_prepare(const StepArgs& a, const PState& st, cudaStream_t s)
 {
     if (a.r.np == 0) return cudaSuccess;
@@ -1869,11 +1903,11 @@ cudaError_t launch_reset_histogram(const SortBufs& sb, int bricks, int tiles, cu
 
 cudaError_t launch_sort(const StepArgs& a, cudaStream_t s, bool write_perm)
 {
-    k_scan<<<a.r.nt, kScanThreads, 0, s>>>(a);
+    launch_chain(a, k_scan, a.r.nt, kScanThreads, 0, s, a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int work = a.r.np > a.r.nt ? a.r.np : a.r.nt;
-    k_scatter<<<n_blocks(work, 256 * kScatterPer), 256, 0, s>>>(a, write_perm ? 1 : 0);
+    launch_chain(a, k_scatter, n_blocks(work, 256 * kScatterPer), 256, 0, s, a, write_perm ? 1 : 0);
     return cudaGetLastError();
 }
 
@@ -1890,25 +1924,25 @@ cudaError_t launch_p2g(const StepArgs& a, cudaStream_t s)
 {
     const int c = min(a.p2g_ctas, n_blocks(max(a.r.np, 1), kP2GWarps * a.p2g_slots));
     const size_t smem = kP2GWarps * p2g_warp_bytes(a.p2g_slots);
-    if (a.solver == MPM_SOLVER_PB) k_p2g<kP2GConstraint><<<c, kP2GThreads, smem, s>>>(a);
-    else if (a.solver == MPM_SOLVER_STANDARD) k_p2g<kP2GStd><<<c, kP2GThreads, smem, s>>>(a);
-    else k_p2g<kP2GStress><<<c, kP2GThreads, smem, s>>>(a);
+    if (a.solver == MPM_SOLVER_PB) launch_chain(a, k_p2g<kP2GConstraint>, c, kP2GThreads, smem, s, a);
+    else if (a.solver == MPM_SOLVER_STANDARD) launch_chain(a, k_p2g<kP2GStd>, c, kP2GThreads, smem, s, a);
+    else launch_chain(a, k_p2g<kP2GStress>, c, kP2GThreads, smem, s, a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_g2p_vc(const StepArgs& a, cudaStream_t s)
 {
     if (a.r.np == 0) return cudaSuccess;
-    k_g2p_vc<<<n_blocks(a.r.np, kVcThreads), kVcThreads, 0, s>>>(a);
+    launch_chain(a, k_g2p_vc, n_blocks(a.r.np, kVcThreads), kVcThreads, 0, s, a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_grid(const StepArgs& a, cudaStream_t s, bool clear)
 {
-    if (!a.any_rigid) k_grid_plain<<<a.grid_plain_ctas, kGridThreads, 0, s>>>(a);
-    else if (a.rigid_ext) k_grid<true><<<a.grid_ctas, kGridThreads, 0, s>>>(a);
-    else k_grid<false><<<a.grid_ctas, kGridThreads, 0, s>>>(a);
-    if (clear) k_grid_clear<<<a.grid_plain_ctas, kGridThreads, 0, s>>>(a);
+    if (!a.any_rigid) launch_chain(a, k_grid_plain, a.grid_plain_ctas, kGridThreads, 0, s, a);
+    else if (a.rigid_ext) launch_chain(a, k_grid<true>, a.grid_ctas, kGridThreads, 0, s, a);
+    else launch_chain(a, k_grid<false>, a.grid_ctas, kGridThreads, 0, s, a);
+    if (clear) launch_chain(a, k_grid_clear, a.grid_plain_ctas, kGridThreads, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -1918,15 +1952,15 @@ static void launch_g2p_variant(const StepArgs& a, cudaStream_t s)
     const int c = min(a.g2p_ctas, n_blocks(max(a.r.np, 1), a.g2p_threads));
     if (a.g2p_regs64) {
         switch (a.g2p_threads) {
-        case 128: k_g2p<128, 8, FLAGS><<<c, 128, 0, s>>>(a); break;
-        case 512: k_g2p<512, 2, FLAGS><<<c, 512, 0, s>>>(a); break;
-        default: k_g2p<256, 4, FLAGS><<<c, 256, 0, s>>>(a); break;
+        case 128: launch_chain(a, k_g2p<128, 8, FLAGS>, c, 128, 0, s, a); break;
+        case 512: launch_chain(a, k_g2p<512, 2, FLAGS>, c, 512, 0, s, a); break;
+        default: launch_chain(a, k_g2p<256, 4, FLAGS>, c, 256, 0, s, a); break;
         }
     } else {
         switch (a.g2p_threads) {
-        case 128: k_g2p<128, 6, FLAGS><<<c, 128, 0, s>>>(a); break;
-        case 512: k_g2p<512, 1, FLAGS><<<c, 512, 0, s>>>(a); break;
-        default: k_g2p<256, 3, FLAGS><<<c, 256, 0, s>>>(a); break;
+        case 128: launch_chain(a, k_g2p<128, 6, FLAGS>, c, 128, 0, s, a); break;
+        case 512: launch_chain(a, k_g2p<512, 1, FLAGS>, c, 512, 0, s, a); break;
+        default: launch_chain(a, k_g2p<256, 3, FLAGS>, c, 256, 0, s, a); break;
         }
     }
 }
@@ -1939,11 +1973,11 @@ cudaError_t launch_g2p(const StepArgs& a, cudaStream_t s)
     // the push-out variant only where a scene has a solid shape: blades, needles and
     // segments push nothing out
     if (a.solver == MPM_SOLVER_STANDARD) {
-        if (a.any_solid) k_g2p<128, 6, kG2PStdGrad | kG2PSolids><<<c, 128, 0, s>>>(a);
-        else k_g2p<128, 6, kG2PStdGrad><<<c, 128, 0, s>>>(a);
+        if (a.any_solid) launch_chain(a, k_g2p<128, 6, kG2PStdGrad | kG2PSolids>, c, 128, 0, s, a);
+        else launch_chain(a, k_g2p<128, 6, kG2PStdGrad>, c, 128, 0, s, a);
     } else if (a.solver == MPM_SOLVER_PB) {
-        if (a.any_solid) k_g2p<128, 6, kG2PNoStress | kG2PSolids><<<c, 128, 0, s>>>(a);
-        else k_g2p<128, 6, kG2PNoStress><<<c, 128, 0, s>>>(a);
+        if (a.any_solid) launch_chain(a, k_g2p<128, 6, kG2PNoStress | kG2PSolids>, c, 128, 0, s, a);
+        else launch_chain(a, k_g2p<128, 6, kG2PNoStress>, c, 128, 0, s, a);
     } else if (a.any_solid) {
         launch_g2p_variant<kG2PSolids>(a, s);
     } else {

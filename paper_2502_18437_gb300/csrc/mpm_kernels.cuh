@@ -71,6 +71,10 @@ constexpr int kP2GThreads = 192;  // six warps, each with slots of its own
 constexpr int kP2GMaxSlots = 64;
 constexpr int kScanThreads = 256;
 constexpr int kMinTileShift = 8;  // a scan tile holds at least kScanThreads bricks
+// Launches of fewer particles are made programmatic (launch_chain).  A substep with and
+// without: 19.6 and 21.0 us at 4k particles, 22.2 and 23.8 at 16k; 26.4 and 25.1 at 64k, 134
+// and 128 at 1M, where CTAs that wait take the place of CTAs that work.
+constexpr int kChainBelow = 1 << 15;
 constexpr int kScatterPer = 4;  // particles per thread of the counting-sort scatter
 // Particle bricks of at least this many particles come first in the active list,
 // so the persistent transfer kernels end on small bricks (a shorter tail)
