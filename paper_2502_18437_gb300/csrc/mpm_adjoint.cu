@@ -52,7 +52,7 @@ struct mpm_tape {
 
 namespace mpm {
 
-constexpr int kAdjThreads = 256;
+constexpr int kAdjThreads = 128;
 
 struct AdjState {
     float* x;
@@ -235,137 +235,125 @@ __global__ void k_adj_seed(StepArgs a, PState st, SeedIn in, AdjState nxt)
 
 // --------------------------------------------------------------- G2P^-1
 
+// xb = grad of sum_I W_I s_I with s_I = c_I + u_I . (q + A o): the derivative of the
+// weights (contracted separably) times s, o the node offset, per cell unit.
+template <class Node, class Value>
+__device__ __forceinline__ void weight_gradient(const float f[3], const float w[9], Node node, Value value, float xb[3])
+{
+    float dw[9];
+    bspline_d(f[0], dw);
+    bspline_d(f[1], dw + 3);
+    bspline_d(f[2], dw + 6);
+    xb[0] = xb[1] = xb[2] = 0.f;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        float a = 0.f, ay = 0.f, az = 0.f;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            float b = 0.f, bz = 0.f;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float v = value(node(i, j, k), i, j, k);
+                b += w[6 + k] * v;
+                bz += dw[6 + k] * v;
+            }
+            a += w[3 + j] * b;
+            ay += dw[3 + j] * b;
+            az += w[3 + j] * bz;
+        }
+        xb[0] += dw[i] * a;
+        xb[1] += w[i] * ay;
+        xb[2] += w[i] * az;
+    }
+}
+
+constexpr int kAdjWarps = kAdjThreads / 32;
+
+// One lane per slot gathers what its particle takes from the nodes and leaves a record of
+// what it gives to them; the warp then adds the records' contributions up as P2G does.
+// (One CTA per brick with shared-memory atomics, 81 per particle: 67 us for 32k particles.)
 __global__ void __launch_bounds__(kAdjThreads) k_g2p_adj(AdjArgs q)
 {
     const StepArgs& a = q.a;
-    __shared__ __align__(128) float4 vw[2][8 * 64];
-    __shared__ float gw[3][kWinNodes];
-    __shared__ __align__(8) unsigned long long bar[2];
-    __shared__ int s_item[2];
-    const int tid = threadIdx.x;
+    __shared__ float4 s_rec[kAdjWarps][32 * (kRecPitch / 4)];
+    __shared__ int s_scene[kAdjWarps][32];
+    __shared__ short s_start[kAdjWarps][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const size_t cap = a.cap;
-    const int n_act = active_bricks(a.sb);
-    int* work = &a.sb.counters[CTR_WORK_G2P];
-    walker_init<kAdjThreads>(a, n_act, vw, bar, s_item, work);
-    unsigned phase[2] = {0u, 0u};
-    int buf = 0;
-    for (;;) {
-        const int item = s_item[buf];
-        if (item >= n_act) break;
-        for (int t = tid; t < 3 * kWinNodes; t += kAdjThreads) (&gw[0][0])[t] = 0.f;
-        if (!walker_next(a, n_act, vw, bar, s_item, work, buf, phase, item)) return;
-        const int e = active_entry(a.sb, item);
-        const int start = a.sb.act_start[e], count = a.sb.act_count[e];
-        const SceneDev sc = a.scenes[a.sb.act_scene[e]];
-        const int n = sc.n, nb = sc.nb, lb = a.sb.act_brick[e] - sc.brick_base;
-        int ox, oy, oz;
-        brick_coords(nb, sc.nb_log2, lb, ox, oy, oz);
-        ox *= 4; oy *= 4; oz *= 4;
-        const float fn = (float)n, dt = a.dt, c4 = 4.f * fn;
-        const float4* win = vw[buf];
-        for (int k = tid; k < count; k += kAdjThreads) {
-            const int s = start + k;
-            const int p = a.sb.perm[s];
-            int bc[3];
-            float f[3], w[9], dw[9], x[3];
-            load_x(a.in, p, x);
-            particle_weights(x[0], x[1], x[2], n, bc, f, w);
-            bspline_d(f[0], dw);
-            bspline_d(f[1], dw + 3);
-            bspline_d(f[2], dw + 6);
-            const int l0 = min(max(bc[0] - ox, 0), 3), l1 = min(max(bc[1] - oy, 0), 3), l2 = min(max(bc[2] - oz, 0), 3);
-            // forward recompute of C'
-            float B[9];
+    const int g = blockIdx.x * kAdjThreads + threadIdx.x;
+    if (active_bricks(a.sb) == 0 || g - lane >= a.r.np) return;
+    const bool valid = g < a.r.np;
+    const int s = a.r.p0 + min(g, a.r.np - 1);
+    const int scene = scene_of_slot(a, s);
+    const SceneDev& sc = a.scenes[scene];
+    const int n = sc.n, nb = sc.nb;
+    const float fn = (float)n, dt = a.dt, c4 = 4.f * fn;
+    const int p = a.sb.perm[s];
+    int bc[3], key = -1;
+    float f[3], w[9], x[3];
+    load_x(a.in, p, x);
+    particle_weights(x[0], x[1], x[2], n, bc, f, w);
+    const GridStencil node(a.V, sc, bc);
+    // forward recompute of v' and C'
+    float vn[3], Cn[9], A[9], qv[3];
+    gather_velocity<0>(f, w, node, vn, Cn);
+    {
+        float F[9], aF[9];
+        load_F(a.in, cap, p, F);
 #pragma unroll
-            for (int i = 0; i < 9; ++i) B[i] = 0.f;
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-#pragma unroll
-                    for (int k2 = 0; k2 < 3; ++k2) {
-                        const int wi = l0 + i, wj = l1 + j, wk = l2 + k2;
-                        const float4 g = win[(((wi >> 2) << 2) | ((wj >> 2) << 1) | (wk >> 2)) * 64 + (wi & 3) * 16 + (wj & 3) * 4 + (wk & 3)];
-                        const float W = w[i] * w[3 + j] * w[6 + k2];
-                        const float d[3] = {(float)i - f[0], (float)j - f[1], (float)k2 - f[2]};
-#pragma unroll
-                        for (int c = 0; c < 3; ++c) {
-                            B[c] += W * g.x * d[c];
-                            B[3 + c] += W * g.y * d[c];
-                            B[6 + c] += W * g.z * d[c];
-                        }
-                    }
-            float Cn[9], F[9], aF[9], aC[9];
-            load_F(a.in, cap, p, F);
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                Cn[i] = c4 * B[i];
-                aF[i] = q.nxt.F[i * cap + s];
-                aC[i] = q.nxt.C[i * cap + s];
-            }
-            float ax[3], vt[3];
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                ax[d] = q.nxt.x[d * cap + s];
-                vt[d] = q.nxt.v[d * cap + s] + dt * ax[d];
-            }
-            // F_bar = (I + dt C')^T F'_bar;  Ct = C'_bar + dt F'_bar F^T
-            float Fb[9], Ct[9];
-#pragma unroll
-            for (int r = 0; r < 3; ++r)
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    Fb[3 * r + c] = aF[3 * r + c] + dt * (Cn[r] * aF[c] + Cn[3 + r] * aF[3 + c] + Cn[6 + r] * aF[6 + c]);
-                    Ct[3 * r + c] = aC[3 * r + c] + dt * (aF[3 * r] * F[3 * c] + aF[3 * r + 1] * F[3 * c + 1] + aF[3 * r + 2] * F[3 * c + 2]);
-                }
-            float xb[3] = {ax[0], ax[1], ax[2]};
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-#pragma unroll
-                    for (int k2 = 0; k2 < 3; ++k2) {
-                        const int wi = l0 + i, wj = l1 + j, wk = l2 + k2;
-                        const float4 g = win[(((wi >> 2) << 2) | ((wj >> 2) << 1) | (wk >> 2)) * 64 + (wi & 3) * 16 + (wj & 3) * 4 + (wk & 3)];
-                        const float vI[3] = {g.x, g.y, g.z};
-                        const float W = w[i] * w[3 + j] * w[6 + k2];
-                        const float gW[3] = {fn * dw[i] * w[3 + j] * w[6 + k2], fn * w[i] * dw[3 + j] * w[6 + k2],
-                                             fn * w[i] * w[3 + j] * dw[6 + k2]};
-                        const float d[3] = {(float)i - f[0], (float)j - f[1], (float)k2 - f[2]};
-                        float Ctd[3], h[3];
-#pragma unroll
-                        for (int r = 0; r < 3; ++r) Ctd[r] = Ct[3 * r] * d[0] + Ct[3 * r + 1] * d[1] + Ct[3 * r + 2] * d[2];
-#pragma unroll
-                        for (int c = 0; c < 3; ++c) h[c] = Ct[c] * vI[0] + Ct[3 + c] * vI[1] + Ct[6 + c] * vI[2];
-                        const int node = (wi * 6 + wj) * 6 + wk;
-#pragma unroll
-                        for (int r = 0; r < 3; ++r) atomicAdd(&gw[r][node], W * (vt[r] + c4 * Ctd[r]));
-                        const float s1 = vI[0] * (vt[0] + c4 * Ctd[0]) + vI[1] * (vt[1] + c4 * Ctd[1]) + vI[2] * (vt[2] + c4 * Ctd[2]);
-#pragma unroll
-                        for (int c = 0; c < 3; ++c) xb[c] += gW[c] * s1 - c4 * fn * W * h[c];
-                    }
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                q.cur.x[d * cap + p] = xb[d];
-                q.cur.v[d * cap + p] = 0.f;
-            }
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                q.cur.F[i * cap + p] = Fb[i];
-                q.cur.C[i * cap + p] = 0.f;
-            }
+        for (int i = 0; i < 9; ++i) {
+            Cn[i] *= c4;
+            aF[i] = q.nxt.F[i * cap + s];
         }
-        __syncthreads();
-        for (int t = tid; t < kWinNodes; t += kAdjThreads) {
-            const float g0 = gw[0][t], g1 = gw[1][t], g2 = gw[2][t];
-            if (g0 == 0.f && g1 == 0.f && g2 == 0.f) continue;
-            const int gi = ox + t / 36, gj = oy + (t / 6) % 6, gk = oz + t % 6;
-            if (gi >= n || gj >= n || gk >= n) continue;
-            red_add_v4(&a.G[node_index(sc, gi, gj, gk)], g0, g1, g2, 0.f);
-        }
-        __syncthreads();
-        buf ^= 1;
+        // F_bar = (I + dt C')^T F'_bar;  A = 4n (C'_bar + dt F'_bar F^T)
+#pragma unroll
+        for (int r = 0; r < 3; ++r)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float Fb = aF[3 * r + c] + dt * (Cn[r] * aF[c] + Cn[3 + r] * aF[3 + c] + Cn[6 + r] * aF[6 + c]);
+                if (valid) q.cur.F[(3 * r + c) * cap + p] = Fb;
+                A[3 * r + c] = c4 * (q.nxt.C[(3 * r + c) * cap + s] +
+                                     dt * (aF[3 * r] * F[3 * c] + aF[3 * r + 1] * F[3 * c + 1] + aF[3 * r + 2] * F[3 * c + 2]));
+            }
     }
+    float ax[3], xb[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        ax[d] = q.nxt.x[d * cap + s];
+        // what a node gets is W (vt + A (o - f)) = W (qv + A (o - 1))
+        qv[d] = q.nxt.v[d * cap + s] + dt * ax[d] -
+                (A[3 * d] * (f[0] - 1.f) + A[3 * d + 1] * (f[1] - 1.f) + A[3 * d + 2] * (f[2] - 1.f));
+    }
+    weight_gradient(
+        f, w, node,
+        [&](const float4 v, int i, int j, int k) {
+            const float o0 = (float)(i - 1), o1 = (float)(j - 1), o2 = (float)(k - 1);
+            return v.x * (qv[0] + A[0] * o0 + A[1] * o1 + A[2] * o2) + v.y * (qv[1] + A[3] * o0 + A[4] * o1 + A[5] * o2) +
+                   v.z * (qv[2] + A[6] * o0 + A[7] * o1 + A[8] * o2);
+        },
+        xb);
+    if (valid) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            q.cur.x[d * cap + p] = ax[d] + fn * (xb[d] - (A[d] * vn[0] + A[3 + d] * vn[1] + A[6 + d] * vn[2]));
+        key = (sc.brick_base + ((bc[0] >> 2) * nb + (bc[1] >> 2)) * nb + (bc[2] >> 2)) * 64 + (bc[0] & 3) * 16 + (bc[1] & 3) * 4 +
+              (bc[2] & 3);
+        float4* rec = s_rec[warp] + lane * (kRecPitch / 4);
+        rec[0] = make_float4(f[0], w[3], w[4], w[5]);
+        rec[1] = make_float4(w[6], w[7], w[8], __int_as_float(key));
+        rec[2] = make_float4(qv[0], qv[1], A[0], A[3]);
+        rec[3] = make_float4(A[1], A[4], A[2], A[5]);
+        rec[4] = make_float4(qv[2], A[6], A[7], A[8]);
+        s_scene[warp][lane] = scene;
+    }
+    const int up = __shfl_up_sync(kFull, key, 1);
+    const bool head = valid && (lane == 0 || key != up);
+    const unsigned heads = __ballot_sync(kFull, head);
+    const int runs = __popc(heads);
+    if (head) s_start[warp][__popc(heads & ((1u << lane) - 1u))] = (short)lane;
+    if (lane == 0) s_start[warp][runs] = (short)min(32, a.r.np - g);
+    __syncwarp();
+    scatter_runs<kP2GAdj>(a, s_rec[warp], s_scene[warp], s_start[warp], runs);
 }
 
 // --------------------------------------------------------------- grid^-1
@@ -419,102 +407,60 @@ __global__ void __launch_bounds__(256) k_grid_adj(StepArgs a)
 __global__ void __launch_bounds__(kAdjThreads) k_p2g_adj(AdjArgs q)
 {
     const StepArgs& a = q.a;
-    __shared__ __align__(128) float4 vw[2][8 * 64];
-    __shared__ __align__(8) unsigned long long bar[2];
-    __shared__ int s_item[2];
-    const int tid = threadIdx.x;
     const size_t cap = a.cap;
-    const int n_act = active_bricks(a.sb);
-    int* work = &a.sb.counters[CTR_WORK_P2G];
-    walker_init<kAdjThreads>(a, n_act, vw, bar, s_item, work);
-    unsigned phase[2] = {0u, 0u};
-    int buf = 0;
-    for (;;) {
-        const int item = s_item[buf];
-        if (item >= n_act) break;
-        if (!walker_next(a, n_act, vw, bar, s_item, work, buf, phase, item)) return;
-        const int e = active_entry(a.sb, item);
-        const int start = a.sb.act_start[e], count = a.sb.act_count[e];
-        const int scene = a.sb.act_scene[e];
-        const SceneDev sc = a.scenes[scene];
-        const int n = sc.n, nb = sc.nb, lb = a.sb.act_brick[e] - sc.brick_base;
-        int ox, oy, oz;
-        brick_coords(nb, sc.nb_log2, lb, ox, oy, oz);
-        ox *= 4; oy *= 4; oz *= 4;
-        const float fn = (float)n, dxs = 1.f / fn, m = sc.m_p;
-        const float kA = a.dt * sc.V0 * 4.f * fn * fn;
-        const float4* win = vw[buf];
-        for (int k = tid; k < count; k += kAdjThreads) {
-            const int s = start + k;
-            const int p = a.sb.perm[s];
-            int bc[3];
-            float f[3], w[9], dw[9], x[3];
-            load_x(a.in, p, x);
-            particle_weights(x[0], x[1], x[2], n, bc, f, w);
-            bspline_d(f[0], dw);
-            bspline_d(f[1], dw + 3);
-            bspline_d(f[2], dw + 6);
-            const int l0 = min(max(bc[0] - ox, 0), 3), l1 = min(max(bc[1] - oy, 0), 3), l2 = min(max(bc[2] - oz, 0), 3);
-            float F[9], C[9], v[3], tau[9];
-            load_F(a.in, cap, p, F);
-            load_C(a.in, cap, p, C);
-            load_v(a.in, cap, p, v);
-            const float mu = sc.pp_mat ? a.in.mu[p] : sc.mu, lam = sc.pp_mat ? a.in.lam[p] : sc.lam;
-            float dummy[9], mub0, lamb0;
-            stress_and_vjp(a.model, F, mu, lam, tau, nullptr, dummy, mub0, lamb0);
-            float A[9];
+    const int g = blockIdx.x * kAdjThreads + threadIdx.x;
+    const int s = a.r.p0 + min(g, a.r.np - 1);
+    const SceneDev& sc = a.scenes[scene_of_slot(a, s)];
+    if (active_bricks(a.sb) == 0 || g >= a.r.np) return;
+    const int n = sc.n;
+    const float fn = (float)n, dxs = 1.f / fn, m = sc.m_p;
+    const float kA = a.dt * sc.V0 * 4.f * fn * fn;
+    const int p = a.sb.perm[s];
+    int bc[3];
+    float f[3], w[9], x[3];
+    load_x(a.in, p, x);
+    particle_weights(x[0], x[1], x[2], n, bc, f, w);
+    const GridStencil node(a.V, sc, bc);  // (P_I_bar, m_I_bar)
+    float P[3], Ab[9];                    // sum W P_bar, sum W P_bar d^T
+    gather_velocity<0>(f, w, node, P, Ab);
 #pragma unroll
-            for (int i = 0; i < 9; ++i) A[i] = m * C[i] - kA * tau[i];
-            float vb[3] = {0.f, 0.f, 0.f}, Ab[9], xb[3] = {0.f, 0.f, 0.f};
+    for (int i = 0; i < 9; ++i) Ab[i] *= dxs;
+    float Ad[9], qv[3];
+    {
+        float F[9], C[9], tau[9], tb[9], Fb[9], mub, lamb;
+        load_F(a.in, cap, p, F);
+        const float mu = sc.pp_mat ? a.in.mu[p] : sc.mu, lam = sc.pp_mat ? a.in.lam[p] : sc.lam;
 #pragma unroll
-            for (int i = 0; i < 9; ++i) Ab[i] = 0.f;
+        for (int i = 0; i < 9; ++i) tb[i] = -kA * Ab[i];
+        stress_and_vjp(a.model, F, mu, lam, tau, tb, Fb, mub, lamb);
+        const int gid = sc.p_begin + state_id(a.in, p);
+        q.gmu[gid] += mub;
+        q.glam[gid] += lamb;
+        load_C(a.in, cap, p, C);
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j)
-#pragma unroll
-                    for (int k2 = 0; k2 < 3; ++k2) {
-                        const int wi = l0 + i, wj = l1 + j, wk = l2 + k2;
-                        const float4 g = win[(((wi >> 2) << 2) | ((wj >> 2) << 1) | (wk >> 2)) * 64 + (wi & 3) * 16 + (wj & 3) * 4 + (wk & 3)];
-                        const float Pb[3] = {g.x, g.y, g.z};
-                        const float mb = g.w;
-                        const float W = w[i] * w[3 + j] * w[6 + k2];
-                        const float gW[3] = {fn * dw[i] * w[3 + j] * w[6 + k2], fn * w[i] * dw[3 + j] * w[6 + k2],
-                                             fn * w[i] * w[3 + j] * dw[6 + k2]};
-                        const float d[3] = {((float)i - f[0]) * dxs, ((float)j - f[1]) * dxs, ((float)k2 - f[2]) * dxs};
-                        float s2 = m * mb;
-#pragma unroll
-                        for (int r = 0; r < 3; ++r) {
-                            const float mom = m * v[r] + A[3 * r] * d[0] + A[3 * r + 1] * d[1] + A[3 * r + 2] * d[2];
-                            s2 += Pb[r] * mom;
-                            vb[r] += W * m * Pb[r];
-#pragma unroll
-                            for (int c = 0; c < 3; ++c) Ab[3 * r + c] += W * Pb[r] * d[c];
-                        }
-#pragma unroll
-                        for (int c = 0; c < 3; ++c)
-                            xb[c] += gW[c] * s2 - W * (A[c] * Pb[0] + A[3 + c] * Pb[1] + A[6 + c] * Pb[2]);
-                    }
-            float tb[9], Fb[9], mub, lamb;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) tb[i] = -kA * Ab[i];
-            stress_and_vjp(a.model, F, mu, lam, tau, tb, Fb, mub, lamb);
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                q.cur.x[d * cap + p] += xb[d];
-                q.cur.v[d * cap + p] = vb[d];
-            }
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                q.cur.C[i * cap + p] = m * Ab[i];
-                q.cur.F[i * cap + p] += Fb[i];
-            }
-            const int gid = sc.p_begin + state_id(a.in, p);
-            q.gmu[gid] += mub;
-            q.glam[gid] += lamb;
+        for (int i = 0; i < 9; ++i) {
+            q.cur.F[i * cap + p] += Fb[i];
+            q.cur.C[i * cap + p] = m * Ab[i];
+            Ad[i] = (m * C[i] - kA * tau[i]) * dxs;
         }
-        __syncthreads();
-        buf ^= 1;
+    }
+    float v[3], xb[3];
+    load_v(a.in, cap, p, v);
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+        qv[d] = m * v[d] - (Ad[3 * d] * (f[0] - 1.f) + Ad[3 * d + 1] * (f[1] - 1.f) + Ad[3 * d + 2] * (f[2] - 1.f));
+    weight_gradient(
+        f, w, node,
+        [&](const float4 b, int i, int j, int k) {
+            const float o0 = (float)(i - 1), o1 = (float)(j - 1), o2 = (float)(k - 1);
+            return m * b.w + b.x * (qv[0] + Ad[0] * o0 + Ad[1] * o1 + Ad[2] * o2) +
+                   b.y * (qv[1] + Ad[3] * o0 + Ad[4] * o1 + Ad[5] * o2) + b.z * (qv[2] + Ad[6] * o0 + Ad[7] * o1 + Ad[8] * o2);
+        },
+        xb);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        q.cur.x[d * cap + p] += fn * (xb[d] - (Ad[d] * P[0] + Ad[3 + d] * P[1] + Ad[6 + d] * P[2]));
+        q.cur.v[d * cap + p] = m * P[d];
     }
 }
 
@@ -667,7 +613,7 @@ static int sort_with_perm(mpm_ctx* c, StepArgs& a, const PState& state, int* per
 {
     MPM_CKA(reset_histogram(c));
     MPM_CKA(launch_prepare(a, state, c->stream));
-    MPM_CKA(launch_sort(a, c->stream, false));
+    MPM_CKA(launch_scan(a, c->stream));
     a.sb.perm = perm;
     return MPM_OK;
 }
@@ -708,7 +654,7 @@ static int backward_device(mpm_ctx* c, const SeedIn& seeds, const AdjOut& outs)
         // recompute the segment's states
         for (int j = j0; j < j1 - 1; ++j) {
             StepArgs a = step_args(c, t->dts[j], 0, c->n_scenes, seg_state(j - j0), seg_state(j - j0 + 1));
-            a.tau_valid = 0;
+            a.tau_valid = j > 0;  // every state but the first is a G2P's, with its stress
             if ((st = sort_with_perm(c, a, seg_state(j - j0), t->perms + (size_t)j * cap))) return st;
             MPM_CKA(launch_p2g(a, c->stream));
             MPM_CKA(launch_grid(a, c->stream, false));
@@ -717,14 +663,12 @@ static int backward_device(mpm_ctx* c, const SeedIn& seeds, const AdjOut& outs)
         // reverse the segment's substeps
         for (int j = j1 - 1; j >= j0; --j) {
             StepArgs a = step_args(c, t->dts[j], 0, c->n_scenes, seg_state(j - j0), seg_state(j - j0));
-            a.tau_valid = 0;
+            a.tau_valid = j > 0;
             if ((st = sort_with_perm(c, a, seg_state(j - j0), t->perms + (size_t)j * cap))) return st;
             MPM_CKA(launch_p2g(a, c->stream));
             MPM_CKA(launch_grid(a, c->stream, true));
             AdjArgs q{a, adj[nxt], adj[nxt ^ 1], gmu, glam};
-            const int ctas = c->num_sms * 2;
-            // the walkers fetch work from the G2P and P2G counters: reset them
-            MPM_CKA(cudaMemsetAsync(c->sb.counters + CTR_WORK_P2G, 0, sizeof(int) * 3, c->stream));
+            const int ctas = n_blocks(std::max(N, 1), kAdjThreads);
             k_g2p_adj<<<ctas, kAdjThreads, 0, c->stream>>>(q);
             MPM_CKA(cudaGetLastError());
             k_grid_adj<<<c->num_sms * 8, 256, 0, c->stream>>>(a);

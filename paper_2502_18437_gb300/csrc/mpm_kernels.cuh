@@ -83,7 +83,9 @@ constexpr int kBigBrick = 256;
 cudaError_t launch_prepare(const StepArgs& a, const PState& st, cudaStream_t s);
 // zero the brick histogram, the tile counts and the list sizes (all scenes)
 cudaError_t launch_reset_histogram(const SortBufs& sb, int bricks, int tiles, cudaStream_t s);
-cudaError_t launch_sort(const StepArgs& a, cudaStream_t s, bool write_perm = true);
+// the scan alone serves launches that bring a permutation of their own
+cudaError_t launch_scan(const StepArgs& a, cudaStream_t s);
+cudaError_t launch_sort(const StepArgs& a, cudaStream_t s);
 cudaError_t launch_p2g(const StepArgs& a, cudaStream_t s);
 cudaError_t prepare_p2g();  // shared-memory opt-in of the P2G variants (once per device, before any launch)
 // clear: reset the P2G accumulator afterwards (G2P does it otherwise)

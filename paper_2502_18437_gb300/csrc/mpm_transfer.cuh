@@ -225,6 +225,265 @@ __device__ __forceinline__ void scan_cells(const int* cell_cnt, int* cell_off, i
     }
 }
 
+// Scene of slot s (scenes own consecutive slots): two warp-wide probes of the
+// scenes' first slots for the warp's first slot, then the few lanes of later scenes
+// step on.  Every lane of the warp calls it.
+__device__ __forceinline__ int scene_of_slot(const StepArgs& a, int s)
+{
+    if (a.r.s1 - a.r.s0 == 1) return a.r.s0;
+    const int lane = threadIdx.x & 31, s_first = __shfl_sync(kFull, s, 0);
+    int lo = a.r.s0, len = a.r.s1 - a.r.s0;
+    while (len > 1) {  // p_begin never decreases: the last scene that starts at or before s_first
+        const int step = (len + 31) >> 5, at = lane * step;
+        const bool le = at < len && a.scenes[lo + at].p_begin <= s_first;
+        const int k = 31 - __clz(__ballot_sync(kFull, le) | 1u);
+        lo += k * step;
+        len = min(step, len - k * step);
+    }
+    while (lo + 1 < a.r.s1 && a.scenes[lo + 1].p_begin <= s) ++lo;
+    return lo;
+}
+
+__device__ __forceinline__ void cp_async16(float4* dst, const float4* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+constexpr int kRecPitch = 20;  // floats per record: an odd number of 16-byte words
+
+// MODE: kP2GStress (MLS-MPM: the Kirchhoff stress, stored by G2P or computed
+// from F), kP2GConstraint (PB-MPM: the co-rotational constraint replaces C
+// and there is no stress term) or kP2GStd (standard MPM, Sec. III-A: W m v and the
+// internal-force impulse -dt V0 tau grad W, Eq. 2, 3).  kP2GAdj: the reverse of G2P
+// adds three values and no mass.
+enum { kP2GStress = 0, kP2GConstraint = 1, kP2GStd = 2, kP2GAdj = 3 };
+
+// Adds a record's contributions to the nodes (i, j, k) of plane i: (p_x, p_y) in
+// acc_a[3 j + k], (p_z, weight) in acc_b.
+template <int MODE>
+__device__ __forceinline__ void p2g_add(const float4* rec, int i, float2 acc_a[9], float2 acc_b[9])
+{
+    const auto two = [](float s) { return make_float2(s, s); };
+    const float4 r0 = rec[0], r1 = rec[1], r2 = rec[2], r3 = rec[3], r4 = rec[4];
+    const float wy[3] = {r0.y, r0.z, r0.w}, wz[3] = {r1.x, r1.y, r1.z};
+    // w_i(f) = alpha + beta (f - gamma)^2
+    const float gam = i == 0 ? 1.5f : (i == 1 ? 1.0f : 0.5f), bet = i == 1 ? -1.0f : 0.5f, alp = i == 1 ? 0.75f : 0.0f;
+    const float e = r0.x - gam, wi = __fmaf_rn(bet * e, e, alp);
+    if (MODE == kP2GStd) {
+        // p = (wx m v - dwx T_x) wy wz - wx (T_y dwy wz + T_z wy dwz)
+        const float dwx = 2.f * bet * e;
+        const float mv[3] = {r2.x, r2.y, r2.z}, T[9] = {r3.x, r3.y, r3.z, r3.y, r3.w, r4.x, r3.z, r4.x, r4.y};
+        float dy[3], dz[3];
+        bspline_d(r2.w, dy);
+        bspline_d(r4.z, dz);
+        float A[3], B[3], C[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            A[c] = wi * mv[c] - dwx * T[3 * c];
+            B[c] = wi * T[3 * c + 1];
+            C[c] = wi * T[3 * c + 2];
+        }
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            float P[3], Q[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                P[c] = wy[j] * A[c] - dy[j] * B[c];
+                Q[c] = -wy[j] * C[c];
+            }
+            const float W = wi * wy[j];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int q = 3 * j + k;
+                acc_a[q] = __ffma2_rn(make_float2(P[0], P[1]), two(wz[k]), acc_a[q]);
+                acc_a[q] = __ffma2_rn(make_float2(Q[0], Q[1]), two(dz[k]), acc_a[q]);
+                acc_b[q] = __ffma2_rn(make_float2(P[2], W), two(wz[k]), acc_b[q]);
+                acc_b[q].x = __fmaf_rn(Q[2], dz[k], acc_b[q].x);
+            }
+        }
+        return;
+    }
+    const float si = (float)(i - 1);
+    const float2 a1 = make_float2(r3.x, r3.y), a2 = make_float2(r3.z, r3.w);
+    const float2 v01 = __ffma2_rn(two(si), make_float2(r2.z, r2.w), make_float2(r2.x, r2.y));
+    const float v2 = __fmaf_rn(si, r4.y, r4.x);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const float wij = wi * wy[j], fj = (float)(j - 1);
+        const float2 s01 = j == 1 ? v01 : __ffma2_rn(two(fj), a1, v01);
+        const float s2 = j == 1 ? v2 : __fmaf_rn(fj, r4.z, v2);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float W = wij * wz[k], fk = (float)(k - 1);
+            const int q = 3 * j + k;
+            const float2 u01 = k == 1 ? s01 : __ffma2_rn(two(fk), a2, s01);
+            const float2 u2w = make_float2(k == 1 ? s2 : __fmaf_rn(fk, r4.w, s2), 1.0f);
+            acc_a[q] = __ffma2_rn(two(W), u01, acc_a[q]);
+            acc_b[q] = __ffma2_rn(two(W), u2w, acc_b[q]);
+        }
+    }
+}
+
+// Phases B and C of P2G: the records' contributions to the nodes, summed by run (of
+// records of one base cell; run r starts at s_start[r]) and node plane i, joined where
+// runs are neighbours in z, and added to G.  Called by a whole warp.
+template <int MODE>
+__device__ __forceinline__ void scatter_runs(const StepArgs& a, const float4* rec, const int* s_scene, const short* s_start,
+                                             int runs)
+{
+    const int lane = threadIdx.x & 31;
+    for (int job0 = 0; job0 < 3 * runs; job0 += 32) {
+        const int job = job0 + lane, run = min(job / 3, runs - 1), i = job - (job / 3) * 3, beg = s_start[run];
+        const bool own = job < 3 * runs;
+        const int end = own ? s_start[run + 1] : beg;
+        float2 acc_a[9], acc_b[9];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) acc_a[q] = acc_b[q] = make_float2(0.f, 0.f);
+        for (int q = beg; q < end; ++q) p2g_add<MODE>(rec + q * (kRecPitch / 4), i, acc_a, acc_b);
+        __syncwarp();
+        const int key = __float_as_int(rec[beg * (kRecPitch / 4) + 1].w);
+        const int ly = (key >> 2) & 3, lz = key & 3;
+        // C: three lanes on lies the next run; where its cell is the next one in z
+        // (of the brick), its nodes 0 and 1 are this run's 1 and 2
+        const int before = __shfl_up_sync(kFull, key, 3);
+        const bool joined = own && lane >= 3 && lz > 0 && before == key - 1;
+        const bool last = !(__shfl_down_sync(kFull, joined, 3) && lane < 29);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const auto join = [&](float v0, float& v1, float v2) {
+                const float c2 = __shfl_up_sync(kFull, v2, 3);
+                if (joined) v1 += c2;
+                const float c1 = __shfl_up_sync(kFull, v1, 3);
+                return joined ? v0 + c1 : v0;
+            };
+            float2 *p = acc_a + 3 * j, *q = acc_b + 3 * j;
+            p[0].x = join(p[0].x, p[1].x, p[2].x);
+            p[0].y = join(p[0].y, p[1].y, p[2].y);
+            q[0].x = join(q[0].x, q[1].x, q[2].x);
+            q[0].y = join(q[0].y, q[1].y, q[2].y);
+        }
+        if (own) {
+            const SceneDev& sc = a.scenes[s_scene[beg]];
+            const int nb = sc.nb, lx = ((key >> 4) & 3) + i;
+            const float m = sc.m_p;
+            float4* g = a.G + (key + i * 16 + (lx > 3 ? (nb * nb - 1) * 64 : 0));
+#pragma unroll
+            for (int q = 0; q < 9; ++q)
+                if (q % 3 == 0 || last) {
+                    float4* to = g + ((q / 3) * 4 + q % 3 + (ly + q / 3 > 3 ? nb * 64 - 16 : 0) + (lz + q % 3 > 3 ? 60 : 0));
+                    if (MODE == kP2GAdj) red_add_v4(to, acc_a[q].x, acc_a[q].y, acc_b[q].x, 0.f);
+                    else red_add_v4(to, acc_b[q].y * m, acc_a[q].x, acc_a[q].y, acc_b[q].x);
+                }
+        }
+    }
+}
+
+// Variants of the forward G2P (template flags).
+enum {
+    kG2PSolids = 1,    // push particles out of solid rigids (some scene has a sphere or a box)
+    kG2PStdGrad = 2,   // standard MPM: L = sum v_I grad phi^T instead of the APIC C (Eq. 5)
+    kG2PNoStress = 4   // PB-MPM: no constitutive update (no stress is stored)
+};
+
+// Velocity and affine matrix gathered at a position:
+//   v = sum W v_I,  B_rc = sum W v_I,r (o_c - f_c),  W = wx_i wy_j wz_k
+// (kG2PStdGrad: the basis gradient in cell units instead, B_rc = sum v_I,r dW/df_c),
+// contracted separably over k, then j, then i; x and y go in paired FMAs.  The
+// velocities are taken relative to the middle node's, whose share is known (sum W = 1,
+// B = 0): a bulk motion then leaves no rounding in B.
+// node(i, j, k) returns (v, m) of the stencil's nodes.
+template <int FLAGS, class Node>
+__device__ __forceinline__ void gather_velocity(const float f[3], const float w[9], Node node, float v[3], float B[9])
+{
+    const float* wy = w + 3;
+    const float* wz = w + 6;
+    float wyd[3], wzd[3];
+    if (FLAGS & kG2PStdGrad) {
+        bspline_d(f[1], wyd);
+        bspline_d(f[2], wzd);
+    } else {
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            wyd[q] = wy[q] * ((float)q - f[1]);
+            wzd[q] = wz[q] * ((float)q - f[2]);
+        }
+    }
+    const auto two = [](float s) { return make_float2(s, s); };
+    const float4 mid = node(1, 1, 1);
+    float2 vp = two(0.f), B0 = two(0.f), B1 = two(0.f), B2 = two(0.f);  // x, y rows
+    float vz = 0.f, Bz0 = 0.f, Bz1 = 0.f, Bz2 = 0.f;                    // z row
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        // weight of plane i (as bspline) and its derivative or moment
+        const float fi = (float)i;
+        const float e = f[0] - (1.5f - 0.5f * fi);
+        const float wx = i == 1 ? 0.75f - e * e : 0.5f * e * e;
+        const float wxd = (FLAGS & kG2PStdGrad) ? (i == 1 ? -2.f * e : e) : wx * (fi - f[0]);
+        float2 A = two(0.f), Ay = two(0.f), Az = two(0.f);
+        float zA = 0.f, zAy = 0.f, zAz = 0.f;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            float2 p = two(0.f), d = two(0.f);
+            float zp = 0.f, zd = 0.f;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float4 g = node(i, j, k);
+                const float2 xy = __fadd2_rn(make_float2(g.x, g.y), make_float2(-mid.x, -mid.y));
+                const float z = g.z - mid.z;
+                p = __ffma2_rn(two(wz[k]), xy, p);
+                d = __ffma2_rn(two(wzd[k]), xy, d);
+                zp = __fmaf_rn(wz[k], z, zp);
+                zd = __fmaf_rn(wzd[k], z, zd);
+            }
+            A = __ffma2_rn(two(wy[j]), p, A);
+            Ay = __ffma2_rn(two(wyd[j]), p, Ay);
+            Az = __ffma2_rn(two(wy[j]), d, Az);
+            zA = __fmaf_rn(wy[j], zp, zA);
+            zAy = __fmaf_rn(wyd[j], zp, zAy);
+            zAz = __fmaf_rn(wy[j], zd, zAz);
+        }
+        vp = __ffma2_rn(two(wx), A, vp);
+        B0 = __ffma2_rn(two(wxd), A, B0);
+        B1 = __ffma2_rn(two(wx), Ay, B1);
+        B2 = __ffma2_rn(two(wx), Az, B2);
+        vz = __fmaf_rn(wx, zA, vz);
+        Bz0 = __fmaf_rn(wxd, zA, Bz0);
+        Bz1 = __fmaf_rn(wx, zAy, Bz1);
+        Bz2 = __fmaf_rn(wx, zAz, Bz2);
+    }
+    v[0] = vp.x + mid.x; v[1] = vp.y + mid.y; v[2] = vz + mid.z;
+    B[0] = B0.x; B[1] = B1.x; B[2] = B2.x;
+    B[3] = B0.y; B[4] = B1.y; B[5] = B2.y;
+    B[6] = Bz0; B[7] = Bz1; B[8] = Bz2;
+}
+
+// Nodes of a base cell's stencil in the brick layout, read through L1.
+struct GridStencil {
+    const float4* V;
+    int x0, sx, o[6];  // first x, stride of bricks along x, node offsets along y and z (with the scene's first node)
+    __device__ __forceinline__ GridStencil(const float4* V_, const SceneDev& sc, const int bc[3]) : V(V_), x0(bc[0])
+    {
+        const int sy = sc.nb * 64;
+        sx = sc.nb * sy;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int y = bc[1] + i, z = bc[2] + i;
+            o[i] = (y >> 2) * sy + (y & 3) * 4 + sc.brick_base * 64;
+            o[3 + i] = (z >> 2) * 64 + (z & 3);
+        }
+    }
+    __device__ __forceinline__ float4 operator()(int i, int j, int k) const
+    {
+        const int x = x0 + i, ox = (x >> 2) * sx + (x & 3) * 16;
+        return __ldg(V + (ox + o[j] + o[3 + k]));
+    }
+};
+
 // Global node index of node (gi, gj, gk) of a scene (brick layout).
 __device__ __forceinline__ int node_index(const SceneDev& sc, int gi, int gj, int gk)
 {
