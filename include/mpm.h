@@ -109,7 +109,8 @@ enum {
                                    substep (forces direct launches); see mpm_phase_stats */
     MPM_OPT_P2G_CHUNK = 8,      /* particles of two passes of a P2G CTA: 384, 576
                                    or 768 (default), i.e. 32, 48 or 64 staged by each
-                                   of its six warps; small launches stage 32        */
+                                   of its six warps; launches that 32 a warp fit on
+                                   the chip at once stage 32                        */
     MPM_OPT_FUSED = 9,          /* 1: fuse each substep's G2P with the next substep's
                                    P2G; 0 (default): separate P2G and G2P kernels */
     MPM_OPT_G2P_REGS64 = 10     /* 1: G2P variant limited to 64 registers (more

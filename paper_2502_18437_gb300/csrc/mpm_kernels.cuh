@@ -108,7 +108,7 @@ struct Fields {
     float* f[4];
 };
 // From this many particles the state is read by id, through records; below, by slot, in one
-// kernel.  Measured, by id and by slot: 35 and 33 us at 64k, 36 and 45 at 131k, 49 and 57 at
+// kernel.  Measured, by id and by slot: 35 and 26 us at 64k, 36 and 37 at 131k, 49 and 57 at
 // 262k, 133 and 219 at 1M, 485 and 1,306 at 4M.
 constexpr int kIoByIdFrom = 1 << 17;
 // state -> arrays (out) or arrays -> state; inv: scratch of np ints, spare: the state's other
