@@ -420,7 +420,7 @@ extern "C" int mpm_create(const mpm_config* cfg, void* stream, mpm_ctx** out)
         c->own_stream = e == cudaSuccess;
     }
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device);
-    if (e == cudaSuccess) e = prepare_p2g();
+    if (e == cudaSuccess) e = prepare_kernels();
     const size_t nbk = (size_t)c->total_bricks;
     // one allocation for all buffers; those that start from zero come first
     struct Part { void** p; size_t bytes; };

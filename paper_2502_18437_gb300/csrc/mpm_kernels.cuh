@@ -87,7 +87,7 @@ cudaError_t launch_reset_histogram(const SortBufs& sb, int bricks, int tiles, cu
 cudaError_t launch_scan(const StepArgs& a, cudaStream_t s);
 cudaError_t launch_sort(const StepArgs& a, cudaStream_t s);
 cudaError_t launch_p2g(const StepArgs& a, cudaStream_t s);
-cudaError_t prepare_p2g();  // shared-memory opt-in of the P2G variants (once per device, before any launch)
+cudaError_t prepare_kernels();  // shared-memory sizes of P2G and G2P (once per device, before any launch)
 // clear: reset the P2G accumulator afterwards (G2P does it otherwise)
 cudaError_t launch_grid(const StepArgs& a, cudaStream_t s, bool clear);
 cudaError_t launch_g2p(const StepArgs& a, cudaStream_t s);
