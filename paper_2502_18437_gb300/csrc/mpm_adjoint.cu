@@ -42,6 +42,7 @@ using namespace mpm;
 struct mpm_tape {
     int K = 0, max_steps = 0, cap = 0;
     std::vector<float> dts;
+    void* arena = nullptr;     // holds all of the below
     std::vector<float*> ckpt;  // states at substeps 0, K, 2K, ...
     float* seg = nullptr;      // K states of the segment being reversed
     int* perms = nullptr;      // [max_steps][cap] recorded permutations
@@ -274,6 +275,7 @@ constexpr int kAdjWarps = kAdjThreads / 32;
 // (One CTA per brick with shared-memory atomics, 81 per particle: 67 us for 32k particles.)
 __global__ void __launch_bounds__(kAdjThreads) k_g2p_adj(AdjArgs q)
 {
+    chain_wait();
     const StepArgs& a = q.a;
     __shared__ float4 s_rec[kAdjWarps][32 * (kRecPitch / 4)];
     __shared__ int s_scene[kAdjWarps][32];
@@ -361,6 +363,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_g2p_adj(AdjArgs q)
 // into V and clears G.
 __global__ void __launch_bounds__(256) k_grid_adj(StepArgs a)
 {
+    chain_wait();
     const int tid = threadIdx.x, grp = tid >> 6, nid = tid & 63;
     const int n_nact = a.sb.counters[CTR_N_NACT];
     for (int base = blockIdx.x * 4; base < n_nact; base += gridDim.x * 4) {
@@ -406,6 +409,7 @@ __global__ void __launch_bounds__(256) k_grid_adj(StepArgs a)
 
 __global__ void __launch_bounds__(kAdjThreads) k_p2g_adj(AdjArgs q)
 {
+    chain_wait();
     const StepArgs& a = q.a;
     const size_t cap = a.cap;
     const int g = blockIdx.x * kAdjThreads + threadIdx.x;
@@ -521,12 +525,7 @@ void mpm_tape_free(mpm_ctx* c)
 {
     if (!c || !c->tape) return;
     mpm_tape* t = c->tape;
-    for (float* p : t->ckpt) cudaFree(p);
-    cudaFree(t->seg);
-    cudaFree(t->perms);
-    cudaFree(t->adj);
-    cudaFree(t->gmat);
-    cudaFree(t->io);
+    cudaFree(t->arena);
     delete t;
     c->tape = nullptr;
 }
@@ -554,17 +553,22 @@ extern "C" int mpm_tape_begin(mpm_ctx* c)
         c->tape = t;
         const size_t sb = state_bytes(c->cap);
         const int n_ckpt = t->max_steps / t->K + 1;
-        cudaError_t e = cudaSuccess;
-        for (int k = 0; k < n_ckpt && e == cudaSuccess; ++k) {
-            float* p = nullptr;
-            e = cudaMalloc(&p, sb);
-            t->ckpt.push_back(p);
-        }
-        if (e == cudaSuccess) e = cudaMalloc(&t->seg, sb * (size_t)t->K);
-        if (e == cudaSuccess) e = cudaMalloc(&t->perms, sizeof(int) * (size_t)c->cap * t->max_steps);
-        if (e == cudaSuccess) e = cudaMalloc(&t->adj, sizeof(float) * 48 * (size_t)c->cap);
-        if (e == cudaSuccess) e = cudaMalloc(&t->gmat, sizeof(float) * 2 * (size_t)c->cap);
-        if (e == cudaSuccess) e = cudaMalloc(&t->io, sizeof(float) * kIoFloats * (size_t)c->cap);
+        const auto round = [](size_t bytes) { return (bytes + 255) & ~(size_t)255; };
+        const size_t cap = c->cap, b_perms = round(sizeof(int) * cap * t->max_steps), b_adj = round(sizeof(float) * 48 * cap),
+                     b_gmat = round(sizeof(float) * 2 * cap), b_io = round(sizeof(float) * kIoFloats * cap);
+        const cudaError_t e = cudaMalloc(&t->arena, sb * ((size_t)n_ckpt + t->K) + b_perms + b_adj + b_gmat + b_io);
+        char* at = static_cast<char*>(t->arena);
+        const auto take = [&](size_t bytes) {
+            char* p = at;
+            at += bytes;
+            return p;
+        };
+        for (int k = 0; k < n_ckpt; ++k) t->ckpt.push_back(reinterpret_cast<float*>(take(sb)));
+        t->seg = reinterpret_cast<float*>(take(sb * (size_t)t->K));
+        t->perms = reinterpret_cast<int*>(take(b_perms));
+        t->adj = reinterpret_cast<float*>(take(b_adj));
+        t->gmat = reinterpret_cast<float*>(take(b_gmat));
+        t->io = reinterpret_cast<float*>(take(b_io));
         if (e != cudaSuccess) {
             mpm_tape_free(c);
             return status_from_cuda(e);
@@ -669,11 +673,11 @@ static int backward_device(mpm_ctx* c, const SeedIn& seeds, const AdjOut& outs)
             MPM_CKA(launch_grid(a, c->stream, true));
             AdjArgs q{a, adj[nxt], adj[nxt ^ 1], gmu, glam};
             const int ctas = n_blocks(std::max(N, 1), kAdjThreads);
-            k_g2p_adj<<<ctas, kAdjThreads, 0, c->stream>>>(q);
+            launch_chain(N, k_g2p_adj, ctas, kAdjThreads, 0, c->stream, q);
             MPM_CKA(cudaGetLastError());
-            k_grid_adj<<<c->num_sms * 8, 256, 0, c->stream>>>(a);
+            launch_chain(N, k_grid_adj, c->num_sms * 8, 256, 0, c->stream, a);
             MPM_CKA(cudaGetLastError());
-            k_p2g_adj<<<ctas, kAdjThreads, 0, c->stream>>>(q);
+            launch_chain(N, k_p2g_adj, ctas, kAdjThreads, 0, c->stream, q);
             MPM_CKA(cudaGetLastError());
             nxt ^= 1;
         }

@@ -293,7 +293,7 @@ int invalidate_pending(mpm_ctx* c)
     return MPM_OK;
 }
 
-cudaError_t reset_histogram(mpm_ctx* c) { return launch_reset_histogram(c->sb, c->total_bricks, c->total_tiles, c->stream); }
+cudaError_t reset_histogram(mpm_ctx* c) { return launch_reset_histogram(c->sb, c->total_bricks, c->total_tiles, c->total_particles, c->stream); }
 
 int ensure_keys(mpm_ctx* c)
 {

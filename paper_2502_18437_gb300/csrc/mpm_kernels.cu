@@ -19,16 +19,6 @@
 
 namespace mpm {
 
-// Small launches of the substep chain are made programmatic: a kernel's CTAs come up
-// while the one before it still runs, and wait here for its end and its writes (every
-// thread, before its first access); the next kernel may come up at once.  Elsewhere both
-// do nothing.
-__device__ __forceinline__ void chain_wait()
-{
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
 // ----------------------------------------------------------------- scan
 //
 // A scan tile is 2^tile_shift consecutive bricks of one scene (tiles never
@@ -213,6 +203,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(StepArgs a)
 
 __global__ void k_reset_histogram(SortBufs sb, int bricks, int tiles)
 {
+    chain_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < bricks && sb.cnt[i]) {
         // only bricks with particles have counts in their cells
@@ -268,6 +259,7 @@ constexpr int kPrepTiles = 2048;
 
 __global__ void __launch_bounds__(256) k_prepare(StepArgs a, PState st)
 {
+    chain_wait();
     __shared__ int s_tile[kPrepTiles];
     const bool block_sums = a.r.nt <= kPrepTiles;
     if (block_sums)
@@ -1645,38 +1637,22 @@ __global__ void k_read_grid(const float4* V, const int* brick_epoch, const int* 
 
 static int n_blocks(long long n, int t) { return (int)((n + t - 1) / t); }
 
-template <class... P, class... A>
-static void launch_chain(const StepArgs& a, void (*k)(P...), int ctas, int threads, size_t smem, cudaStream_t s, A... args)
-{
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(ctas);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute programmatic;
-    programmatic.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    programmatic.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &programmatic;
-    cfg.numAttrs = a.r.np < kChainBelow ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, k, args...);
-}
-
 cudaError_t launch_prepare(const StepArgs& a, const PState& st, cudaStream_t s)
 {
     if (a.r.np == 0) return cudaSuccess;
-    k_prepare<<<n_blocks(a.r.np, 256), 256, 0, s>>>(a, st);
+    launch_chain(a.r.np, k_prepare, n_blocks(a.r.np, 256), 256, 0, s, a, st);
     return cudaGetLastError();
 }
 
-cudaError_t launch_reset_histogram(const SortBufs& sb, int bricks, int tiles, cudaStream_t s)
+cudaError_t launch_reset_histogram(const SortBufs& sb, int bricks, int tiles, int np, cudaStream_t s)
 {
-    k_reset_histogram<<<n_blocks(max(bricks, 32), 256), 256, 0, s>>>(sb, bricks, tiles);
+    launch_chain(np, k_reset_histogram, n_blocks(max(bricks, 32), 256), 256, 0, s, sb, bricks, tiles);
     return cudaGetLastError();
 }
 
 cudaError_t launch_scan(const StepArgs& a, cudaStream_t s)
 {
-    launch_chain(a, k_scan, a.r.nt, kScanThreads, 0, s, a);
+    launch_chain(a.r.np, k_scan, a.r.nt, kScanThreads, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -1684,7 +1660,7 @@ cudaError_t launch_sort(const StepArgs& a, cudaStream_t s)
 {
     cudaError_t e = launch_scan(a, s);
     if (e != cudaSuccess) return e;
-    launch_chain(a, k_scatter, n_blocks(max(a.r.np, a.r.nt), 256 * kScatterPer), 256, 0, s, a);
+    launch_chain(a.r.np, k_scatter, n_blocks(max(a.r.np, a.r.nt), 256 * kScatterPer), 256, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -1704,25 +1680,25 @@ cudaError_t launch_p2g(const StepArgs& a, cudaStream_t s)
 {
     const int c = min(a.p2g_ctas, n_blocks(max(a.r.np, 1), kP2GWarps * a.p2g_slots));
     const size_t smem = kP2GWarps * p2g_warp_bytes(a.p2g_slots);
-    if (a.solver == MPM_SOLVER_PB) launch_chain(a, k_p2g<kP2GConstraint>, c, kP2GThreads, smem, s, a);
-    else if (a.solver == MPM_SOLVER_STANDARD) launch_chain(a, k_p2g<kP2GStd>, c, kP2GThreads, smem, s, a);
-    else launch_chain(a, k_p2g<kP2GStress>, c, kP2GThreads, smem, s, a);
+    if (a.solver == MPM_SOLVER_PB) launch_chain(a.r.np, k_p2g<kP2GConstraint>, c, kP2GThreads, smem, s, a);
+    else if (a.solver == MPM_SOLVER_STANDARD) launch_chain(a.r.np, k_p2g<kP2GStd>, c, kP2GThreads, smem, s, a);
+    else launch_chain(a.r.np, k_p2g<kP2GStress>, c, kP2GThreads, smem, s, a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_g2p_vc(const StepArgs& a, cudaStream_t s)
 {
     if (a.r.np == 0) return cudaSuccess;
-    launch_chain(a, k_g2p_vc, n_blocks(a.r.np, kVcThreads), kVcThreads, 0, s, a);
+    launch_chain(a.r.np, k_g2p_vc, n_blocks(a.r.np, kVcThreads), kVcThreads, 0, s, a);
     return cudaGetLastError();
 }
 
 cudaError_t launch_grid(const StepArgs& a, cudaStream_t s, bool clear)
 {
-    if (!a.any_rigid) launch_chain(a, k_grid_plain, a.grid_plain_ctas, kGridThreads, 0, s, a);
-    else if (a.rigid_ext) launch_chain(a, k_grid<true>, a.grid_ctas, kGridThreads, 0, s, a);
-    else launch_chain(a, k_grid<false>, a.grid_ctas, kGridThreads, 0, s, a);
-    if (clear) launch_chain(a, k_grid_clear, a.grid_plain_ctas, kGridThreads, 0, s, a);
+    if (!a.any_rigid) launch_chain(a.r.np, k_grid_plain, a.grid_plain_ctas, kGridThreads, 0, s, a);
+    else if (a.rigid_ext) launch_chain(a.r.np, k_grid<true>, a.grid_ctas, kGridThreads, 0, s, a);
+    else launch_chain(a.r.np, k_grid<false>, a.grid_ctas, kGridThreads, 0, s, a);
+    if (clear) launch_chain(a.r.np, k_grid_clear, a.grid_plain_ctas, kGridThreads, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -1732,15 +1708,15 @@ static void launch_g2p_variant(const StepArgs& a, cudaStream_t s)
     const int c = min(a.g2p_ctas, n_blocks(max(a.r.np, 1), a.g2p_threads));
     if (a.g2p_regs64) {
         switch (a.g2p_threads) {
-        case 128: launch_chain(a, k_g2p<128, 8, FLAGS>, c, 128, 0, s, a); break;
-        case 512: launch_chain(a, k_g2p<512, 2, FLAGS>, c, 512, 0, s, a); break;
-        default: launch_chain(a, k_g2p<256, 4, FLAGS>, c, 256, 0, s, a); break;
+        case 128: launch_chain(a.r.np, k_g2p<128, 8, FLAGS>, c, 128, 0, s, a); break;
+        case 512: launch_chain(a.r.np, k_g2p<512, 2, FLAGS>, c, 512, 0, s, a); break;
+        default: launch_chain(a.r.np, k_g2p<256, 4, FLAGS>, c, 256, 0, s, a); break;
         }
     } else {
         switch (a.g2p_threads) {
-        case 128: launch_chain(a, k_g2p<128, 6, FLAGS>, c, 128, 0, s, a); break;
-        case 512: launch_chain(a, k_g2p<512, 1, FLAGS>, c, 512, 0, s, a); break;
-        default: launch_chain(a, k_g2p<256, 3, FLAGS>, c, 256, 0, s, a); break;
+        case 128: launch_chain(a.r.np, k_g2p<128, 6, FLAGS>, c, 128, 0, s, a); break;
+        case 512: launch_chain(a.r.np, k_g2p<512, 1, FLAGS>, c, 512, 0, s, a); break;
+        default: launch_chain(a.r.np, k_g2p<256, 3, FLAGS>, c, 256, 0, s, a); break;
         }
     }
 }
@@ -1753,11 +1729,11 @@ cudaError_t launch_g2p(const StepArgs& a, cudaStream_t s)
     // the push-out variant only where a scene has a solid shape: blades, needles and
     // segments push nothing out
     if (a.solver == MPM_SOLVER_STANDARD) {
-        if (a.any_solid) launch_chain(a, k_g2p<128, 6, kG2PStdGrad | kG2PSolids>, c, 128, 0, s, a);
-        else launch_chain(a, k_g2p<128, 6, kG2PStdGrad>, c, 128, 0, s, a);
+        if (a.any_solid) launch_chain(a.r.np, k_g2p<128, 6, kG2PStdGrad | kG2PSolids>, c, 128, 0, s, a);
+        else launch_chain(a.r.np, k_g2p<128, 6, kG2PStdGrad>, c, 128, 0, s, a);
     } else if (a.solver == MPM_SOLVER_PB) {
-        if (a.any_solid) launch_chain(a, k_g2p<128, 6, kG2PNoStress | kG2PSolids>, c, 128, 0, s, a);
-        else launch_chain(a, k_g2p<128, 6, kG2PNoStress>, c, 128, 0, s, a);
+        if (a.any_solid) launch_chain(a.r.np, k_g2p<128, 6, kG2PNoStress | kG2PSolids>, c, 128, 0, s, a);
+        else launch_chain(a.r.np, k_g2p<128, 6, kG2PNoStress>, c, 128, 0, s, a);
     } else if (a.any_solid) {
         launch_g2p_variant<kG2PSolids>(a, s);
     } else {

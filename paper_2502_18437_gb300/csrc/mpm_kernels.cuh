@@ -72,9 +72,10 @@ constexpr int kP2GMaxSlots = 64;
 constexpr int kScanThreads = 256;
 constexpr int kMinTileShift = 8;  // a scan tile holds at least kScanThreads bricks
 // Launches of fewer particles are made programmatic (launch_chain).  A substep with and
-// without: 19.6 and 21.0 us at 4k particles, 22.2 and 23.8 at 16k; 26.4 and 25.1 at 64k, 134
-// and 128 at 1M, where CTAs that wait take the place of CTAs that work.
-constexpr int kChainBelow = 1 << 15;
+// without: 19.6 and 21.0 us at 4k particles, 22.2 and 23.8 at 16k, 22.4 and 23.7 at 32k, 24.3
+// and 24.9 at 48k; 26.4 and 25.1 at 64k, 134 and 128 at 1M, where CTAs that wait take the
+// place of CTAs that work.
+constexpr int kChainBelow = 48 << 10;
 constexpr int kScatterPer = 4;  // particles per thread of the counting-sort scatter
 // Particle bricks of at least this many particles come first in the active list,
 // so the persistent transfer kernels end on small bricks (a shorter tail)
@@ -82,7 +83,7 @@ constexpr int kBigBrick = 256;
 
 cudaError_t launch_prepare(const StepArgs& a, const PState& st, cudaStream_t s);
 // zero the brick histogram, the tile counts and the list sizes (all scenes)
-cudaError_t launch_reset_histogram(const SortBufs& sb, int bricks, int tiles, cudaStream_t s);
+cudaError_t launch_reset_histogram(const SortBufs& sb, int bricks, int tiles, int np, cudaStream_t s);
 // the scan alone serves launches that bring a permutation of their own
 cudaError_t launch_scan(const StepArgs& a, cudaStream_t s);
 cudaError_t launch_sort(const StepArgs& a, cudaStream_t s);

@@ -69,6 +69,32 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsig
     return false;
 }
 
+// Small launches of the substep chain are made programmatic: a kernel's CTAs come up
+// while the one before it still runs, and wait here for its end and its writes (every
+// thread, before its first access); the next kernel may come up at once.  Elsewhere both
+// do nothing.
+__device__ __forceinline__ void chain_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... P, class... A>
+void launch_chain(int np, void (*k)(P...), int ctas, int threads, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute programmatic;
+    programmatic.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    programmatic.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &programmatic;
+    cfg.numAttrs = np < kChainBelow ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 constexpr unsigned kFull = 0xffffffffu;
 
 // ----------------------------------------------------- brick key + rank
