@@ -171,6 +171,7 @@ StepArgs step_args(mpm_ctx* c, float dt, int s0, int s1, const PState& in, const
     a.sb = c->sb;
     a.scenes = c->d_scenes;
     a.rigids = c->d_rigids;
+    a.pose = c->d_pose;
     a.impulse = c->d_impulse;
     a.t_scene = c->d_time;
     a.epoch = c->d_epoch;
@@ -452,6 +453,7 @@ extern "C" int mpm_create(const mpm_config* cfg, void* stream, mpm_ctx** out)
     alloc((void**)&c->d_scenes, sizeof(SceneDev) * c->n_scenes);
     alloc((void**)&c->d_rigids, sizeof(RigidDev) * c->n_scenes * kMaxRigids);
     alloc((void**)&c->d_inv, sizeof(int) * c->cap);
+    alloc((void**)&c->d_pose, sizeof(RigidPose) * c->n_scenes * kMaxRigids);
     size_t zero = 0, total = 0;
     for (size_t i = 0; i < parts.size(); ++i) {
         total += parts[i].bytes;

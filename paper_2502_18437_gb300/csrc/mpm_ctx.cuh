@@ -37,6 +37,7 @@ struct mpm_ctx {
     int* brick_epoch = nullptr;
     mpm::SceneDev* d_scenes = nullptr;
     mpm::RigidDev* d_rigids = nullptr;
+    mpm::RigidPose* d_pose = nullptr;
     double* d_impulse = nullptr;
     unsigned* d_err = nullptr;
     double* d_time = nullptr;

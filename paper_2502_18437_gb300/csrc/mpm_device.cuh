@@ -60,8 +60,7 @@ __device__ __forceinline__ void brick_coords(int nb, int nb_log2, int lb, int& b
 constexpr int kMaxTris = MPM_MAX_MESH_TRIANGLES;
 constexpr int kMaxSpine = MPM_MAX_SPINE_POINTS;
 
-// Shape data shared by the device copy and the staged pose: segment points or
-// mesh vertices (body frame) and the mesh's triangles and spine polyline.
+// Shape data: segment points or mesh vertices (body frame) and the mesh's triangles and spine polyline.
 struct RigidShape {
     float pts[kMaxPts * 3];
     unsigned char tris[kMaxTris * 3];  // vertex indices (< kMaxPts)
@@ -81,15 +80,9 @@ struct RigidDev {
     RigidShape shape;
 };
 
-// Pose of a rigid at the current scene time, staged in shared memory.
-struct RigidCur {
-    int type, n_pts, n_tris, n_spine;
-    float c[3], R[9], vel[3], omega[3];
-    float mu_k, c_d, margin, radius;
-    float half[3];
-    float thickness, spine_radius;
-    float lo[3], hi[3];
-    RigidShape shape;
+// Pose of a rigid at the scene's clock: centre and rotation matrix.
+struct RigidPose {
+    float c[3], R[9];
 };
 
 // Pose of a solid rigid (sphere, box) at the end of the substep, for the
@@ -146,16 +139,6 @@ __device__ __forceinline__ void load_v(const PState& s, size_t cap, int p, float
 }
 
 // C and, in t6, the stored stress
-__device__ __forceinline__ void load_C_tau(const PState& s, size_t cap, int p, float C[9], float t6[6])
-{
-    const float4 a = plane(s, cap, 4, p), b = plane(s, cap, 5, p), c = plane(s, cap, 6, p), d = plane(s, cap, 7, p);
-    C[0] = a.x; C[1] = a.y; C[2] = a.z; C[3] = a.w;
-    C[4] = b.x; C[5] = b.y; C[6] = b.z; C[7] = b.w;
-    C[8] = c.x;
-    t6[0] = c.y; t6[1] = c.z; t6[2] = c.w;
-    t6[3] = d.x; t6[4] = d.y; t6[5] = d.z;
-}
-
 __device__ __forceinline__ void load_C(const PState& s, size_t cap, int p, float C[9])
 {
     const float4 a = plane(s, cap, 4, p), b = plane(s, cap, 5, p);
@@ -169,9 +152,7 @@ enum {
     CTR_LAST_ACT = 0,  // active particle bricks and node bricks of the last finished substep
     CTR_LAST_NACT = 1,
     CTR_DONE_G2P = 2,  // CTAs of the G2P launch that have finished (the last one advances the clocks)
-    CTR_WORK_P2G = 3,  // dynamic work counters of the persistent kernels
-    CTR_WORK_GRID = 4,
-    CTR_WORK_G2P = 5,
+    CTR_WORK_G2P = 5,  // dynamic work counter of the fused kernel
     CTR_N_BIG = 6,     // active particle bricks of at least kBigBrick particles
     CTR_N_SMALL = 7,   // the other active particle bricks
     CTR_N_NACT = 8,    // active node bricks

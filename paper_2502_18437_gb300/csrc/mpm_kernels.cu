@@ -69,11 +69,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(StepArgs a)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const SortBufs& sb = a.sb;
     const int tile = a.r.t0 + blockIdx.x;
-    if (blockIdx.x == 0 && tid == 0) {
-        sb.counters[CTR_WORK_P2G] = 0;
-        sb.counters[CTR_WORK_GRID] = 0;
-        sb.counters[CTR_WORK_G2P] = 0;
-    }
+    if (blockIdx.x == 0 && tid == 0) sb.counters[CTR_WORK_G2P] = 0;
     // scene of the tile
     int s = a.r.s0;
     if (a.r.s1 - a.r.s0 > 1) {
@@ -85,6 +81,11 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(StepArgs a)
         }
     }
     const SceneDev& sc = a.scenes[s];
+    if (a.any_rigid && tile == sc.tile_base && tid < sc.n_rigid) {
+        // the rigids' poses at the scene's clock, for the grid update
+        RigidPose& P = a.pose[s * kMaxRigids + tid];
+        rigid_pose_at(a.rigids[s * kMaxRigids + tid], a.t_scene[s], P.c, P.R);
+    }
     const int nb = sc.nb, bricks = nb * nb * nb;
     const int l0 = (tile - sc.tile_base) << sb.tile_shift, l1 = min(l0 + (1 << sb.tile_shift), bricks);
     // particles of the tiles before this one, of the whole range, and of the tiles
@@ -527,7 +528,7 @@ __device__ __forceinline__ float closest_on_triangle_f(float p0, float p1, float
 
 // Region of the triangle-mesh slicer at body point p (3 sticky spine, 1
 // regular, 0 none) and its body-frame normal nl.
-__device__ __forceinline__ int mesh_slicer_region(const RigidCur& R, float p0, float p1, float p2, float nl[3])
+__device__ __forceinline__ int mesh_slicer_region(const RigidDev& R, float p0, float p1, float p2, float nl[3])
 {
     float dsp = 3.4e38f;
     for (int k = 0; k + 1 < R.n_spine; ++k) {
@@ -573,13 +574,13 @@ __device__ __forceinline__ int mesh_slicer_region(const RigidCur& R, float p0, f
 // EXT: the launch has arcs or mesh slicers (a separate instance of the grid
 // kernel, so that the common shapes keep their registers).
 template <bool EXT>
-__device__ int rigid_region(const RigidCur& R, float3 x, float3& n, float3& t)
+__device__ int rigid_region(const RigidDev& R, const RigidPose& P, float3 x, float3& n, float3& t)
 {
-    const float dx0 = x.x - R.c[0], dx1 = x.y - R.c[1], dx2 = x.z - R.c[2];
+    const float dx0 = x.x - P.c[0], dx1 = x.y - P.c[1], dx2 = x.z - P.c[2];
     // body coordinates p = R^T (x - c)
-    const float p0 = R.R[0] * dx0 + R.R[3] * dx1 + R.R[6] * dx2;
-    const float p1 = R.R[1] * dx0 + R.R[4] * dx1 + R.R[7] * dx2;
-    const float p2 = R.R[2] * dx0 + R.R[5] * dx1 + R.R[8] * dx2;
+    const float p0 = P.R[0] * dx0 + P.R[3] * dx1 + P.R[6] * dx2;
+    const float p1 = P.R[1] * dx0 + P.R[4] * dx1 + P.R[7] * dx2;
+    const float p2 = P.R[2] * dx0 + P.R[5] * dx1 + P.R[8] * dx2;
     float nl0 = 0.f, nl1 = 0.f, nl2 = 0.f, tl0 = 0.f, tl1 = 0.f, tl2 = 0.f;
     int code = 0;
     // a thread's segments (or a mesh's triangles) are looked at by the nodes near it only:
@@ -684,10 +685,10 @@ __device__ int rigid_region(const RigidCur& R, float3 x, float3& n, float3& t)
             if (L > 0.f) { tl0 = e0 / L; tl1 = e1 / L; tl2 = e2 / L; }
         }
     }
-    n = f3(R.R[0] * nl0 + R.R[1] * nl1 + R.R[2] * nl2, R.R[3] * nl0 + R.R[4] * nl1 + R.R[5] * nl2,
-           R.R[6] * nl0 + R.R[7] * nl1 + R.R[8] * nl2);
-    t = f3(R.R[0] * tl0 + R.R[1] * tl1 + R.R[2] * tl2, R.R[3] * tl0 + R.R[4] * tl1 + R.R[5] * tl2,
-           R.R[6] * tl0 + R.R[7] * tl1 + R.R[8] * tl2);
+    n = f3(P.R[0] * nl0 + P.R[1] * nl1 + P.R[2] * nl2, P.R[3] * nl0 + P.R[4] * nl1 + P.R[5] * nl2,
+           P.R[6] * nl0 + P.R[7] * nl1 + P.R[8] * nl2);
+    t = f3(P.R[0] * tl0 + P.R[1] * tl1 + P.R[2] * tl2, P.R[3] * tl0 + P.R[4] * tl1 + P.R[5] * tl2,
+           P.R[6] * tl0 + P.R[7] * tl1 + P.R[8] * tl2);
     return code;
 }
 
@@ -696,12 +697,12 @@ __device__ int rigid_region(const RigidCur& R, float3 x, float3& n, float3& t)
 // with v_t the tangential part (regular) or the part along the 1D tangent.
 // Returns whether the node was changed; dp = node momentum change.
 template <bool EXT>
-__device__ bool rigid_contact(const RigidCur& R, float3 x, float m, float3& v, float3& dp)
+__device__ bool rigid_contact(const RigidDev& R, const RigidPose& P, float3 x, float m, float3& v, float3& dp)
 {
     float3 n, t;
-    const int code = rigid_region<EXT>(R, x, n, t);
+    const int code = rigid_region<EXT>(R, P, x, n, t);
     if (code == 0) return false;
-    const float r0 = x.x - R.c[0], r1 = x.y - R.c[1], r2 = x.z - R.c[2];
+    const float r0 = x.x - P.c[0], r1 = x.y - P.c[1], r2 = x.z - P.c[2];
     const float vr0 = R.vel[0] + R.omega[1] * r2 - R.omega[2] * r1;
     const float vr1 = R.vel[1] + R.omega[2] * r0 - R.omega[0] * r2;
     const float vr2 = R.vel[2] + R.omega[0] * r1 - R.omega[1] * r0;
@@ -729,60 +730,16 @@ __device__ bool rigid_contact(const RigidCur& R, float3 x, float m, float3& v, f
     return true;
 }
 
-__device__ void stage_rigid(const RigidDev& src, double t_now, RigidCur& dst)
-{
-    dst.type = src.type;
-    dst.n_pts = src.n_pts;
-    dst.n_tris = src.n_tris;
-    dst.n_spine = src.n_spine;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        dst.vel[i] = src.vel[i];
-        dst.omega[i] = src.omega[i];
-        dst.half[i] = src.half[i];
-        dst.lo[i] = src.lo[i];
-        dst.hi[i] = src.hi[i];
-    }
-    rigid_pose_at(src, t_now, dst.c, dst.R);
-    dst.mu_k = src.mu_k;
-    dst.c_d = src.c_d;
-    dst.margin = src.margin;
-    dst.radius = src.radius;
-    dst.thickness = src.thickness;
-    dst.spine_radius = src.spine_radius;
-}
-
 constexpr int kGridThreads = 256;  // 4 node bricks per iteration
 
-__device__ void flush_impulse(const StepArgs& a, const float* simp, int scene, int nr, int tid)
-{
-    for (int t = tid; t < nr * 6; t += kGridThreads)
-        if (simp[t] != 0.f) atomicAdd(&a.impulse[scene * kMaxRigids * 6 + t], (double)simp[t]);
-}
-
-// The scene's nr rigids at its clock, with their shapes, and empty impulse sums.
-__device__ __forceinline__ void stage_scene(const StepArgs& a, int scene, int nr, RigidCur* rig, float* simp, int tid)
-{
-    const double t_now = a.t_scene[scene];
-    if (tid < nr) stage_rigid(a.rigids[scene * kMaxRigids + tid], t_now, rig[tid]);
-    constexpr int kShapeWords = (int)(sizeof(RigidShape) / sizeof(int));
-    static_assert(sizeof(RigidShape) % sizeof(int) == 0, "shape copied in words");
-    for (int t = tid; t < nr * kShapeWords; t += kGridThreads) {
-        const int r = t / kShapeWords, k = t % kShapeWords;
-        reinterpret_cast<int*>(&rig[r].shape)[k] = reinterpret_cast<const int*>(&a.rigids[scene * kMaxRigids + r].shape)[k];
-    }
-    for (int t = tid; t < kMaxRigids * 6; t += kGridThreads) simp[t] = 0.f;
-}
-
-// Grid update of the active node bricks: 64 threads per brick, one node each.
-// Rigids of a scene are staged in shared memory (posed at the scene's clock).
-// Grid update of node nid of node brick B (Eq. 3, contact, walls), clearing
-// the P2G accumulator; rigid impulses are summed into simp (shared).
-// The node's P2G accumulator is reset afterwards by k_grid_clear: loading and
-// clearing the freshly reduced lines in one kernel measured far slower.
+// Grid update of node nid of node brick B (Eq. 3, contact, walls) against the scene's nr
+// rigids, at the poses that the scan left; each warp adds its momentum to the rigids'
+// impulses.  64 threads per brick, one node each.
+// The node's P2G accumulator is reset later: loading and clearing the freshly reduced lines
+// in one kernel measured far slower.
 template <bool EXT>
-__device__ __forceinline__ void grid_node(const StepArgs& a, int B, int scene, int nid, int lane, const RigidCur* rig,
-                                          int nr, float* simp)
+__device__ __forceinline__ void grid_node(const StepArgs& a, int B, int scene, int nid, int lane, const RigidDev* rig,
+                                          const RigidPose* pose, int nr)
 {
     const SceneDev sc = a.scenes[scene];
     const int n = sc.n, lb = B - sc.brick_base;
@@ -802,7 +759,7 @@ __device__ __forceinline__ void grid_node(const StepArgs& a, int B, int scene, i
         const float3 xI = f3(gi * dxs, gj * dxs, gk * dxs);
         for (int r = 0; r < nr; ++r) {
             float3 dp;
-            if (rigid_contact<EXT>(rig[r], xI, g.x, v, dp)) {
+            if (rigid_contact<EXT>(rig[r], pose[r], xI, g.x, v, dp)) {
                 touched |= 1u << r;
                 dpr[r][0] = dp.x; dpr[r][1] = dp.y; dpr[r][2] = dp.z;
             }
@@ -833,7 +790,7 @@ __device__ __forceinline__ void grid_node(const StepArgs& a, int B, int scene, i
         float val[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         if (on) {
             const float d0 = -dpr[r][0], d1 = -dpr[r][1], d2 = -dpr[r][2];
-            const float r0 = gi * dxs - rig[r].c[0], r1 = gj * dxs - rig[r].c[1], r2 = gk * dxs - rig[r].c[2];
+            const float r0 = gi * dxs - pose[r].c[0], r1 = gj * dxs - pose[r].c[1], r2 = gk * dxs - pose[r].c[2];
             val[0] = d0; val[1] = d1; val[2] = d2;
             val[3] = r1 * d2 - r2 * d1;
             val[4] = r2 * d0 - r0 * d2;
@@ -844,7 +801,7 @@ __device__ __forceinline__ void grid_node(const StepArgs& a, int B, int scene, i
             float x = val[c];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
-            if (lane == 0) atomicAdd(&simp[r * 6 + c], x);
+            if (lane == 0 && x != 0.f) atomicAdd(&a.impulse[(scene * kMaxRigids + r) * 6 + c], (double)x);
         }
     }
 }
@@ -860,7 +817,7 @@ __global__ void __launch_bounds__(kGridThreads, 8) k_grid_plain(StepArgs a)
     for (int base = blockIdx.x * 4; base < n_nact; base += gridDim.x * 4) {
         const int item = base + grp;
         if (item < n_nact)
-            grid_node<false>(a, a.sb.nact_brick[item], a.sb.nact_scene[item], nid, lane, nullptr, 0, nullptr);
+            grid_node<false>(a, a.sb.nact_brick[item], a.sb.nact_scene[item], nid, lane, nullptr, nullptr, 0);
     }
 }
 
@@ -884,101 +841,41 @@ __global__ void __launch_bounds__(kGridThreads, 8) k_grid_clear(StepArgs a)
     }
 }
 
+// One scene's rigids are staged in shared memory (a thread's segments are walked over and
+// over: slab_256k 53.4 us a substep staged, 54.8 not).  Those of many scenes are read
+// where they are, by uniform loads that stay in L1: staged scene by scene, with a table of
+// the CTA's bricks and barriers at each change - bricks come interleaved by scan tile - a
+// substep of 256 scenes with their blades took 377 us, so 352.
 template <bool EXT>
 __global__ void __launch_bounds__(kGridThreads, 4) k_grid(StepArgs a)
 {
+    __shared__ RigidDev s_rig[kMaxRigids];
+    __shared__ RigidPose s_pose[kMaxRigids];
     chain_wait();
-    __shared__ RigidCur rig[kMaxRigids];
-    __shared__ float simp[kMaxRigids * 6];
-    // per brick of a chunk of the list: node brick, scene, the scene's rigid count
-    __shared__ int s_brk[kGridThreads], s_scn[kGridThreads], s_nr[kGridThreads];
-    __shared__ int s_scene[4];
-    __shared__ int s_staged, s_nrig, s_target;
     const int tid = threadIdx.x, lane = tid & 31, grp = tid >> 6, nid = tid & 63;
     const int n_nact = a.sb.counters[CTR_N_NACT];
     if (a.r.s1 - a.r.s0 == 1) {
-        // one scene: its rigids are staged at once, and every CTA takes bricks in turn (no
-        // table of scenes and its barriers: 1 to 2 us of a substep)
         const int nr = a.scenes[a.r.s0].n_rigid;
-        stage_scene(a, a.r.s0, nr, rig, simp, tid);
+        static_assert(sizeof(RigidDev) % sizeof(int) == 0 && sizeof(RigidPose) % sizeof(int) == 0, "copied in words");
+        const int* rig = reinterpret_cast<const int*>(a.rigids + a.r.s0 * kMaxRigids);
+        const int* pose = reinterpret_cast<const int*>(a.pose + a.r.s0 * kMaxRigids);
+        for (int t = tid; t < nr * (int)(sizeof(RigidDev) / sizeof(int)); t += kGridThreads) reinterpret_cast<int*>(s_rig)[t] = rig[t];
+        for (int t = tid; t < nr * (int)(sizeof(RigidPose) / sizeof(int)); t += kGridThreads)
+            reinterpret_cast<int*>(s_pose)[t] = pose[t];
         __syncthreads();
         for (int base = blockIdx.x * 4; base < n_nact; base += gridDim.x * 4) {
             const int item = base + grp;
-            if (item < n_nact) grid_node<EXT>(a, a.sb.nact_brick[item], a.r.s0, nid, lane, rig, nr, simp);
+            if (item < n_nact) grid_node<EXT>(a, a.sb.nact_brick[item], a.r.s0, nid, lane, s_rig, s_pose, nr);
         }
-        __syncthreads();
-        flush_impulse(a, simp, a.r.s0, nr, tid);
         return;
     }
-    if (tid == 0) { s_staged = -1; s_nrig = 0; }
-    // each CTA takes a contiguous run of the node-brick list (scenes are contiguous
-    // in it), so that it stages a scene's rigids and flushes their impulses about
-    // once; groups of 4 bricks of the staged scene (or of scenes without rigids)
-    // then run without barriers
-    const int per = ((n_nact + gridDim.x - 1) / gridDim.x + 3) & ~3;
-    const int first = blockIdx.x * per, last = min(first + per, n_nact);
-    for (int c0 = first; c0 < last; c0 += kGridThreads) {
-        const int c1 = min(c0 + kGridThreads, last);
-        __syncthreads();  // the previous chunk's table is no longer read
-        if (c0 + tid < c1) {
-            const int sc = a.sb.nact_scene[c0 + tid];
-            s_brk[tid] = a.sb.nact_brick[c0 + tid];
-            s_scn[tid] = sc;
-            s_nr[tid] = a.scenes[sc].n_rigid;
-        }
-        __syncthreads();
-        for (int base = c0; base < c1; base += 4) {
-            const int item = base + grp;
-            const int my_scene = item < c1 ? s_scn[item - c0] : -1;
-            const int gl = min(base + 3, c1 - 1) - c0;
-            bool no_rigid = true, staged = true;
-            for (int g = base - c0; g <= gl; ++g) {
-                no_rigid = no_rigid && s_nr[g] == 0;
-                staged = staged && s_scn[g] == s_staged;
-            }
-            const int my_brick = my_scene >= 0 ? s_brk[item - c0] : 0;
-            if (no_rigid) {
-                if (my_scene >= 0) grid_node<EXT>(a, my_brick, my_scene, nid, lane, nullptr, 0, nullptr);
-                continue;
-            }
-            if (staged) {
-                if (my_scene >= 0) grid_node<EXT>(a, my_brick, my_scene, nid, lane, rig, s_nrig, simp);
-                continue;
-            }
-            if (nid == 0) s_scene[grp] = my_scene;
-            bool done = my_scene < 0;
-            __syncthreads();
-            for (;;) {
-                // next scene to process among the 4 bricks (usually all the same)
-                if (tid == 0) {
-                    int t = -1;
-                    for (int g = 0; g < 4; ++g)
-                        if (s_scene[g] >= 0 && (t < 0 || s_scene[g] < t)) t = s_scene[g];
-                    s_target = t;
-                }
-                __syncthreads();
-                const int target = s_target;
-                if (target < 0) break;
-                if (target != s_staged) {
-                    if (s_staged >= 0) flush_impulse(a, simp, s_staged, s_nrig, tid);
-                    __syncthreads();
-                    const int nr = a.scenes[target].n_rigid;
-                    stage_scene(a, target, nr, rig, simp, tid);
-                    if (tid == 0) { s_staged = target; s_nrig = nr; }
-                    __syncthreads();
-                }
-                if (!done && my_scene == target) {
-                    done = true;
-                    grid_node<EXT>(a, my_brick, target, nid, lane, rig, s_nrig, simp);
-                }
-                __syncthreads();
-                if (nid == 0 && my_scene == target) s_scene[grp] = -1;
-                __syncthreads();
-            }
-        }
+    for (int base = blockIdx.x * 4; base < n_nact; base += gridDim.x * 4) {
+        const int item = base + grp;
+        if (item >= n_nact) continue;
+        const int scene = a.sb.nact_scene[item];
+        grid_node<EXT>(a, a.sb.nact_brick[item], scene, nid, lane, a.rigids + scene * kMaxRigids, a.pose + scene * kMaxRigids,
+                       a.scenes[scene].n_rigid);
     }
-    __syncthreads();
-    if (s_staged >= 0) flush_impulse(a, simp, s_staged, s_nrig, tid);
 }
 
 // ------------------------------------------------------------------ G2P

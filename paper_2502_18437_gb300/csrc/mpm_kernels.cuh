@@ -38,6 +38,7 @@ struct StepArgs {
     SortBufs sb;
     const SceneDev* scenes;
     const RigidDev* rigids;      // [n_scenes * kMaxRigids]
+    RigidPose* pose;             // [n_scenes * kMaxRigids] at the scenes' clocks, by the scan
     double* impulse;             // [n_scenes * kMaxRigids * 6]
     double* t_scene;             // [n_scenes] scene clocks
     int* epoch;                  // [n_scenes] substep counters
@@ -102,8 +103,6 @@ int occupancy_grid_plain();
 cudaError_t launch_init_particles(const PState& st, int cap, int p_at, int n, int id0, const float* x,
                                   const float* v, const float* E, const float* nu, float E0, float nu0,
                                   cudaStream_t s);
-cudaError_t launch_permute_to_id(const PState& src, const PState& dst, int cap, int p0, int np,
-                                 cudaStream_t s);
 // x, v, C, F (null: not moved) of one scene as arrays in particle-id order
 struct Fields {
     float* f[4];
