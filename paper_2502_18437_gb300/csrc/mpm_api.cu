@@ -376,7 +376,7 @@ extern "C" int mpm_create(const mpm_config* cfg, void* stream, mpm_ctx** out)
     if (bricks * 64 >= ((long long)1 << 31)) { delete c; return MPM_ERR_INVALID_ARGUMENT; }
     c->brick_base[c->n_scenes] = (int)bricks;
     c->total_bricks = (int)bricks;
-    // scan tiles: 2^shift bricks of one scene, at least 256; wider tiles keep
+    // scan tiles: 2^shift bricks of one scene, at least 64; wider tiles keep
     // the number of tiles (whose counts every scan CTA adds up) near 2048 or less
     {
         int shift = kMinTileShift;

@@ -71,7 +71,11 @@ constexpr int kStateFloats = 34;  // eight float4 planes, mu, lam
 constexpr int kP2GThreads = 192;  // six warps, each with slots of its own
 constexpr int kP2GMaxSlots = 64;
 constexpr int kScanThreads = 256;
-constexpr int kMinTileShift = 8;  // a scan tile holds at least kScanThreads bricks
+// A scan tile holds 64 bricks or more: its CTA also turns the cells' counts of its particle
+// bricks into first slots, a warp a brick, which is what takes long.  With 256 bricks or more
+// a substep took 127.5 us on the 1M block (now 118.0: tiles of 128, see mpm_create), 33.2 with
+// the indenter at 100k (31.7), 22.1 at 16k (20.9).
+constexpr int kMinTileShift = 6;
 // Launches of fewer particles are made programmatic (launch_chain).  A substep with and
 // without: 19.6 and 21.0 us at 4k particles, 22.2 and 23.8 at 16k, 22.4 and 23.7 at 32k, 24.3
 // and 24.9 at 48k; 26.4 and 25.1 at 64k, 134 and 128 at 1M, where CTAs that wait take the
