@@ -318,9 +318,9 @@ __global__ void __launch_bounds__(256) k_prepare(StepArgs a, PState st)
 // batch ahead.  Before, a CTA took a brick: ranks in its cells, work items, staged item
 // sums and a 6^3 window, one behind the other with a barrier between: 35.7 M
 // instructions, 13.5 us for a lone brick and so 66 us for the 1M block's 2,744 and 19 us
-// for 64k particles.  Now 49 us and 6 us; PB-MPM's cycles at 131k 39 -> 17 us; the
-// standard MPM at 131k, which took shared-memory atomics, 97 -> 13 us.  The bricks' cell
-// counts come from G2P, so that the sort orders the slots by cell.
+// for 64k particles.  Now 43 and 8.5 us, 5.9 us at 4k; PB-MPM's cycles at 131k 39 -> 16 us.
+// The standard MPM's took shared-memory atomics, 97 us at 131k; now its whole substep
+// takes 41 us.
 // Joining halves the reductions, and with them the error of the sums: C of a falling 64k
 // block is 4.8e-6 off after 25 substeps, as before; without, 5.4e-6.
 // Tried: a lane per node column (j, k), three groups of lanes at a third of the chunk
