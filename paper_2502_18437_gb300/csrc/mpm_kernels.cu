@@ -1301,7 +1301,8 @@ __global__ void __launch_bounds__(kVcThreads) k_g2p_vc(StepArgs a)
 // ------------------------------------------------------- state I/O kernels
 //
 // x, v, C and F of one scene as arrays in particle-id order (null: not moved), all
-// fields in one pass over the planes.  Particle ids are in no order by slot, so one side
+// fields in one pass over the planes; a slot whose id is not of the scene (a substep that
+// a device error cut short wrote none) is left out.  Particle ids are in no order by slot, so one side
 // is scattered over HBM, and the sectors it half uses are the cost: one kernel a field
 // took 105 us to write 1M particles' state and 255 us to read it, now 75 and 133 us;
 // writing through records in id order instead, 177 us.
@@ -1424,9 +1425,8 @@ __global__ void __launch_bounds__(kIoBlock) k_arrays_by_slot(PState st, int cap,
         const int k = f < 2 ? 3 : 9;
 #pragma unroll
         for (int i = 0; i < k; ++i) {
-            const int at = i * 32 + lane, particle = at / k;
-            float* a = h.f[f] + (size_t)__shfl_sync(kFull, id, particle) * k + (at - particle * k);
-            if (particle < cnt) *a = first[f][at];
+            const int at = i * 32 + lane, particle = at / k, to = __shfl_sync(kFull, id, particle);
+            if (particle < cnt && (unsigned)to < (unsigned)np) h.f[f][(size_t)to * k + (at - particle * k)] = first[f][at];
         }
     }
 }
@@ -1436,6 +1436,7 @@ __global__ void __launch_bounds__(kIoBlock) k_state_by_slot(PState st, int cap, 
     const int g = blockIdx.x * kIoBlock + threadIdx.x;
     if (g >= np) return;
     const int s = p0 + g, id = state_id(st, s);
+    if ((unsigned)id >= (unsigned)np) return;
     const size_t i = id;
     fields_to_planes(st, cap, s, id, h.f[0] ? h.f[0] + 3 * i : nullptr, h.f[1] ? h.f[1] + 3 * i : nullptr,
                      h.f[2] ? h.f[2] + 9 * i : nullptr, h.f[3] ? h.f[3] + 9 * i : nullptr);
@@ -1683,7 +1684,9 @@ cudaError_t launch_fields(const PState& st, const PState& spare, int cap, int p0
                           bool host, cudaStream_t s)
 {
     if (np == 0) return cudaSuccess;
-    float4* rec = spare.q;
+    // the records (whole sectors) leave plane 0 alone: a substep that a device error skipped
+    // leaves the spare buffer unwritten and current, and its ids are indexes
+    float4* rec = spare.q + (((size_t)cap + 1) & ~(size_t)1);
     if (out && (host || np >= kIoByIdFrom)) {
         k_pack<<<n_blocks(np, kIoBlock), kIoBlock, 0, s>>>(st, cap, p0, np, inv, rec);
         k_fields_by_id<true><<<n_blocks(np, kIoBlock), kIoBlock, 0, s>>>(st, cap, p0, np, inv, rec, h);

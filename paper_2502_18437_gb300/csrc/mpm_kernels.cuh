@@ -116,7 +116,7 @@ struct Fields {
 // 262k, 133 and 219 at 1M, 485 and 1,306 at 4M.
 constexpr int kIoByIdFrom = 1 << 17;
 // state -> arrays (out) or arrays -> state; inv: scratch of np ints, spare: the state's other
-// buffer (scratch); host: the arrays are pinned host memory
+// buffer (all but its plane 0 is scratch); host: the arrays are pinned host memory
 cudaError_t launch_fields(const PState& st, const PState& spare, int cap, int p0, int np, int* inv, const Fields& h, bool out,
                           bool host, cudaStream_t s);
 cudaError_t launch_order(const PState& st, int p0, int np, int* dst, cudaStream_t s);  // ids by slot
