@@ -314,7 +314,9 @@ int mpm_tape_begin(mpm_ctx* ctx);
  * initial velocities at mpm_tape_begin.  Rigids and walls in contact are
  * differentiated as the masks they apply (the contact law's friction branch
  * is not differentiated: backward returns STATE if any scene has a rigid).
- * Blocks until done (bounded).  Errors: INVALID_ARGUMENT, STATE, TIMEOUT, CUDA. */
+ * Blocks until done (bounded).  After MPM_EBIT_TIMEOUT or MPM_EBIT_INTERNAL, which
+ * leave a substep undone, nothing is run and that error returned.
+ * Errors: INVALID_ARGUMENT, STATE, TIMEOUT, INTERNAL, CUDA. */
 int mpm_backward(mpm_ctx* ctx, const float* dL_dx, const float* dL_dv, float* dL_dE,
                  float* dL_dnu, float* dL_dv0, int mem);
 

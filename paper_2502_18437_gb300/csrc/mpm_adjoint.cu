@@ -638,6 +638,14 @@ static int backward_device(mpm_ctx* c, const SeedIn& seeds, const AdjOut& outs)
     if ((st = wait_stream(c))) return st;  // bounded; the copies below then complete at once
     MPM_CKA(cudaMemcpy(t_save.data(), c->d_time, sizeof(double) * c->n_scenes, cudaMemcpyDeviceToHost));
     MPM_CKA(cudaMemcpy(e_save.data(), c->d_epoch, sizeof(int) * c->n_scenes, cudaMemcpyDeviceToHost));
+    // a substep that a device error cut short left slots, and the permutation recorded for it,
+    // unwritten: there is nothing to reverse, and both hold indexes
+    std::vector<unsigned> err(c->n_scenes);
+    MPM_CKA(cudaMemcpy(err.data(), c->d_err, sizeof(unsigned) * c->n_scenes, cudaMemcpyDeviceToHost));
+    for (const unsigned bits : err) {
+        if (bits & MPM_EBIT_TIMEOUT) return MPM_ERR_TIMEOUT;
+        if (bits & MPM_EBIT_INTERNAL) return MPM_ERR_INTERNAL;
+    }
 
     AdjState adj[2] = {adj_view(t->adj, c->cap), adj_view(t->adj + 24 * cap, c->cap)};
     int nxt = 0;

@@ -123,3 +123,20 @@ def test_state_after_a_skipped_substep_keeps_its_ids():
             x, order = (np.asarray(out[f].cpu() if device else out[f]) for f in ("x", "order"))
             assert np.array_equal(np.sort(order), np.arange(len(order)))
             assert np.array_equal(x, older)
+
+
+def test_backward_refuses_a_tape_with_a_skipped_substep():
+    sc = W.elastic_cube(n_side=9)
+    with mpm.from_workload(sc, tape_checkpoint_every=2, tape_max_substeps=4) as sim:
+        sim.tape_begin()
+        sim.substep(sc["dt"], 2)
+        ones = np.ones((len(sc["x"]), 3), np.float32)
+        dE, dnu, dv0 = sim.backward(ones, ones)
+        assert np.abs(dv0).max() > 0
+        sim.substep(sc["dt"], 1)  # (the counts are made anew after a reverse pass)
+        spoil_sort(sim)
+        sim.substep(sc["dt"], 1)
+        for reverse in (lambda: sim.backward(ones, ones), lambda: sim.backward_state({"v": ones})):
+            with pytest.raises(mpm.MPMError) as e:
+                reverse()
+            assert e.value.status == -10
