@@ -273,6 +273,7 @@ constexpr int kAdjWarps = kAdjThreads / 32;
 // One lane per slot gathers what its particle takes from the nodes and leaves a record of
 // what it gives to them; the warp then adds the records' contributions up as P2G does.
 // (One CTA per brick with shared-memory atomics, 81 per particle: 67 us for 32k particles.)
+template <bool READ_ONLY>
 __global__ void __launch_bounds__(kAdjThreads) k_g2p_adj(AdjArgs q)
 {
     chain_wait();
@@ -295,7 +296,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_g2p_adj(AdjArgs q)
     float f[3], w[9], x[3];
     load_x(a.in, p, x);
     particle_weights(x[0], x[1], x[2], n, bc, f, w);
-    const GridStencil node(a.V, sc, bc);
+    const GridStencil<READ_ONLY> node(a.V, sc, bc);
     // forward recompute of v' and C'
     float vn[3], Cn[9], A[9], qv[3];
     gather_velocity<0>(f, w, node, vn, Cn);
@@ -407,6 +408,7 @@ __global__ void __launch_bounds__(256) k_grid_adj(StepArgs a)
 
 // --------------------------------------------------------------- P2G^-1
 
+template <bool READ_ONLY>
 __global__ void __launch_bounds__(kAdjThreads) k_p2g_adj(AdjArgs q)
 {
     chain_wait();
@@ -424,7 +426,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_p2g_adj(AdjArgs q)
     float f[3], w[9], x[3];
     load_x(a.in, p, x);
     particle_weights(x[0], x[1], x[2], n, bc, f, w);
-    const GridStencil node(a.V, sc, bc);  // (P_I_bar, m_I_bar)
+    const GridStencil<READ_ONLY> node(a.V, sc, bc);  // (P_I_bar, m_I_bar)
     float P[3], Ab[9];                    // sum W P_bar, sum W P_bar d^T
     gather_velocity<0>(f, w, node, P, Ab);
 #pragma unroll
@@ -681,11 +683,13 @@ static int backward_device(mpm_ctx* c, const SeedIn& seeds, const AdjOut& outs)
             MPM_CKA(launch_grid(a, c->stream, true));
             AdjArgs q{a, adj[nxt], adj[nxt ^ 1], gmu, glam};
             const int ctas = n_blocks(std::max(N, 1), kAdjThreads);
-            launch_chain(N, k_g2p_adj, ctas, kAdjThreads, 0, c->stream, q);
+            if (N < kChainBelow) launch_chain(N, k_g2p_adj<false>, ctas, kAdjThreads, 0, c->stream, q);
+            else launch_alone(k_g2p_adj<true>, ctas, kAdjThreads, 0, c->stream, q);
             MPM_CKA(cudaGetLastError());
             launch_chain(N, k_grid_adj, c->num_sms * 8, 256, 0, c->stream, a);
             MPM_CKA(cudaGetLastError());
-            launch_chain(N, k_p2g_adj, ctas, kAdjThreads, 0, c->stream, q);
+            if (N < kChainBelow) launch_chain(N, k_p2g_adj<false>, ctas, kAdjThreads, 0, c->stream, q);
+            else launch_alone(k_p2g_adj<true>, ctas, kAdjThreads, 0, c->stream, q);
             MPM_CKA(cudaGetLastError());
             nxt ^= 1;
         }

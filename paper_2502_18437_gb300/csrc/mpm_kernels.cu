@@ -1053,7 +1053,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_g2p(StepArgs a)
             if (valid) a.sb.key[s] = key;
         };
         unsigned ebits = g2p_particle<FLAGS>(
-            a, sc, s_q[0][tid], mu, lam, [&](const int* bc) { return GridStencil(a.V, sc, bc); },
+            a, sc, s_q[0][tid], mu, lam, [&](const int* bc) { return GridStencil<(FLAGS & kG2PReadOnly) != 0>(a.V, sc, bc); },
             [&](float* F) {
                 const float4 u = s_q[1][tid], v = s_q[2][tid];
                 F[0] = u.x; F[1] = u.y; F[2] = u.z; F[3] = u.w;
@@ -1270,6 +1270,7 @@ __global__ void __launch_bounds__(kFusedThreads, 4) k_g2p2g(StepArgs a)
 
 constexpr int kVcThreads = 128;
 
+template <bool READ_ONLY>
 __global__ void __launch_bounds__(kVcThreads) k_g2p_vc(StepArgs a)
 {
     chain_wait();
@@ -1286,7 +1287,7 @@ __global__ void __launch_bounds__(kVcThreads) k_g2p_vc(StepArgs a)
     int bc[3];
     load_x(a.in, p, x);
     particle_weights(x[0], x[1], x[2], sc.n, bc, f, w);
-    gather_velocity<0>(f, w, GridStencil(a.V, sc, bc), v, B);
+    gather_velocity<0>(f, w, GridStencil<READ_ONLY>(a.V, sc, bc), v, B);
     const float c4 = 4.0f * (float)sc.n;
 #pragma unroll
     for (int i = 0; i < 9; ++i) B[i] *= c4;
@@ -1576,7 +1577,7 @@ cudaError_t prepare_kernels()
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_p2g<kP2GStd>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     // G2P of large launches keeps to the shared memory it needs: the rest is L1, which holds
     // the nodes (4M block 461 -> 449 us a substep, 256 scenes 382 -> 376)
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_g2p<128, 6, 0>, cudaFuncAttributePreferredSharedMemoryCarveout, 25);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_g2p<128, 6, kG2PReadOnly>, cudaFuncAttributePreferredSharedMemoryCarveout, 25);
     return e;
 }
 
@@ -1593,7 +1594,9 @@ cudaError_t launch_p2g(const StepArgs& a, cudaStream_t s)
 cudaError_t launch_g2p_vc(const StepArgs& a, cudaStream_t s)
 {
     if (a.r.np == 0) return cudaSuccess;
-    launch_chain(a.r.np, k_g2p_vc, n_blocks(a.r.np, kVcThreads), kVcThreads, 0, s, a);
+    const int c = n_blocks(a.r.np, kVcThreads);
+    if (a.r.np < kChainBelow) launch_chain(a.r.np, k_g2p_vc<false>, c, kVcThreads, 0, s, a);
+    else launch_alone(k_g2p_vc<true>, c, kVcThreads, 0, s, a);
     return cudaGetLastError();
 }
 
@@ -1606,38 +1609,52 @@ cudaError_t launch_grid(const StepArgs& a, cudaStream_t s, bool clear)
     return cudaGetLastError();
 }
 
+// Only the shapes that small launches take by default exist with ordinary loads too, for
+// programmatic launches (GridStencil).
 template <int FLAGS>
 static void launch_g2p_variant(const StepArgs& a, cudaStream_t s)
 {
     const int c = min(a.g2p_ctas, n_blocks(max(a.r.np, 1), a.g2p_threads));
+    constexpr int RO = FLAGS | kG2PReadOnly;
     if (a.g2p_regs64) {
         switch (a.g2p_threads) {
-        case 128: launch_chain(a.r.np, k_g2p<128, 8, FLAGS>, c, 128, 0, s, a); break;
-        case 512: launch_chain(a.r.np, k_g2p<512, 2, FLAGS>, c, 512, 0, s, a); break;
-        default: launch_chain(a.r.np, k_g2p<256, 4, FLAGS>, c, 256, 0, s, a); break;
+        case 128: launch_alone(k_g2p<128, 8, RO>, c, 128, 0, s, a); break;
+        case 512: launch_alone(k_g2p<512, 2, RO>, c, 512, 0, s, a); break;
+        default: launch_alone(k_g2p<256, 4, RO>, c, 256, 0, s, a); break;
         }
     } else {
         switch (a.g2p_threads) {
-        case 128: launch_chain(a.r.np, k_g2p<128, 6, FLAGS>, c, 128, 0, s, a); break;
-        case 512: launch_chain(a.r.np, k_g2p<512, 1, FLAGS>, c, 512, 0, s, a); break;
-        default: launch_chain(a.r.np, k_g2p<256, 3, FLAGS>, c, 256, 0, s, a); break;
+        case 128: launch_alone(k_g2p<128, 6, RO>, c, 128, 0, s, a); break;
+        case 512: launch_alone(k_g2p<512, 1, RO>, c, 512, 0, s, a); break;
+        default:
+            if (a.r.np < kChainBelow) launch_chain(a.r.np, k_g2p<256, 3, FLAGS>, c, 256, 0, s, a);
+            else launch_alone(k_g2p<256, 3, RO>, c, 256, 0, s, a);
+            break;
         }
     }
+}
+
+// The one shape of the standard-MPM and PB-MPM variants.
+template <int FLAGS>
+static void launch_g2p_128(const StepArgs& a, cudaStream_t s)
+{
+    const int c = min(a.g2p_ctas, n_blocks(max(a.r.np, 1), 128));
+    if (a.r.np < kChainBelow) launch_chain(a.r.np, k_g2p<128, 6, FLAGS>, c, 128, 0, s, a);
+    else launch_alone(k_g2p<128, 6, FLAGS | kG2PReadOnly>, c, 128, 0, s, a);
 }
 
 // The standard-MPM and PB-MPM variants exist in one launch shape only (128
 // threads, 80 registers): the MLS-MPM shapes are what the tuner explores.
 cudaError_t launch_g2p(const StepArgs& a, cudaStream_t s)
 {
-    const int c = min(a.g2p_ctas, n_blocks(max(a.r.np, 1), 128));
     // the push-out variant only where a scene has a solid shape: blades, needles and
     // segments push nothing out
     if (a.solver == MPM_SOLVER_STANDARD) {
-        if (a.any_solid) launch_chain(a.r.np, k_g2p<128, 6, kG2PStdGrad | kG2PSolids>, c, 128, 0, s, a);
-        else launch_chain(a.r.np, k_g2p<128, 6, kG2PStdGrad>, c, 128, 0, s, a);
+        if (a.any_solid) launch_g2p_128<kG2PStdGrad | kG2PSolids>(a, s);
+        else launch_g2p_128<kG2PStdGrad>(a, s);
     } else if (a.solver == MPM_SOLVER_PB) {
-        if (a.any_solid) launch_chain(a.r.np, k_g2p<128, 6, kG2PNoStress | kG2PSolids>, c, 128, 0, s, a);
-        else launch_chain(a.r.np, k_g2p<128, 6, kG2PNoStress>, c, 128, 0, s, a);
+        if (a.any_solid) launch_g2p_128<kG2PNoStress | kG2PSolids>(a, s);
+        else launch_g2p_128<kG2PNoStress>(a, s);
     } else if (a.any_solid) {
         launch_g2p_variant<kG2PSolids>(a, s);
     } else {
@@ -1736,13 +1753,13 @@ int occupancy_g2p(int threads, int regs64)
     // shared memory; its occupancy bounds both
     int b = 0;
     if (regs64) {
-        if (threads == 128) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<128, 8, kG2PSolids>, 128, 0);
-        else if (threads == 512) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<512, 2, kG2PSolids>, 512, 0);
-        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<256, 4, kG2PSolids>, 256, 0);
+        if (threads == 128) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<128, 8, kG2PSolids | kG2PReadOnly>, 128, 0);
+        else if (threads == 512) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<512, 2, kG2PSolids | kG2PReadOnly>, 512, 0);
+        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<256, 4, kG2PSolids | kG2PReadOnly>, 256, 0);
     } else {
-        if (threads == 128) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<128, 6, kG2PSolids>, 128, 0);
-        else if (threads == 512) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<512, 1, kG2PSolids>, 512, 0);
-        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<256, 3, kG2PSolids>, 256, 0);
+        if (threads == 128) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<128, 6, kG2PSolids | kG2PReadOnly>, 128, 0);
+        else if (threads == 512) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<512, 1, kG2PSolids | kG2PReadOnly>, 512, 0);
+        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_g2p<256, 3, kG2PSolids | kG2PReadOnly>, 256, 0);
     }
     return b;
 }
