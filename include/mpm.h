@@ -107,10 +107,11 @@ enum {
                                    a call of k substeps replays ceil(k/chunk) graphs */
     MPM_OPT_PHASE_TIMING = 7,   /* 0/1: record CUDA events around each phase of every
                                    substep (forces direct launches); see mpm_phase_stats */
-    MPM_OPT_P2G_CHUNK = 8,      /* particles of two passes of a P2G CTA: 384, 576
-                                   or 768 (default), i.e. 32, 48 or 64 staged by each
-                                   of its six warps; launches that 32 a warp fit on
-                                   the chip at once stage 32                        */
+    MPM_OPT_P2G_CHUNK = 8,      /* particles of two passes of a P2G CTA: 384, 576 or
+                                   768, i.e. 32, 48 or 64 staged by each of its six
+                                   warps; until it is set 384 for launches that 32 a
+                                   warp fit on the chip at once, else 768 (reads back
+                                   the shape of a launch over all scenes)           */
     MPM_OPT_FUSED = 9,          /* 1: fuse each substep's G2P with the next substep's
                                    P2G; 0 (default): separate P2G and G2P kernels */
     MPM_OPT_G2P_REGS64 = 10     /* 1: G2P variant limited to 64 registers (more

@@ -139,14 +139,14 @@ static int g2p_threads_for(const mpm_ctx* c, int np)
     return np < (1 << 19) ? 256 : 128;
 }
 
-// Slots that each P2G warp stages: a warp's share of half the set pass, and 32 where that
-// gives every warp that fits on the chip one chunk at most (a pass of 32 lanes takes 64
-// slots' runs as well as 32 slots': at 131k particles, 1.1 chunks of 32 a warp, a substep of
-// the standard MPM takes 44.9 us with 32 and 41.1 with 64).
-static int p2g_slots_for(const mpm_ctx* c, int np)
+// Slots that each P2G warp stages: a warp's share of half the set pass, or by default 32 where
+// that gives every warp that fits on the chip one chunk at most and 64 above (a pass of 32
+// lanes takes 64 slots' runs as well as 32 slots': at 131k particles, 1.1 chunks of 32 a warp,
+// a substep of the standard MPM takes 44.9 us with 32 and 41.1 with 64).
+int p2g_slots_for(const mpm_ctx* c, int np)
 {
-    const int slots = c->p2g_chunk / (2 * kP2GThreads / 32);
-    return (long long)np < 32ll * c->num_sms * 24 ? 32 : slots;
+    if (c->p2g_chunk) return c->p2g_chunk / (2 * kP2GThreads / 32);
+    return (long long)np < 32ll * c->num_sms * 24 ? 32 : 64;
 }
 
 static int cap_occ(const mpm_ctx* c, int occ)
@@ -501,7 +501,7 @@ extern "C" int mpm_get_option(mpm_ctx* c, int option, int64_t* value)
     case MPM_OPT_CTAS_PER_SM: *value = c->ctas_per_sm; break;
     case MPM_OPT_GRAPH_CHUNK: *value = c->graph_chunk; break;
     case MPM_OPT_PHASE_TIMING: *value = c->phase_timing; break;
-    case MPM_OPT_P2G_CHUNK: *value = c->p2g_chunk; break;
+    case MPM_OPT_P2G_CHUNK: *value = p2g_slots_for(c, c->total_particles) * (2 * kP2GThreads / 32); break;
     case MPM_OPT_FUSED: *value = c->fused; break;
     case MPM_OPT_G2P_REGS64: *value = c->g2p_regs64; break;
     default: return MPM_ERR_INVALID_ARGUMENT;

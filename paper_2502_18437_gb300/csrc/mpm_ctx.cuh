@@ -60,7 +60,7 @@ struct mpm_ctx {
     // options
     int use_graphs = 1;
     int launch_mode = 0;
-    int p2g_chunk = 4 * mpm::kP2GThreads;
+    int p2g_chunk = 0;    // 0: by the launch's particle count
     int g2p_threads = 0;  // 0: by the launch's particle count
     int g2p_regs64 = 0;
     int ctas_per_sm = 0;
@@ -86,6 +86,7 @@ namespace mpm {
 // helpers shared by the C ABI translation units
 int status_from_cuda(cudaError_t e);
 int wait_stream(mpm_ctx* c);
+int p2g_slots_for(const mpm_ctx* c, int np);  // slots that each P2G warp stages
 StepArgs step_args(mpm_ctx* c, float dt, int s0, int s1, const PState& in, const PState& out);
 int enqueue_substep(mpm_ctx* c, float dt, const PState& in, const PState& out, bool need_p2g);
 int invalidate_pending(mpm_ctx* c);
