@@ -239,7 +239,9 @@ int mpm_add_particles(mpm_ctx* ctx, int scene, int64_t n, const float* x, const 
 /* Create or replace rigid `rigid_id` (0..MPM_MAX_RIGIDS-1) of `scene`; a type
  * of MPM_RIGID_NONE removes it.  Rigids act on the grid in id order.  The
  * pose given is the pose at the current simulation time; the rigid's
- * accumulated impulse is kept.  Errors: INVALID_ARGUMENT, CUDA. */
+ * accumulated impulse is kept.  Enqueued on the stream; refused (CUDA, nothing
+ * changed) while the stream is being captured into a graph.
+ * Errors: INVALID_ARGUMENT, CUDA. */
 int mpm_set_rigid(mpm_ctx* ctx, int scene, int rigid_id, const mpm_rigid* r);
 
 /* ---- simulation ------------------------------------------------------ */

@@ -723,6 +723,10 @@ extern "C" int mpm_set_rigid(mpm_ctx* c, int scene, int rigid_id, const mpm_rigi
             d.hi[i] = hi + wide;
         }
     }
+    // refused before anything changes: poses belong to a moment, not to a graph
+    cudaStreamCaptureStatus capturing;
+    MPM_CK(cudaStreamIsCapturing(c->stream, &capturing));
+    if (capturing != cudaStreamCaptureStatusNone) return MPM_ERR_CUDA;
     c->h_rigids[slot] = d;
     if (c->rigid_type[slot] != d.type) clear_graphs(c);  // captured launches carry the kinds of rigids
     c->rigid_type[slot] = d.type;
@@ -735,9 +739,6 @@ extern "C" int mpm_set_rigid(mpm_ctx* c, int scene, int rigid_id, const mpm_rigi
         clear_graphs(c);  // captured substeps carry whether any scene has a rigid
     }
     // the description travels in the launch's arguments: nothing to wait for
-    cudaStreamCaptureStatus capturing;
-    MPM_CK(cudaStreamIsCapturing(c->stream, &capturing));
-    if (capturing != cudaStreamCaptureStatusNone) return MPM_ERR_CUDA;  // poses belong to a moment, not to a graph
     MPM_CK(launch_set_rigid(d, c->d_rigids + slot, c->stream));
     return upload_scenes(c);
 }
