@@ -707,8 +707,9 @@ extern "C" int mpm_set_rigid(mpm_ctx* c, int scene, int rigid_id, const mpm_rigi
         for (int k = 0; k < 3 * d.n_pts; ++k) d.shape.pts[k] = (&r->points[0][0])[k];
         // (widened by far more than the distances' rounding, relative to the shape and its reach;
         // without end where a point is not finite)
-        const float reach = std::max(r->type == MPM_SEGMENTS ? r->radius : std::max(0.5f * r->thickness, r->spine_radius), 0.f) +
-                            std::max(r->margin, 0.f);
+        // (fmax leaves a NaN out: a comparison with it touches nothing, but the other reach still does)
+        const float reach = std::fmax(r->type == MPM_SEGMENTS ? r->radius : std::fmax(0.5f * r->thickness, r->spine_radius), 0.f) +
+                            std::fmax(r->margin, 0.f);
         for (int i = 0; i < 3 && d.n_pts > 0; ++i) {
             float lo = d.shape.pts[i], hi = lo, big = std::fabs(lo), sum = lo;
             for (int k = 1; k < d.n_pts; ++k) {
