@@ -35,8 +35,10 @@ if ROOT not in sys.path:
 METRIC = "particle-substeps/s at 1M particles FP32"
 UNIT = "particle-substeps/s"
 SUBSTEPS_PER_STEP = 25
-# scan, scatter, P2G, grid update, accumulator reset, G2P
-KERNELS_PER_SUBSTEP = 6
+# scan, scatter, P2G, grid update, G2P
+KERNELS_PER_SUBSTEP = 5
+KERNELS_PER_REKEY = 2   # histogram reset and keys, before the first substep from a written state
+KERNELS_PER_RESTART = 1 + KERNELS_PER_REKEY  # the state write moves all fields in one kernel
 TRAJECTORY_STEPS = 20  # 20 x 25 = the block's 500-substep trajectory
 FALL_SUBSTEPS = 150    # the block is still falling (F close to I) before this substep
 
@@ -177,9 +179,9 @@ def measured_peaks():
 #   grid  (m, mv) written by P2G 16, read 16, velocity written 12 and read by
 #         G2P 12, accumulator cleared 16                     72 B per active node
 # (~270 B per particle-substep at 8 particles per cell.)  This design moves
-# somewhat more (implementation_bytes): the stress is stored by G2P and read
-# by P2G instead of F (24 + 24 B for 36 B), particle ids, the next substep's
-# brick key and rank, and the permutation rewritten in cell order.
+# somewhat more (moved_bytes): state in whole 16-byte words, 128 B of which G2P
+# writes per particle (the stress and the id among them), the next substep's key
+# and rank, and the counts of particles per cell.
 
 ALGO_PER_PARTICLE = {"sort": 16, "p2g": 96, "grid": 0, "g2p": 144}
 ALGO_PER_NODE = {"sort": 0, "p2g": 0, "grid": 72, "g2p": 0}
@@ -192,7 +194,8 @@ def algorithmic_bytes(N, active_nodes):
 
 
 def implementation_bytes(N, bricks, active_nodes, pp_mat=False):
-    """Bytes this design's kernels move at least once per substep:
+    """Bytes of the layout before the sort by cell, for comparison with records of
+    that time (moved_bytes: the present one):
       sort  scan: brick count + node flag (8 B per brick of the grid); scatter:
             key, rank and the brick offset read, slot and its cell written (17 B
             per particle)
@@ -209,6 +212,38 @@ def implementation_bytes(N, bricks, active_nodes, pp_mat=False):
         "grid": 48 * active_nodes,
         "g2p": (188 + extra) * N + 16 * active_nodes,
     }
+
+
+def moved_bytes(N, bricks, active_nodes, pp_mat=False):
+    """Bytes this design's kernels move at least once per substep (particle bricks
+    counted as node bricks, which they all are):
+      sort  scan: particles per brick (4 B per brick of the grid), particles per cell
+            of the particle bricks read and turned into first slots (8 B per node);
+            scatter: key, rank and first slot read, permutation written (16 B per particle)
+      p2g   permutation 4 + six of the state's eight 16-byte words 96 read, one 16-byte
+            reduction per active node
+      grid  (m, mv) read, (v, m) written, the cell's count cleared: 36 B per active node
+      g2p   permutation 4 + four words 64 read, eight words 128 + key, rank 8 written
+            (+ mu, lambda 16 with per-particle materials); (v, m) read and (m, mv)
+            cleared, 32 B per active node"""
+    extra = 16 if pp_mat else 0
+    return {
+        "sort": 4 * bricks + 16 * N + 8 * active_nodes,
+        "p2g": 100 * N + 16 * active_nodes,
+        "grid": 36 * active_nodes,
+        "g2p": (204 + extra) * N + 32 * active_nodes,
+    }
+
+
+def timed_launches(substeps, restarts):
+    """Kernels launched in the timed region, which starts from a written state."""
+    return KERNELS_PER_SUBSTEP * substeps + KERNELS_PER_REKEY + KERNELS_PER_RESTART * restarts
+
+
+def published(roofline):
+    """The roofline object as the JSON line carries it: without the bytes of the
+    layout before the sort by cell."""
+    return {k: v for k, v in roofline.items() if not k.startswith("implementation_bytes")}
 
 
 def kernel_source_digest():
@@ -271,10 +306,11 @@ def roofline_fields(N, bricks, active_nodes, per_launch_ms, substep_ms, peak, pe
     """The `roofline` object of the JSON line: the dominant kernel (largest share
     of the substep's device time), its algorithmic bytes per launch divided by its
     mean launch duration, against the measured HBM copy peak; the whole substep's
-    algorithmic bytes over the substep time beside it.  `implementation_bytes`
-    reports what this design's kernels move, for comparison."""
+    algorithmic bytes over the substep time beside it.  `moved_bytes` reports what
+    this design's kernels move, for comparison."""
     ab = algorithmic_bytes(N, active_nodes)
     ib = implementation_bytes(N, bricks, active_nodes, pp_mat)
+    mb = moved_bytes(N, bricks, active_nodes, pp_mat)
     tot = sum(per_launch_ms.values())
     dom = max(per_launch_ms, key=per_launch_ms.get)
     achieved = ab[dom] / (per_launch_ms[dom] / 1e3) / 1e9
@@ -291,6 +327,8 @@ def roofline_fields(N, bricks, active_nodes, per_launch_ms, substep_ms, peak, pe
             "whole_substep_frac": round(step / (substep_ms / 1e3) / 1e9 / peak, 4),
             "implementation_bytes_per_particle_substep": round(sum(ib.values()) / N, 1),
             "implementation_bytes_per_launch": ib[dom],
+            "moved_bytes_per_particle_substep": round(sum(mb.values()) / N, 1),
+            "moved_bytes_per_launch": mb[dom],
             "active_nodes": active_nodes}
 
 
@@ -456,11 +494,11 @@ def run_ours(args):
                        "l2": "working set > 129 MB L2 between iterations (no flush)",
                        "launch": (f"per step: mpm_substep(dt, {SUBSTEPS_PER_STEP}) = {graphs} CUDA graph replay(s) "
                                   f"of up to {chunk} substeps, {KERNELS_PER_SUBSTEP} kernels per substep"
-                                  + "; the first substep runs directly after the key kernel of the initial "
-                                  "state" + ("" if restarts == 0 else "; each restart adds 4 state-write kernels "
-                                             "and the key kernel"))},
-            "gpu_launches": KERNELS_PER_SUBSTEP * total_substeps + 1 + restarts * (4 + 1), "clocks": clk,
-            "roofline": roofline}
+                                  + "; the first substep runs directly after the two key kernels of the initial "
+                                  "state" + ("" if restarts == 0 else "; each restart adds the state-write kernel "
+                                             "and the two key kernels"))},
+            "gpu_launches": timed_launches(total_substeps, restarts), "clocks": clk,
+            "roofline": published(roofline)}
     if tuned:
         line["config"]["autotuned"] = tuned
 
