@@ -119,7 +119,6 @@ __device__ void stress_and_vjp(int model, const float F[9], float mu, float lam,
         mul_abt(F, F, FFt);
 #pragma unroll
         for (int i = 0; i < 9; ++i) tau[i] = mu * (FFt[i] - ((i % 4 == 0) ? 1.f : 0.f)) + ((i % 4 == 0) ? lam * lnJ : 0.f);
-        if (!tb) return;
         const float tr = tb[0] + tb[4] + tb[8];
         // F_bar = mu (tb + tb^T) F + lambda tr(tb) F^-T
 #pragma unroll
@@ -148,7 +147,6 @@ __device__ void stress_and_vjp(int model, const float F[9], float mu, float lam,
     mul_abt(P, F, PFt);
 #pragma unroll
     for (int i = 0; i < 9; ++i) tau[i] = 2.f * mu * PFt[i] + ((i % 4 == 0) ? lam * (J - 1.f) * J : 0.f);
-    if (!tb) return;
     const float tr = tb[0] + tb[4] + tb[8];
     // G = tb F;  F_bar = 2 mu G + 2 mu tb^T P + lambda (2J - 1) tr(tb) J F^-T + polar part
     float G[9];
