@@ -23,7 +23,9 @@
  *    every input before the call returns; output buffers are owned by the
  *    caller.
  *  - Every call returns MPM_OK (0) or a negative MPM_ERR_* code; no call traps
- *    the GPU, and every wait is bounded by mpm_config.timeout_ms.
+ *    the GPU, and every wait is bounded by mpm_config.timeout_ms.  A waiting call
+ *    polls for its first 20 ms, yielding its core between polls but keeping it
+ *    busy when nothing else wants it, and sleeps between polls after that.
  *  - Errors found on the device (a particle leaving the grid, a non-finite
  *    value, an inverted element where the law has no answer) are recorded per
  *    scene, are sticky until mpm_destroy, and are returned by the blocking

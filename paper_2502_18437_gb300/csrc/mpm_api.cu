@@ -129,9 +129,13 @@ void clear_graphs(mpm_ctx* c)
 }
 
 // G2P CTA size of a launch over np particles: the set value, or by default 256
-// threads below 512k particles (fewer particle bricks than 128-thread CTA slots:
-// more threads per brick shorten each CTA's brick) and 128 above.  The
-// standard-MPM and PB-MPM G2P variants exist at 128 threads only.
+// threads below 512k particles and 128 above.  Both hold 24 warps of 80 registers on an
+// SM; what decides is that the 128-thread shape leaves L1 the shared memory it does not
+// need (prepare_kernels).  A substep with 128 and with 256 threads: 4M particles 400 and
+// 415 us, 1M 121.0 and 119.6, 262k 42.3 and 41.5, 131k 32.4 and 33.1, 16k 19.1 and 19.2;
+// with a sphere in the scene 4M 419 and 421, 1M 134.4 and 132.1, 262k 46.8 and 46.5, 131k
+// 36.3 and 36.7, 16k 22.1 and 24.9.  The standard-MPM and PB-MPM G2P variants exist at
+// 128 threads only.
 static int g2p_threads_for(const mpm_ctx* c, int np)
 {
     if (c->cfg.solver != MPM_SOLVER_MLS) return 128;

@@ -91,8 +91,8 @@ StepArgs step_args(mpm_ctx* c, float dt, int s0, int s1, const PState& in, const
 int enqueue_substep(mpm_ctx* c, float dt, const PState& in, const PState& out, bool need_p2g);
 int invalidate_pending(mpm_ctx* c);
 int ensure_keys(mpm_ctx* c);
-// Zero the brick histogram, the node-brick flags and the tile sums (before keys
-// are recomputed from stored positions).
+// Zero the particle counts of bricks, cells and scan tiles and the sizes of the lists
+// (before keys are recomputed from stored positions).
 cudaError_t reset_histogram(mpm_ctx* c);
 int upload_scenes(mpm_ctx* c);
 int ensure_stage(mpm_ctx* c, size_t bytes);

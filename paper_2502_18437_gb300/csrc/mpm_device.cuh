@@ -138,7 +138,6 @@ __device__ __forceinline__ void load_v(const PState& s, size_t cap, int p, float
     v[0] = a.y; v[1] = a.z; v[2] = a.w;
 }
 
-// C and, in t6, the stored stress
 __device__ __forceinline__ void load_C(const PState& s, size_t cap, int p, float C[9])
 {
     const float4 a = plane(s, cap, 4, p), b = plane(s, cap, 5, p);

@@ -25,10 +25,10 @@ namespace mpm {
 // straddle scenes).  The key producers (G2P, k_prepare) count the particles of
 // every brick and every tile as they go, so each CTA of the scan (one per tile of
 // the range) knows the first slot of its bricks from the tile counts before it,
-// without waiting for another CTA.  The lists of active particle bricks and node
-// bricks need no order beyond the big bricks first (they start the persistent
-// transfer kernels, which then end on small ones), so each CTA appends its own to
-// them with one atomic per list.  A node brick is active when it or one of its 7
+// without waiting for another CTA.  The list of node bricks (the grid update's and the
+// reset's) needs no order, that of particle bricks (the fused kernel's; the others only
+// ask whether it is empty) only the big bricks first, so that the fused kernel's CTAs
+// end on small ones: each CTA appends its own to them with one atomic per list.  A node brick is active when it or one of its 7
 // lower neighbours (-1 in any subset of the axes) holds particles, since a
 // particle's 3-node stencil reaches at most 2 nodes beyond its base cell, i.e.
 // into the next brick: the scan looks the 8 counts up.  (Before, the first warp of

@@ -83,7 +83,7 @@ constexpr int kMinTileShift = 6;
 constexpr int kChainBelow = 48 << 10;
 constexpr int kScatterPer = 4;  // particles per thread of the counting-sort scatter
 // Particle bricks of at least this many particles come first in the active list,
-// so the persistent transfer kernels end on small bricks (a shorter tail)
+// so the fused kernel, whose CTAs take bricks in turn, ends on small ones (a shorter tail)
 constexpr int kBigBrick = 256;
 
 cudaError_t launch_prepare(const StepArgs& a, const PState& st, cudaStream_t s);

@@ -610,9 +610,7 @@ __device__ __forceinline__ void walker_exit(const StepArgs& a)
     if (threadIdx.x < 32) count_out(a);
 }
 
-// Poses at the end of the substep (clock + dt) of the solid rigids of a scene,
-// staged in shared memory by the threads tid < kMaxRigids of a group; the rigid
-// slots in use (shapes other than sphere and box are staged with type -1).
+// Centre and rotation matrix of a rigid at clock t_now.
 __device__ __forceinline__ void rigid_pose_at(const RigidDev& src, double t_now, float c[3], float R[9])
 {
     const float tau = (float)(t_now - src.t_set);
@@ -635,6 +633,9 @@ __device__ __forceinline__ void rigid_pose_at(const RigidDev& src, double t_now,
     quat_to_mat(qw, qx, qy, qz, R);
 }
 
+// Poses at the end of the substep (clock + dt) of the solid rigids of a scene,
+// staged in shared memory by the threads tid < kMaxRigids of a group; the rigid
+// slots in use (shapes other than sphere and box are staged with type -1).
 __device__ __forceinline__ void stage_solids(const StepArgs& a, int scene, SolidPose* poses, int tid)
 {
     const int nr = a.scenes[scene].n_rigid;
