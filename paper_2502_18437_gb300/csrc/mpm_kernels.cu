@@ -1305,7 +1305,7 @@ __global__ void __launch_bounds__(kVcThreads) k_g2p_vc(StepArgs a)
 // fields in one pass over the planes; a slot whose id is not of the scene (a substep that
 // a device error cut short wrote none) is left out.  Particle ids are in no order by slot, so one side
 // is scattered over HBM, and the sectors it half uses are the cost: one kernel a field
-// took 105 us to write 1M particles' state and 255 us to read it, now 75 and 133 us;
+// took 105 us to write 1M particles' state and 255 us to read it, now 75 and 117 us;
 // writing through records in id order instead, 177 us.
 
 // particle ids by slot
@@ -1445,9 +1445,10 @@ __global__ void __launch_bounds__(kIoBlock) k_state_by_slot(PState st, int cap, 
 
 // A CTA per kIoBlock consecutive ids: the arrays move as whole 16-byte words of one
 // contiguous chunk each (they may be pinned host memory, over the host link), through
-// shared memory; the particles' side, records on the way out and planes on the way in, is
-// the scattered one.
-template <bool OUT>
+// shared memory; the particles' side, planes or records, is the scattered one.  (Pinned
+// arrays are read and written from the planes: with records x of 4M particles took 429 us
+// to read, so 311, and all fields 2,247, so 2,151.)
+template <bool OUT, bool RECORDS>
 __global__ void __launch_bounds__(kIoBlock) k_fields_by_id(PState st, int cap, int p0, int np, const int* __restrict__ inv,
                                                            const float4* rec, Fields h)
 {
@@ -1460,7 +1461,12 @@ __global__ void __launch_bounds__(kIoBlock) k_fields_by_id(PState st, int cap, i
     const bool own = t < cnt && (unsigned)(s - p0) < (unsigned)np;
     float* const first[4] = {buf, buf + 3 * kIoBlock, buf + 6 * kIoBlock, buf + 15 * kIoBlock};
     const auto entry = [&](int f) { return h.f[f] ? first[f] + t * (f < 2 ? 3 : 9) : nullptr; };
-    if (OUT) {
+    if (OUT && !RECORDS) {
+        if (own)
+            planes_to_fields(st, cap, s, h.f[0] ? st.q[s] : make_float4(0.f, 0.f, 0.f, 0.f), entry(0), entry(1), entry(2), entry(3));
+        __syncthreads();
+    }
+    if (OUT && RECORDS) {
         if (own) {
             float r[kIoFloats];
 #pragma unroll
@@ -1704,14 +1710,24 @@ cudaError_t launch_fields(const PState& st, const PState& spare, int cap, int p0
     // the records (whole sectors) leave plane 0 alone: a substep that a device error skipped
     // leaves the spare buffer unwritten and current, and its ids are indexes
     float4* rec = spare.q + (((size_t)cap + 1) & ~(size_t)1);
-    if (out && (host || np >= kIoByIdFrom)) {
+    int fields = 0;
+    size_t bytes = 0;
+    for (int f = 0; f < 4; ++f)
+        if (h.f[f]) {
+            ++fields;
+            bytes += (size_t)np * sizeof(float) * (f < 2 ? 3 : 9);
+        }
+    if (out && host) {
+        k_id_inverse<<<n_blocks(np, 256), 256, 0, s>>>(st, p0, np, inv);
+        k_fields_by_id<true, false><<<n_blocks(np, kIoBlock), kIoBlock, 0, s>>>(st, cap, p0, np, inv, rec, h);
+    } else if (out && fields >= 3 && bytes >= kIoRecordsFrom) {
         k_pack<<<n_blocks(np, kIoBlock), kIoBlock, 0, s>>>(st, cap, p0, np, inv, rec);
-        k_fields_by_id<true><<<n_blocks(np, kIoBlock), kIoBlock, 0, s>>>(st, cap, p0, np, inv, rec, h);
+        k_fields_by_id<true, true><<<n_blocks(np, kIoBlock), kIoBlock, 0, s>>>(st, cap, p0, np, inv, rec, h);
     } else if (out) {
         k_arrays_by_slot<<<n_blocks(np, kIoBlock), kIoBlock, 0, s>>>(st, cap, p0, np, h);
     } else if (host) {
         k_id_inverse<<<n_blocks(np, 256), 256, 0, s>>>(st, p0, np, inv);
-        k_fields_by_id<false><<<n_blocks(np, kIoBlock), kIoBlock, 0, s>>>(st, cap, p0, np, inv, rec, h);
+        k_fields_by_id<false, false><<<n_blocks(np, kIoBlock), kIoBlock, 0, s>>>(st, cap, p0, np, inv, rec, h);
     } else {
         k_state_by_slot<<<n_blocks(np, kIoBlock), kIoBlock, 0, s>>>(st, cap, p0, np, h);
     }

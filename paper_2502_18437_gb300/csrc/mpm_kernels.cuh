@@ -111,10 +111,13 @@ cudaError_t launch_init_particles(const PState& st, int cap, int p_at, int n, in
 struct Fields {
     float* f[4];
 };
-// From this many particles the state is read by id, through records; below, by slot, in one
-// kernel.  Measured, by id and by slot: 35 and 26 us at 64k, 36 and 37 at 131k, 49 and 57 at
-// 262k, 133 and 219 at 1M, 485 and 1,306 at 4M.
-constexpr int kIoByIdFrom = 1 << 17;
+// Three or more fields whose arrays hold this many bytes are read into device memory through
+// records, all others by slot, in one kernel: the entries that a warp scatters come together
+// in L2 (129 MB) while it holds the arrays.  A read through records and by slot: x, v, C and F
+// 128 and 117 us at 1M particles (101 MB), 189 and 230 at 1.5M, 475 and 755 at 4M; x, C and F
+// 180 and 187 at 1.5M; x, v and C 226 and 194 at 2M, 448 and 499 at 4M; C and F 454 and 449 at
+// 4M, 2,072 and 1,910 at 16M; x alone 114 and 27 at 1M, 397 and 44 at 4M.
+constexpr size_t kIoRecordsFrom = 120'000'000;
 // state -> arrays (out) or arrays -> state; inv: scratch of np ints, spare: the state's other
 // buffer (all but its plane 0 is scratch); host: the arrays are pinned host memory
 cudaError_t launch_fields(const PState& st, const PState& spare, int cap, int p0, int np, int* inv, const Fields& h, bool out,

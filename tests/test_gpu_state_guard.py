@@ -140,3 +140,32 @@ def test_backward_refuses_a_tape_with_a_skipped_substep():
             with pytest.raises(mpm.MPMError) as e:
                 reverse()
             assert e.value.status == -10
+
+
+@pytest.mark.parametrize("fields,count", [("xvCF", 1250000), ("xvCF", 1250113), ("xCF", 1428672), ("xvC", 2000001),
+                                          ("CF", 1700000), ("x", 2000001)])
+def test_large_reads_take_the_scenes_own_ids(fields, count):
+    # the sizes from which three or more fields go through records, and fields that never do
+    torch = pytest.importorskip("torch")
+    p0, cap = 7, count + 9
+    g = torch.Generator(device="cuda").manual_seed(count)
+    state = torch.randn((8, cap, 4), generator=g, device="cuda")
+    ids = torch.randperm(count, generator=g, device="cuda").int()
+    state[0, p0:p0 + count, 3] = ids.view(torch.float32)
+    by_slot = state.permute(1, 0, 2).reshape(cap, 32)[p0:p0 + count]
+    spare = torch.randn((8, cap, 4), generator=g, device="cuda")
+    first = spare[0].clone()
+    inv = torch.empty(cap, dtype=torch.int32, device="cuda")
+    arrs, h = {}, Fields()
+    for k, f in enumerate("xvCF"):
+        if f in fields:
+            arrs[f] = torch.zeros((count + 2 * MARGIN, COMPS[f]), device="cuda")
+            h.f[k] = arrs[f].data_ptr() + 4 * MARGIN * COMPS[f]
+    st, sp = PState(state.data_ptr(), None, None), PState(spare.data_ptr(), None, None)
+    assert launch_fields()(ct.byref(st), ct.byref(sp), cap, p0, count, inv.data_ptr(), ct.byref(h), True, False,
+                           torch.cuda.current_stream().cuda_stream) == 0
+    for f, a in arrs.items():
+        want = torch.zeros_like(a)
+        want[MARGIN + ids.long()] = by_slot[:, list(AT[f])]
+        assert torch.equal(a, want), f
+    assert torch.equal(spare[0].view(torch.int32), first.view(torch.int32))
