@@ -55,8 +55,7 @@ def parse():
     p.add_argument("--profile-substeps", type=int, default=0,
                    help="run this many substeps with direct launches and exit (the command profiles use)")
     p.add_argument("--profile-batched-substeps", type=int, default=0,
-                   help="run the 256-scene batched workload for this many substeps with direct launches "
-                        "(P2G passes of 576, 128-thread 64-register G2P) and exit")
+                   help="run the 256-scene batched workload for this many substeps with direct launches and exit")
     return p.parse_args()
 
 
@@ -394,8 +393,7 @@ def run_ours(args):
         # the command of the batched ncu summary under profiles/: direct launches, no timing
         bstream = torch.cuda.Stream()
         bsim = mpm.from_scenes(workloads.batched_scenes(), stream=bstream.cuda_stream)
-        for k, v in (("use_graphs", 0), ("p2g_chunk", 576), ("g2p_threads", 128), ("g2p_regs64", 1)):
-            bsim.set_option(k, v)
+        bsim.set_option("use_graphs", 0)
         bsim.substep(1e-4, args.profile_batched_substeps)
         errs = [bsim.error_bits(s) for s in range(256)]
         bsim.close()
